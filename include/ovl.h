@@ -230,9 +230,9 @@ int ovl_batch_solve(ovl_batch* batch, int k, double mu, double kappa, const void
  * combination; *nsolves the number of such solves.  reset != 0 clears the totals. */
 int ovl_batch_profile(ovl_batch* batch, double* ms3, int* nsolves, int reset);
 /* Launch shapes of the batched kernels.  The first solve in each precision times the candidates
- * (pass-1 site blocks of 64, 128 or 256 sites; the regeneration kernel at 3 to 6 blocks per SM
- * with one sequence per block, or at 2 to 4 blocks per SM with two sequences of one lattice per
- * block) with short eager solves of the batch itself and keeps the fastest (OVL_NO_TUNE skips
+ * (pass-1 site blocks of 64, 128 or 256 sites; the double-float regeneration kernel at 3 or 4 times
+ * 128 threads per SM; the FP64 one at 3 to 6 blocks per SM with one sequence per block, or at 2 to 4
+ * blocks per SM with two sequences of one lattice per block) with short eager solves of the batch itself and keeps the fastest (OVL_NO_TUNE skips
  * this).  The choice is cached per (GPU model, SM count, precision, lattice extents and
  * right-hand sides of every context): later batches of the same shape in the process take it
  * without timing, and when the environment variable OVL_TUNE_CACHE names a file the choices are
@@ -240,8 +240,9 @@ int ovl_batch_profile(ovl_batch* batch, double* ms3, int* nsolves, int reset);
  * chosen shapes (NULL pointers are skipped); returns OVL_ESTATE before the first tuning. */
 int ovl_batch_tuning(const ovl_batch* batch, int* pass1_block_sites, int* regen_blocks_per_sm,
                      int* regen_seqs_per_block);
-/* Pins the launch shapes (pass1_block_sites 64, 128 or 256; regen_blocks_per_sm 2 to 6;
- * regen_seqs_per_block 1 or 2) and turns the autotuner off for this batch.  OVL_EINVAL for any
+/* Pins the launch shapes (pass1_block_sites 64, 128 or 256; regen_blocks_per_sm 2 to 6, of which the
+ * double-float regeneration takes 2 and 3 as 3 x 128 threads per SM, 4 to 6 as 4 x 128;
+ * regen_seqs_per_block 1 or 2, which the double-float regeneration ignores) and turns the autotuner off for this batch.  OVL_EINVAL for any
  * other value (nothing changed). */
 int ovl_batch_set_tuning(ovl_batch* batch, int pass1_block_sites, int regen_blocks_per_sm,
                          int regen_seqs_per_block);

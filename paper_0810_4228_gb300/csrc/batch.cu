@@ -34,6 +34,13 @@
 
 namespace ovl {
 
+// per-step coefficients of the double-float regeneration (see k_b_regen_coef)
+struct RegenCoefDf {
+    float4 kb;        // kappa / beta_i (real; .x hi, .y lo)
+    float4 cu, cl;    // cr of the upper and the lower spins {re hi, re lo, im hi, im lo}
+    float4 cg, cc;    // cg; c_{i+1}
+};
+
 struct BSeq {
     Geom g;
     size_t n;                 // 12 V
@@ -48,6 +55,8 @@ struct BSeq {
     double2* V;               // FP64 one-pass: stored basis, k + 1 vectors (else null)
     double2* r[3];            // FP64 regeneration ring (two-pass)
     double2* y;
+    const double2* bR;        // b_perp^R (start of the regeneration)
+    RegenCoefDf* rc;          // per-step coefficients of the double-float regeneration (mixed)
     KState* ks;
     double2* alpha;
     double2* beta;
@@ -569,94 +578,376 @@ __global__ void __launch_bounds__(BP1_T, 3) k_bp1(BP1Args a) {
     }
 }
 
-// Regeneration (Sec. 5): r_{i+1} = ((A - alpha_i) r_i - gamma_{i-1} r_{i-1}) / beta_i, y += c_{i+1} r_{i+1},
-// in FP64 (R = double) or double-float (R = df; ring and y converted beforehand).  One block per
-// 32-site tile of a sequence: warp h applies hop h (direction-uniform code) to the tile's sites, the
-// eight partial sums meet in shared memory, and 128 threads (site, spin) finish three components each.
-template <class R> __device__ __forceinline__ cx<R> cvt_coef(cx<double> z);
-template <> __device__ __forceinline__ cx<double> cvt_coef<double>(cx<double> z) { return z; }
-template <> __device__ __forceinline__ cx<df> cvt_coef<df>(cx<double> z) { return mk(df(z.r), df(z.i)); }
+// Regeneration (Sec. 5): r_{i+1} = ((A - alpha_i) r_i - gamma_{i-1} r_{i-1}) / beta_i, y += c_{i+1} r_{i+1}:
+// in double-float (k_b_regen_df, mixed solves) or in FP64 (k_b_regen, k_b_regen2).
 
-// Hop h of the double-float regeneration at site i, written straight to out[0..6) (the half
-// spinor, spins 0 and 1, colours 0..2, times the hop coefficient): spin row by spin row, the
-// neighbour's two spin components that row needs are projected and the link applied row by row (U)
-// or column by column (U^dag), so that only one projected row, one link row and two accumulators
-// are live at a time (few registers: six blocks per SM with little spilling; measured on the
-// 48-sequence batch, pass 2 317.9 -> 305.2 ms against projecting both rows first).  The link is
-// read once per spin row (the second time from L1).  The operations and their order per output are
-// those of hop_half_uniform with mul_link / mul_link_dag, so the results are the same.
-__device__ __forceinline__ void hop_half_rows_df(int h, const Geom& g, const int* __restrict__ nbr, int i,
-                                                 const dfc* __restrict__ U, const dfc* __restrict__ x,
-                                                 const HopCoef<df>& hc, cx<df>* __restrict__ out) {
-    const int nu = h & 3;
-    const bool fwd = h < 4;
-    // neighbour and boundary phase from the lattice's table (no coordinate arithmetic per hop)
-    const int ne = __ldg(nbr + (size_t)h * g.V + i);
-    const int nb = ne < 0 ? ~ne : ne;
-    const df ph = ne < 0 ? df(-1) : df(1);
-    const bool hi2 = nu >= 2, im = (nu & 1) == 0;
-    const bool n0 = (nu == 3) ? !fwd : fwd;
-    const bool n1 = (nu == 0) ? fwd : !fwd;
-    const float4* xv = reinterpret_cast<const float4*>(x);
-    const size_t V = (size_t)g.V;
-    auto ldx = [&](int q) {
-        const float4 v = __ldg(xv + (size_t)q * V + nb);
-        return mk(df(v.x, v.y), df(v.z, v.w));
-    };
-    const df cf = (fwd ? (nu == 3 ? hc.f[3] : hc.f[0]) : (nu == 3 ? hc.b[3] : hc.b[0])) * ph;
-    const float4* uv = reinterpret_cast<const float4*>(U) + (size_t)nu * 9 * V + (fwd ? i : nb);
-    // spin rows one after the other: the projected row sp (three colours) and one link row at a
-    // time (the link read twice, from L1 the second time): fewer live registers
+// ---- double-float regeneration ----------------------------------------------------------------
+// Vectors (r, y) of the pass are stored with the two spins of a half spinor side by side: chunk
+// (P * 3 + colour) * 2 + part of a site is the float4 {hi of spin 2P, hi of spin 2P + 1, lo, lo} of the
+// real (part 0) or imaginary (part 1) part, the operand layout of the packed FP32x2 arithmetic.
+//
+// Coefficients of a step, formed once per sequence (k_b_regen_coef) and stored as double-float: with
+// S the sum of the hops (e^{+-mu} on the temporal ones, kappa taken out), A r = r - kappa S on the upper
+// spins and -(r - kappa S) on the lower, so
+//   r_{i+1} = cr r_i -+ (kappa / beta_i) S + cg r_{i-1},  cr = (+-1 - alpha_i) / beta_i, cg = -gamma_{i-1} / beta_i.
+
+__device__ __forceinline__ float4 df4(cx<double> z) {
+    const df r(z.r), i(z.i);
+    return make_float4(r.hi, r.lo, i.hi, i.lo);
+}
+
+// grid (steps / 128, sequences)
+__global__ void k_b_regen_coef(const BSeq* __restrict__ S, double kappa) {
+    const BSeq& q = S[blockIdx.y];
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (q.ks->status || i + 1 >= q.ks->kused) return;
+    const double ib = 1.0 / q.beta[i].x;  // beta_i is real
+    const cx<double> a = ib * d2c(q.alpha[i]);
+    RegenCoefDf c;
+    c.kb = df4(mk(ib * kappa, 0.0));
+    c.cu = df4(mk(ib - a.r, -a.i));
+    c.cl = df4(mk(-ib - a.r, -a.i));
+    c.cg = i > 0 ? df4(-(ib * d2c(q.gamma[i - 1]))) : make_float4(0.f, 0.f, 0.f, 0.f);
+    c.cc = df4(d2c(q.cvec[i + 1]));
+    q.rc[i] = c;
+}
+
+// r_1 = b_perp / |b_perp|, y += c_1 r_1 in FP64, both then split into the packed layout (y in place: a
+// thread owns its site); one launch for all sequences, blocks as in the pass-1 shape of 128 sites.
+__global__ void __launch_bounds__(128) k_b_regen_start(const BSeq* __restrict__ S, const int* __restrict__ bseq) {
+    const BSeq& q = S[bseq[blockIdx.x]];
+    const int site = (blockIdx.x - q.blk0[1]) * 128 + threadIdx.x;
+    if (site >= q.g.V) return;
+    const size_t V = (size_t)q.g.V;
+    const bool run = !q.ks->status && q.ks->nR != 0.0;
+    const cx<double> sv = mk(run ? 1.0 / q.ks->nR : 0.0, 0.0), c0 = d2c(q.cvec[0]);
+    df yr[12], yi[12];
+    float4* r0 = reinterpret_cast<float4*>(q.r[0]);
+    float4* yo = reinterpret_cast<float4*>(q.y);
 #pragma unroll
-    for (int sp = 0; sp < 2; ++sp) {
-        cx<df> hs[3];
-        const bool nn = sp == 0 ? n0 : n1;
-        const int so = hi2 ? 2 + sp : 3 - sp;
-#pragma unroll
-        for (int a = 0; a < 3; ++a) hs[a] = add_lazy(ldx(3 * sp + a), unit_mul(ldx(3 * so + a), im, nn));
+    for (int P = 0; P < 2; ++P)
 #pragma unroll
         for (int a = 0; a < 3; ++a) {
-            cx<df> u[3];
+            cx<df> z[2];
 #pragma unroll
-            for (int k = 0; k < 3; ++k) {
-                const float4 v = __ldg(uv + (size_t)(fwd ? 3 * a + k : 3 * k + a) * V);
-                u[k] = mk(df(v.x, v.y), df(v.z, v.w));
-            }
-            dfacc re, imv;
-            if (fwd) {
-                dfacc_first(re, u[0].r, hs[0].r, false);
-                dfacc_add(re, u[0].i, hs[0].i, true);
-                dfacc_first(imv, u[0].r, hs[0].i, false);
-                dfacc_add(imv, u[0].i, hs[0].r, false);
-#pragma unroll
-                for (int k = 1; k < 3; ++k) {
-                    dfacc_add(re, u[k].r, hs[k].r, false);
-                    dfacc_add(re, u[k].i, hs[k].i, true);
-                    dfacc_add(imv, u[k].r, hs[k].i, false);
-                    dfacc_add(imv, u[k].i, hs[k].r, false);
+            for (int h = 0; h < 2; ++h) {
+                const int c = 3 * (2 * P + h) + a;
+                cx<double> y = d2c(q.y[(size_t)c * V + site]);
+                if (run) {
+                    const cx<double> v = sv * d2c(q.bR[(size_t)c * V + site]);
+                    cfma(y, c0, v);
+                    z[h] = mk(df(v.r), df(v.i));
                 }
-            } else {
-                dfacc_first(re, u[0].r, hs[0].r, false);
-                dfacc_add(re, u[0].i, hs[0].i, false);
-                dfacc_first(imv, u[0].r, hs[0].i, false);
-                dfacc_add(imv, u[0].i, hs[0].r, true);
-#pragma unroll
-                for (int k = 1; k < 3; ++k) {
-                    dfacc_add(re, u[k].r, hs[k].r, false);
-                    dfacc_add(re, u[k].i, hs[k].i, false);
-                    dfacc_add(imv, u[k].r, hs[k].i, false);
-                    dfacc_add(imv, u[k].i, hs[k].r, true);
-                }
+                yr[c] = df(y.r);
+                yi[c] = df(y.i);
             }
-            out[3 * sp + a] = cf * mk(dfacc_value(re), dfacc_value(imv));
+            if (run) {
+                const size_t e = (size_t)(P * 3 + a) * 2 * V + site;
+                r0[e] = make_float4(z[0].r.hi, z[1].r.hi, z[0].r.lo, z[1].r.lo);
+                r0[e + V] = make_float4(z[0].i.hi, z[1].i.hi, z[0].i.lo, z[1].i.lo);
+            }
+        }
+#pragma unroll
+    for (int P = 0; P < 2; ++P)
+#pragma unroll
+        for (int a = 0; a < 3; ++a) {
+            const int c0_ = 6 * P + a, c1_ = 6 * P + 3 + a;
+            const size_t e = (size_t)(P * 3 + a) * 2 * V + site;
+            yo[e] = make_float4(yr[c0_].hi, yr[c1_].hi, yr[c0_].lo, yr[c1_].lo);
+            yo[e + V] = make_float4(yi[c0_].hi, yi[c1_].hi, yi[c0_].lo, yi[c1_].lo);
+        }
+}
+
+// y back to FP64 in the component layout (in place)
+__global__ void __launch_bounds__(128) k_b_regen_out(const BSeq* __restrict__ S, const int* __restrict__ bseq) {
+    const BSeq& q = S[bseq[blockIdx.x]];
+    const int site = (blockIdx.x - q.blk0[1]) * 128 + threadIdx.x;
+    if (site >= q.g.V) return;
+    const size_t V = (size_t)q.g.V;
+    float4 v[12];
+    const float4* yi = reinterpret_cast<const float4*>(q.y);
+#pragma unroll
+    for (int c = 0; c < 12; ++c) v[c] = yi[(size_t)c * V + site];
+#pragma unroll
+    for (int P = 0; P < 2; ++P)
+#pragma unroll
+        for (int a = 0; a < 3; ++a) {
+            const float4 re = v[(P * 3 + a) * 2], im = v[(P * 3 + a) * 2 + 1];
+            q.y[(size_t)(6 * P + a) * V + site] =
+                make_double2((double)re.x + (double)re.z, (double)im.x + (double)im.z);
+            q.y[(size_t)(6 * P + 3 + a) * V + site] =
+                make_double2((double)re.y + (double)re.w, (double)im.y + (double)im.w);
+        }
+}
+
+// real and imaginary sums of a pair of spins
+struct CAcc2 {
+    dfacc2 r, i;
+};
+
+// 16-byte asynchronous copy global -> shared (completion: cp.async.wait_group, a hardware wait)
+__device__ __forceinline__ void cp_async16(float4* dst, const float4* src) {
+    const unsigned d = (unsigned)__cvta_generic_to_shared(dst);
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 16;" ::"r"(d), "l"(src) : "memory");
+}
+__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+template <int N> __device__ __forceinline__ void cp_async_wait() {
+    asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory");
+}
+
+// Projected half spinor h (both spins packed): (1 + S gamma_NU) psi, spins 0 and 1, of the spinor in the
+// slots p[0], p[T], ... p[11 T]; sg the signs of the lower components in them (+-1, from the sense).
+template <int NU, int T>
+__device__ __forceinline__ void project_dfx(const float4* p, float2 sg, CAcc2 (&h)[3]) {
+    constexpr bool HI2 = NU >= 2, IM = (NU & 1) == 0;
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {
+        const float4 ur = p[2 * a * T], ui = p[(2 * a + 1) * T];
+        float4 lr = p[(6 + 2 * a) * T], li = p[(7 + 2 * a) * T];
+        if (!HI2) {  // spin 0 takes the lower spin 3, spin 1 the lower spin 2
+            lr = make_float4(lr.y, lr.x, lr.w, lr.z);
+            li = make_float4(li.y, li.x, li.w, li.z);
+        }
+        h[a].r.s = make_float2(ur.x, ur.y), h[a].r.e = make_float2(ur.z, ur.w);
+        h[a].i.s = make_float2(ui.x, ui.y), h[a].i.e = make_float2(ui.z, ui.w);
+        const float2 lrh = make_float2(lr.x, lr.y), lrl = make_float2(lr.z, lr.w);
+        const float2 lih = make_float2(li.x, li.y), lil = make_float2(li.z, li.w);
+        if (IM) {  // + sg i (lower)
+            dfacc2_add_signed(h[a].r, f2_neg(sg), lih, lil);
+            dfacc2_add_signed(h[a].i, sg, lrh, lrl);
+        } else {
+            dfacc2_add_signed(h[a].r, sg, lrh, lrl);
+            dfacc2_add_signed(h[a].i, sg, lih, lil);
         }
     }
 }
 
-template <class R, int LF, int MINB>
+// One thread per site and sequence: the eight hops one after the other, the four spins' sums in
+// registers (double-float, spins packed in pairs), then the recurrence and y in the same thread.
+// The hop loop is rolled (direction and sense are uniform), the link product is one piece of code for U
+// and U^dag (row or column addressing and the sign of the imaginary parts), one link row at a time.
+// Bound by the FP32 pipe: 10800 FP32 operations per site and step (per hop 12 projection sums of 8, 12
+// sums of 6 products at 64, 24 spin sums of 8; per part of an output component 52 for the recurrence, 30
+// for y and three renormalisations of 3; the temporal coefficients 168).  With the loads left to the hop
+// that uses them a warp stood on them 70 % of its time at 16 warps per SM (415 us below); each thread's
+// copies for the next hop now go to its own slots of shared memory while it computes the present one (no
+// block barrier anywhere).
+// Measured on the 48-sequence batch (706752 sites): 290 us per launch, 26.3 Top/s = 0.65 of the FP32 issue
+// rate, FMA pipe 67 % busy; the form before this one (eight hop warps per 32-site tile, half spinors
+// through shared memory, scalar instructions) took 552.  16^3 x 32, one source: 121 -> 64 us;
+// 12 sources on 8^4: 59.8 -> 28.9 us.  Against the FP64 pass after 480 steps: 1.7 ... 2.0e-14 (2.0 ...
+// 2.3e-14 before; y's low part is what that error is made of).  Blocks of 64: 32 and 128 differ by less
+// than 1 %; four sequences of a lattice in one block were no faster (their links meet in L2 either way).
+constexpr int RD_T = 64;  // sites per block
+constexpr size_t RD_SM = 21 * RD_T * sizeof(float4);
+template <int MINB>
+__global__ void __launch_bounds__(RD_T, 2 * MINB) k_b_regen_df(const BSeq* __restrict__ S,
+                                                               const int2* __restrict__ work, int i, df emu,
+                                                               df emum) {
+    const int2 wk = work[blockIdx.x];  // sequence, first site (set-up data)
+    const BSeq& q = S[wk.x];
+    const size_t V = (size_t)q.g.V;
+    // (threads past the lattice take its last site and write nothing)
+    const bool own = wk.y + (int)threadIdx.x < q.g.V;
+    const int site = own ? wk.y + (int)threadIdx.x : q.g.V - 1;
+    int ne = __ldg(q.nbr + site), nx = __ldg(q.nbr + 4 * V + site);
+    pdl_wait_and_release();
+    const float4* __restrict__ x = reinterpret_cast<const float4*>(q.r[i % 3]);
+    const float4* __restrict__ U = reinterpret_cast<const float4*>(q.Udf);
+    // this thread's operands of a hop: 12 chunks of the neighbour's spinor, then 9 link elements
+    extern __shared__ __align__(16) float4 rd_sm[];
+    float4* ps = rd_sm + threadIdx.x;
+    float4* us = ps + 12 * RD_T;
+    // copies of hop hh's spinor / link row a (hop order: direction hh >> 1, forward first)
+    auto fetch_spinor = [&](int ne) {
+        const float4* xb = x + (ne < 0 ? ~ne : ne);
+#pragma unroll
+        for (int c = 0; c < 12; ++c) cp_async16(ps + c * RD_T, xb + (size_t)c * V);
+    };
+    auto fetch_row = [&](int hh, int ne, int a) {
+        const bool fwd = (hh & 1) == 0;
+        const float4* u = U + (size_t)(hh >> 1) * 9 * V + (fwd ? site : (ne < 0 ? ~ne : ne));
+        const size_t srow = fwd ? 3 * V : V, scol = fwd ? V : 3 * V;  // U: row a; U^dag: column a
+#pragma unroll
+        for (int k = 0; k < 3; ++k) cp_async16(us + (3 * a + k) * RD_T, u + (size_t)a * srow + (size_t)k * scol);
+    };
+    const float2 one = make_float2(1.f, 1.f);
+    CAcc2 up[3], lw[3];
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {
+        up[a].r.s = up[a].r.e = up[a].i.s = up[a].i.e = make_float2(0.f, 0.f);
+        lw[a] = up[a];
+    }
+    // the first hop's copies leave before the state is read (a finished sequence only drops them)
+    fetch_spinor(ne);
+    cp_async_commit();
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {
+        fetch_row(0, ne, a);
+        cp_async_commit();
+    }
+    if (q.ks->status || i + 1 >= q.ks->kused) {
+        cp_async_wait<0>();
+        return;
+    }
+    const float4* __restrict__ xm = reinterpret_cast<const float4*>(q.r[(i + 2) % 3]);
+#pragma unroll 1
+    for (int hh = 0; hh < 8; ++hh) {
+        const int nu = hh >> 1;
+        const bool fwd = (hh & 1) == 0;
+        if (hh == 4) {  // the lower sums were kept as spins (3, 2) for nu < 2; (2, 3) from here
+#pragma unroll
+            for (int a = 0; a < 3; ++a) {
+                lw[a].r.s = make_float2(lw[a].r.s.y, lw[a].r.s.x);
+                lw[a].r.e = make_float2(lw[a].r.e.y, lw[a].r.e.x);
+                lw[a].i.s = make_float2(lw[a].i.s.y, lw[a].i.s.x);
+                lw[a].i.e = make_float2(lw[a].i.e.y, lw[a].i.e.x);
+            }
+        }
+        const bool flip = ne < 0;  // the hop crosses the antiperiodic boundary
+        ne = nx;
+        if (hh < 6) nx = __ldg(q.nbr + (size_t)(((hh + 2) >> 1) + (fwd ? 0 : 4)) * V + site);
+        const float fs = fwd ? 1.f : -1.f;
+        // signs of the projected lower components in spins 0, 1 (chiral basis)
+        const float2 sg = make_float2(nu == 3 ? fs : -fs, nu == 0 ? -fs : fs);
+        CAcc2 h[3];
+        // groups in flight: this hop's spinor and three link rows, one group each; every group is
+        // replaced by the next hop's once it is consumed, so three younger ones are always behind
+        cp_async_wait<3>();
+        switch (nu) {
+            case 0: project_dfx<0, RD_T>(ps, sg, h); break;
+            case 1: project_dfx<1, RD_T>(ps, sg, h); break;
+            case 2: project_dfx<2, RD_T>(ps, sg, h); break;
+            default: project_dfx<3, RD_T>(ps, sg, h); break;
+        }
+        // behind the last hop come the recurrence's operands: the own r_i in the spinor's slots, the first
+        // nine chunks of r_{i-1} in the link's
+        fetch_spinor(hh < 7 ? ne : site);
+        cp_async_commit();
+        // signs of the half spinor in the lower spins: (from spin 0, from spin 1)
+        const float sA = fs, sB = (nu == 0 || nu == 3) ? fs : -fs;
+        const float2 lsg = nu < 2 ? make_float2(sB, sA) : make_float2(sA, sB);
+        const bool im = (nu & 1) == 0;
+#pragma unroll
+        for (int a = 0; a < 3; ++a) {
+            CAcc2 o;
+            cp_async_wait<3>();
+            const float4 u3[3] = {us[3 * a * RD_T], us[(3 * a + 1) * RD_T], us[(3 * a + 2) * RD_T]};
+            if (hh < 7) {
+                fetch_row(hh + 1, ne, a);
+            } else if (i > 0) {
+#pragma unroll
+                for (int k = 0; k < 3; ++k)
+                    cp_async16(us + (3 * a + k) * RD_T, xm + (size_t)(3 * a + k) * V + site);
+            }
+            cp_async_commit();
+#pragma unroll
+            for (int k = 0; k < 3; ++k) {
+                const float4 v = u3[k];
+                const float2 rh = f2_dup(v.x), rl = f2_dup(v.y);
+                const float2 ih = f2_dup(fs * v.z), il = f2_dup(fs * v.w);  // U^dag: conjugate
+                if (k == 0) {
+                    dfacc2_first(o.r, rh, rl, h[k].r.s, h[k].r.e);
+                    dfacc2_first(o.i, rh, rl, h[k].i.s, h[k].i.e);
+                } else {
+                    dfacc2_add(o.r, rh, rl, h[k].r.s, h[k].r.e);
+                    dfacc2_add(o.i, rh, rl, h[k].i.s, h[k].i.e);
+                }
+                dfacc2_add(o.r, f2_neg(ih), f2_neg(il), h[k].i.s, h[k].i.e);
+                dfacc2_add(o.i, ih, il, h[k].r.s, h[k].r.e);
+            }
+            if (nu == 3) {
+                const df e0 = fwd ? emu : emum;
+                const float2 ch = f2_dup(flip ? -e0.hi : e0.hi), cl = f2_dup(flip ? -e0.lo : e0.lo);
+                dfacc2 t;
+                dfacc2_first(t, ch, cl, o.r.s, o.r.e);
+                o.r = t;
+                dfacc2_first(t, ch, cl, o.i.s, o.i.e);
+                o.i = t;
+            }
+            dfacc2_add_signed(up[a].r, one, o.r.s, o.r.e);
+            dfacc2_add_signed(up[a].i, one, o.i.s, o.i.e);
+            if (im) {
+                dfacc2_add_signed(lw[a].r, f2_neg(lsg), o.i.s, o.i.e);
+                dfacc2_add_signed(lw[a].i, lsg, o.r.s, o.r.e);
+            } else {
+                dfacc2_add_signed(lw[a].r, lsg, o.r.s, o.r.e);
+                dfacc2_add_signed(lw[a].i, lsg, o.i.s, o.i.e);
+            }
+        }
+    }
+    const RegenCoefDf* __restrict__ rc = q.rc + i;
+    const float4 kb = __ldg(&rc->kb), cg = __ldg(&rc->cg), cc = __ldg(&rc->cc);
+    float4* __restrict__ xn = reinterpret_cast<float4*>(q.r[(i + 1) % 3]);
+    float4* __restrict__ y = reinterpret_cast<float4*>(q.y);
+    cp_async_wait<0>();
+    if (!own) return;
+#pragma unroll
+    for (int P = 0; P < 2; ++P) {
+        const float4 cr = __ldg(P ? &rc->cl : &rc->cu);
+        const float ks_ = P ? 1.f : -1.f;
+        const float2 kh = f2_dup(ks_ * kb.x), kl = f2_dup(ks_ * kb.y);
+        const float2 arh = f2_dup(cr.x), arl = f2_dup(cr.y), aih = f2_dup(cr.z), ail = f2_dup(cr.w);
+        const float2 grh = f2_dup(cg.x), grl = f2_dup(cg.y), gih = f2_dup(cg.z), gil = f2_dup(cg.w);
+        const float2 crh = f2_dup(cc.x), crl = f2_dup(cc.y), cih = f2_dup(cc.z), cil = f2_dup(cc.w);
+#pragma unroll
+        for (int a = 0; a < 3; ++a) {
+            const size_t e = (size_t)(P * 3 + a) * 2 * V + site;
+            CAcc2 s = P ? lw[a] : up[a];
+            s.r = dfacc2_value(s.r);
+            s.i = dfacc2_value(s.i);
+            const int c = (P * 3 + a) * 2;
+            const float4 xr = ps[c * RD_T], xi = ps[(c + 1) * RD_T];
+            const float2 xrh = make_float2(xr.x, xr.y), xrl = make_float2(xr.z, xr.w);
+            const float2 xih = make_float2(xi.x, xi.y), xil = make_float2(xi.z, xi.w);
+            CAcc2 z;
+            dfacc2_first(z.r, kh, kl, s.r.s, s.r.e);
+            dfacc2_first(z.i, kh, kl, s.i.s, s.i.e);
+            dfacc2_add(z.r, arh, arl, xrh, xrl);
+            dfacc2_add(z.i, arh, arl, xih, xil);
+            dfacc2_add(z.r, f2_neg(aih), f2_neg(ail), xih, xil);
+            dfacc2_add(z.i, aih, ail, xrh, xrl);
+            if (i > 0) {
+                const float4 mr = c < 9 ? us[c * RD_T] : __ldg(xm + e);
+                const float4 mi = c + 1 < 9 ? us[(c + 1) * RD_T] : __ldg(xm + e + V);
+                const float2 mrh = make_float2(mr.x, mr.y), mrl = make_float2(mr.z, mr.w);
+                const float2 mih = make_float2(mi.x, mi.y), mil = make_float2(mi.z, mi.w);
+                dfacc2_add(z.r, grh, grl, mrh, mrl);
+                dfacc2_add(z.i, grh, grl, mih, mil);
+                dfacc2_add(z.r, f2_neg(gih), f2_neg(gil), mih, mil);
+                dfacc2_add(z.i, gih, gil, mrh, mrl);
+            }
+            const dfacc2 zr = dfacc2_value(z.r), zi = dfacc2_value(z.i);
+            xn[e] = make_float4(zr.s.x, zr.s.y, zr.e.x, zr.e.y);
+            xn[e + V] = make_float4(zi.s.x, zi.s.y, zi.e.x, zi.e.y);
+            const float4 y0 = y[e], y1 = y[e + V];
+            // c z summed by itself, then added to y: every rounding at the scale of y's low part stays in y
+            // for the rest of the pass (over 480 steps they are its error), and this way there is one
+            dfacc2 yr, yi, pr, pi;
+            yr.s = make_float2(y0.x, y0.y), yr.e = make_float2(y0.z, y0.w);
+            yi.s = make_float2(y1.x, y1.y), yi.e = make_float2(y1.z, y1.w);
+            dfacc2_first(pr, crh, crl, zr.s, zr.e);
+            dfacc2_first(pi, crh, crl, zi.s, zi.e);
+            dfacc2_add(pr, f2_neg(cih), f2_neg(cil), zi.s, zi.e);
+            dfacc2_add(pi, cih, cil, zr.s, zr.e);
+            dfacc2_add_tight(yr, pr.s, pr.e);
+            dfacc2_add_tight(yi, pi.s, pi.e);
+            yr = dfacc2_value(yr);
+            yi = dfacc2_value(yi);
+            y[e] = make_float4(yr.s.x, yr.s.y, yr.e.x, yr.e.y);
+            y[e + V] = make_float4(yi.s.x, yi.s.y, yi.e.x, yi.e.y);
+        }
+    }
+}
+
+// ---- FP64 regeneration: one block per 32-site tile of a sequence: warp h applies hop h
+// (direction-uniform code) to the tile's sites, the eight partial sums meet in shared memory, and 256
+// threads (site, part) finish the components.
+template <int MINB>
 __global__ void __launch_bounds__(8 * TT, MINB) k_b_regen(const BSeq* __restrict__ S, const int* __restrict__ tseq, int i,
-                                                    HopCoef<R> hc) {
-    using VT = typename VecT<R>::T;
+                                                    HopCoef<double> hc) {
+    using R = double;
+    using VT = double2;
     extern __shared__ __align__(16) unsigned char smraw[];
     cx<R>(*dirpart)[TT][6] = reinterpret_cast<cx<R>(*)[TT][6]>(smraw);  // [8][TT][2 spins x 3 colours]
     __shared__ cx<R> cf[4];
@@ -666,30 +957,26 @@ __global__ void __launch_bounds__(8 * TT, MINB) k_b_regen(const BSeq* __restrict
     if (ks->status || i + 1 >= ks->kused) return;
     if (threadIdx.x == 0) {
         const cx<double> ib = cdiv(mk(1.0, 0.0), d2c(q.beta[i]));
-        cf[0] = cvt_coef<R>(ib);
-        cf[1] = cvt_coef<R>(ib * d2c(q.alpha[i]));
-        cf[2] = cvt_coef<R>(i > 0 ? ib * d2c(q.gamma[i - 1]) : mk(0.0, 0.0));
-        cf[3] = cvt_coef<R>(d2c(q.cvec[i + 1]));
+        cf[0] = (ib);
+        cf[1] = (ib * d2c(q.alpha[i]));
+        cf[2] = (i > 0 ? ib * d2c(q.gamma[i - 1]) : mk(0.0, 0.0));
+        cf[3] = (d2c(q.cvec[i + 1]));
     }
     const int tile = blockIdx.x - q.tile0;
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     const VT* ri = (const VT*)q.r[i % 3];
-    const void* U = LF == LINK_DF ? q.Udf : (const void*)q.U64;
+    const void* U = q.U64;
     {
         // warp wid: hop wid of the tile's 32 sites, kept as its half spinor
         const int i0 = tile * TT + lane;
         if (i0 < q.g.V) {
-            if constexpr (LF == LINK_DF) {
-                hop_half_rows_df(wid, q.g, q.nbr, i0, (const dfc*)U, (const dfc*)ri, hc, dirpart[wid][lane]);
-            } else {
-                const Coord c = site_coord(q.g, i0);
-                const VT* const xs[1] = {ri};
-                const HopCoef<R> hcs[1] = {hc};
-                Half<R> hp[1];
-                hop_half_uniform<LF, R, 1>(wid, q.g, c, i0, U, xs, hp, hcs);
+            const Coord c = site_coord(q.g, i0);
+            const VT* const xs[1] = {ri};
+            const HopCoef<R> hcs[1] = {hc};
+            Half<R> hp[1];
+            hop_half_uniform<LINK_F64, R, 1>(wid, q.g, c, i0, U, xs, hp, hcs);
 #pragma unroll
-                for (int c6 = 0; c6 < 6; ++c6) dirpart[wid][lane][c6] = hp[0].h[c6 / 3][c6 % 3];
-            }
+            for (int c6 = 0; c6 < 6; ++c6) dirpart[wid][lane][c6] = hp[0].h[c6 / 3][c6 % 3];
         }
     }
     __syncthreads();
@@ -722,10 +1009,11 @@ __global__ void __launch_bounds__(8 * TT, MINB) k_b_regen(const BSeq* __restrict
 // the neighbour index once and runs the two sequences' double-float products as independent chains
 // (twice the work in flight per warp); the epilogue spreads the 2 x 32 sites x 12 components over
 // the 256 threads, three each.  Same arithmetic per sequence as k_b_regen.
-template <class R, int LF, int MINB>
+template <int MINB>
 __global__ void __launch_bounds__(8 * TT, MINB) k_b_regen2(const BSeq* __restrict__ S, const int4* __restrict__ work,
-                                                     int i, HopCoef<R> hc) {
-    using VT = typename VecT<R>::T;
+                                                     int i, HopCoef<double> hc) {
+    using R = double;
+    using VT = double2;
     extern __shared__ __align__(16) unsigned char smraw[];
     cx<R>(*dirpart)[8][TT][6] = reinterpret_cast<cx<R>(*)[8][TT][6]>(smraw);  // [2][8][TT][6]
     __shared__ cx<R> cf[2][4];
@@ -740,34 +1028,29 @@ __global__ void __launch_bounds__(8 * TT, MINB) k_b_regen2(const BSeq* __restric
     if (threadIdx.x < 2 && (threadIdx.x == 0 || two)) {
         const BSeq& q = threadIdx.x ? qb : qa;
         const cx<double> ib = cdiv(mk(1.0, 0.0), d2c(q.beta[i]));
-        cf[threadIdx.x][0] = cvt_coef<R>(ib);
-        cf[threadIdx.x][1] = cvt_coef<R>(ib * d2c(q.alpha[i]));
-        cf[threadIdx.x][2] = cvt_coef<R>(i > 0 ? ib * d2c(q.gamma[i - 1]) : mk(0.0, 0.0));
-        cf[threadIdx.x][3] = cvt_coef<R>(d2c(q.cvec[i + 1]));
+        cf[threadIdx.x][0] = (ib);
+        cf[threadIdx.x][1] = (ib * d2c(q.alpha[i]));
+        cf[threadIdx.x][2] = (i > 0 ? ib * d2c(q.gamma[i - 1]) : mk(0.0, 0.0));
+        cf[threadIdx.x][3] = (d2c(q.cvec[i + 1]));
     }
     const int tile = wk.z;
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     const Geom& g = qa.g;
     const VT* ra = (const VT*)qa.r[i % 3];
     const VT* rb = two ? (const VT*)qb.r[i % 3] : ra;
-    const void* U = LF == LINK_DF ? qa.Udf : (const void*)qa.U64;
+    const void* U = qa.U64;
     {
         const int i0 = tile * TT + lane;
         if (i0 < g.V) {
-            if constexpr (LF == LINK_DF) {
-                hop_half_rows_df(wid, g, qa.nbr, i0, (const dfc*)U, (const dfc*)ra, hc, dirpart[0][wid][lane]);
-                hop_half_rows_df(wid, g, qa.nbr, i0, (const dfc*)U, (const dfc*)rb, hc, dirpart[1][wid][lane]);
-            } else {
-                const Coord c = site_coord(g, i0);
-                const VT* const xs[2] = {ra, rb};
-                const HopCoef<R> hcs[2] = {hc, hc};
-                Half<R> hp[2];
-                hop_half_uniform<LF, R, 2>(wid, g, c, i0, U, xs, hp, hcs);
+            const Coord c = site_coord(g, i0);
+            const VT* const xs[2] = {ra, rb};
+            const HopCoef<R> hcs[2] = {hc, hc};
+            Half<R> hp[2];
+            hop_half_uniform<LINK_F64, R, 2>(wid, g, c, i0, U, xs, hp, hcs);
 #pragma unroll
-                for (int c6 = 0; c6 < 6; ++c6) {
-                    dirpart[0][wid][lane][c6] = hp[0].h[c6 / 3][c6 % 3];
-                    dirpart[1][wid][lane][c6] = hp[1].h[c6 / 3][c6 % 3];
-                }
+            for (int c6 = 0; c6 < 6; ++c6) {
+                dirpart[0][wid][lane][c6] = hp[0].h[c6 / 3][c6 % 3];
+                dirpart[1][wid][lane][c6] = hp[1].h[c6 / 3][c6 % 3];
             }
         }
     }
@@ -818,8 +1101,10 @@ struct ovl_batch {
     ovl::BSeq* dseq = nullptr;
     int* dbseq[ovl::NSHAPE] = {nullptr, nullptr, nullptr};
     int* dtseq = nullptr;
-    int4* dpair = nullptr;         // regeneration work of two sequences per block: (a, b, tile, two)
+    int4* dpair = nullptr;         // FP64 regeneration, two sequences per block: (a, b, tile, two)
     int npair_blocks = 0;
+    int2* drd = nullptr;           // double-float regeneration work: (sequence, first site)
+    int nrd = 0;
     unsigned int* pbar = nullptr;  // per-sequence barrier counters of the persistent pass 1
     int bp1_fit = -1;              // persistent pass 1 fits the GPU (-1: not yet determined)
     int nblocks[ovl::NSHAPE] = {0, 0, 0};
@@ -926,6 +1211,18 @@ int balloc(ovl_batch* b, int mode, int kmax) {
             s0 += b->nrhs[j];
         }
     }
+    // double-float regeneration: blocks of RD_T sites of one sequence, a lattice's sequences side by
+    // side (the same links are read at about the same time)
+    std::vector<int2> rtable;
+    if (mode == 1) {
+        int s0 = 0;
+        for (size_t j = 0; j < b->ctx.size(); ++j) {
+            for (int site = 0; site < b->ctx[j]->g.V; site += ovl::RD_T)
+                for (int r = 0; r < b->nrhs[j]; ++r) rtable.push_back(make_int2(s0 + r, site));
+            s0 += b->nrhs[j];
+        }
+    }
+    const size_t rcb = mode == 1 ? ns * kk * sizeof(ovl::RegenCoefDf) : 0;
     std::vector<size_t> pro_off(ns + 1, 0);
     std::vector<int> pro_m(ns, 0);
     for (int s = 0; s < ns; ++s) {
@@ -939,6 +1236,7 @@ int balloc(ovl_batch* b, int mode, int kmax) {
              al(ns * 64 * sizeof(unsigned int)) + al(ns * sizeof(ovl::BSeq)) + al(nblocks[0] * sizeof(int)) +
              al(nblocks[1] * sizeof(int)) + al(nblocks[2] * sizeof(int)) +
              al(ntiles * sizeof(int)) + al(ns * sizeof(unsigned int)) + al(ptable.size() * sizeof(int4)) +
+             al(rtable.size() * sizeof(int2)) + al(rcb) +
              al(pro_off[ns] * sizeof(double)) + al(64 * sizeof(unsigned int));
     if (cudaMalloc(&b->mem, total) != cudaSuccess) {
         b->mem = nullptr;
@@ -964,6 +1262,9 @@ int balloc(ovl_batch* b, int mode, int kmax) {
     b->pbar = (unsigned int*)take(ns * sizeof(unsigned int));
     b->dpair = (int4*)take(ptable.size() * sizeof(int4));
     b->npair_blocks = (int)ptable.size();
+    b->drd = (int2*)take(rtable.size() * sizeof(int2));
+    b->nrd = (int)rtable.size();
+    ovl::RegenCoefDf* rc = (ovl::RegenCoefDf*)take(rcb);
     b->part = (double*)take(pro_off[ns] * sizeof(double));
     b->pro_off = pro_off;
     b->pro_m = pro_m;
@@ -988,6 +1289,8 @@ int balloc(ovl_batch* b, int mode, int kmax) {
         b->bR[s] = (double2*)take(n * sizeof(double2));
         b->bL[s] = (double2*)take(n * sizeof(double2));
         q.y = (double2*)take(n * sizeof(double2));
+        q.bR = b->bR[s];
+        q.rc = mode == 1 ? rc + s * kk : nullptr;
         for (int j = 0; j < 3; ++j) q.r[j] = (double2*)take(n * sizeof(double2));
         if (mode == 1) {
             for (int j = 0; j < 3; ++j) q.v[j] = take(n * sizeof(float2)), q.w[j] = take(n * sizeof(float2));
@@ -1033,6 +1336,7 @@ int balloc(ovl_batch* b, int mode, int kmax) {
         cudaMemcpy(b->dbseq[2], table[2].data(), table[2].size() * sizeof(int), cudaMemcpyHostToDevice) != cudaSuccess ||
         cudaMemcpy(b->dtseq, ttable.data(), ttable.size() * sizeof(int), cudaMemcpyHostToDevice) != cudaSuccess ||
         cudaMemcpy(b->dpair, ptable.data(), ptable.size() * sizeof(int4), cudaMemcpyHostToDevice) != cudaSuccess ||
+        cudaMemcpy(b->drd, rtable.data(), rtable.size() * sizeof(int2), cudaMemcpyHostToDevice) != cudaSuccess ||
         cudaMemset(b->qcnt, 0, ns * 64 * sizeof(unsigned int)) != cudaSuccess ||
         cudaMemset(b->counter, 0, 64 * sizeof(unsigned int)) != cudaSuccess) {
         bfree(b);
@@ -1110,37 +1414,33 @@ void pass1_step(ovl_batch* b, int i, int k, double mu, double kappa, bool mixed,
     }
 }
 
-// One regeneration step of every sequence, blocks-per-SM bound MINB (one or two sequences per block).
+// One double-float regeneration step of every sequence, compiled for 3 or 4 times 128 threads per SM (163
+// or 128 registers).  Neither is best everywhere: 48 sequences on four lattices 303 / 290 us, 12 on 8^4
+// 28.9 / 36.8 us (768 blocks: at eight per SM the next step's blocks, launched early, crowd on a few SMs).
 template <int MINB>
-void regen_step(ovl_batch* b, int i, double mu, double kappa, bool dfm, cudaStream_t st) {
+void regen_df_step(ovl_batch* b, int i, double mu, cudaStream_t st) {
+    static unsigned long long attr_dev = 0;
+    if (ovl::first_use_on_device(attr_dev))
+        cudaFuncSetAttribute(ovl::k_b_regen_df<MINB>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ovl::RD_SM);
+    launch_pdl(ovl::k_b_regen_df<MINB>, b->nrd, ovl::RD_T, ovl::RD_SM, st, (const ovl::BSeq*)b->dseq,
+               (const int2*)b->drd, i, ovl::df(exp(mu)), ovl::df(exp(-mu)));
+}
+
+// One FP64 regeneration step of every sequence, blocks-per-SM bound MINB (one or two sequences per block).
+template <int MINB>
+void regen_step(ovl_batch* b, int i, double mu, double kappa, cudaStream_t st) {
+    const ovl::BSeq* S = b->dseq;
     const size_t smr = (size_t)8 * ovl::TT * 6 * 16;
     static unsigned long long attr_dev = 0;
     if (ovl::first_use_on_device(attr_dev)) {
-        cudaFuncSetAttribute(ovl::k_b_regen<ovl::df, ovl::LINK_DF, MINB>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)smr);
-        cudaFuncSetAttribute(ovl::k_b_regen<double, ovl::LINK_F64, MINB>,
-                             cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smr);
-        cudaFuncSetAttribute(ovl::k_b_regen2<ovl::df, ovl::LINK_DF, MINB>,
-                             cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(2 * smr));
-        cudaFuncSetAttribute(ovl::k_b_regen2<double, ovl::LINK_F64, MINB>,
-                             cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(2 * smr));
+        cudaFuncSetAttribute(ovl::k_b_regen<MINB>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smr);
+        cudaFuncSetAttribute(ovl::k_b_regen2<MINB>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(2 * smr));
     }
-    const ovl::BSeq* S = b->dseq;
-    if (b->regen_pair) {
-        if (dfm)
-            launch_pdl(ovl::k_b_regen2<ovl::df, ovl::LINK_DF, MINB>, b->npair_blocks, 8 * ovl::TT, 2 * smr, st, S,
-                       (const int4*)b->dpair, i, ovl::make_coef<ovl::df>(mu, kappa));
-        else
-            launch_pdl(ovl::k_b_regen2<double, ovl::LINK_F64, MINB>, b->npair_blocks, 8 * ovl::TT, 2 * smr, st, S,
-                       (const int4*)b->dpair, i, ovl::make_coef<double>(mu, kappa));
-        return;
-    }
-    const int* tab = b->dtseq;
-    if (dfm)
-        launch_pdl(ovl::k_b_regen<ovl::df, ovl::LINK_DF, MINB>, b->ntiles, 8 * ovl::TT, smr, st, S, tab, i,
-                   ovl::make_coef<ovl::df>(mu, kappa));
+    if (b->regen_pair)
+        launch_pdl(ovl::k_b_regen2<MINB>, b->npair_blocks, 8 * ovl::TT, 2 * smr, st, S, (const int4*)b->dpair, i,
+                   ovl::make_coef<double>(mu, kappa));
     else
-        launch_pdl(ovl::k_b_regen<double, ovl::LINK_F64, MINB>, b->ntiles, 8 * ovl::TT, smr, st, S, tab, i,
+        launch_pdl(ovl::k_b_regen<MINB>, b->ntiles, 8 * ovl::TT, smr, st, S, (const int*)b->dtseq, i,
                    ovl::make_coef<double>(mu, kappa));
 }
 
@@ -1222,25 +1522,30 @@ int enqueue_batch(ovl_batch* b, int k, double mu, double kappa, int flags, cudaS
     if (twopass) {
         // mixed: double-float regeneration unless OVL_PASS2_F64 (ring and y converted in place)
         const bool dfm = mixed && !(flags & OVL_PASS2_F64);
-        for (int s = 0; s < ns; ++s) {
-            const ovl::BSeq& q = b->hseq[s];
-            ovl::launch_scale_start(b->bR[s], q.r[0], q.y, q.cvec, q.ks, q.n, st);
-            if (dfm) {
-                ovl::launch_f64_to_df(q.r[0], q.n, st);
-                ovl::launch_f64_to_df(q.y, q.n, st);
+        if (dfm) {
+            if (k > 1) ovl::k_b_regen_coef<<<dim3((k + 126) / 128, ns), 128, 0, st>>>(b->dseq, kappa);
+            ovl::k_b_regen_start<<<b->nblocks[1], 128, 0, st>>>(b->dseq, b->dbseq[1]);
+        } else {
+            for (int s = 0; s < ns; ++s) {
+                const ovl::BSeq& q = b->hseq[s];
+                ovl::launch_scale_start(b->bR[s], q.r[0], q.y, q.cvec, q.ks, q.n, st);
             }
         }
         for (int i = 0; i + 1 < k; ++i) {
+            if (dfm) {
+                if (b->regen_minb <= 3) regen_df_step<3>(b, i, mu, st);
+                else regen_df_step<4>(b, i, mu, st);
+                continue;
+            }
             switch (b->regen_minb) {
-                case 2: regen_step<2>(b, i, mu, kappa, dfm, st); break;
-                case 4: regen_step<4>(b, i, mu, kappa, dfm, st); break;
-                case 5: regen_step<5>(b, i, mu, kappa, dfm, st); break;
-                case 6: regen_step<6>(b, i, mu, kappa, dfm, st); break;
-                default: regen_step<3>(b, i, mu, kappa, dfm, st); break;
+                case 2: regen_step<2>(b, i, mu, kappa, st); break;
+                case 4: regen_step<4>(b, i, mu, kappa, st); break;
+                case 5: regen_step<5>(b, i, mu, kappa, st); break;
+                case 6: regen_step<6>(b, i, mu, kappa, st); break;
+                default: regen_step<3>(b, i, mu, kappa, st); break;
             }
         }
-        if (dfm)
-            for (int s = 0; s < ns; ++s) ovl::launch_df_to_f64(b->hseq[s].y, b->hseq[s].n, st);
+        if (dfm) ovl::k_b_regen_out<<<b->nblocks[1], 128, 0, st>>>(b->dseq, b->dbseq[1]);
     } else {
         for (int s = 0; s < ns; ++s) {
             const ovl::BSeq& q = b->hseq[s];
@@ -1262,7 +1567,9 @@ std::string tune_key(const ovl_batch* b) {
     cudaGetDevice(&dev);
     cudaDeviceProp pr{};
     cudaGetDeviceProperties(&pr, dev);
-    std::string k = std::string(pr.name) + "/" + std::to_string(pr.multiProcessorCount) + "/m" + std::to_string(b->mode);
+    // ("/r2": the double-float regeneration of one thread per site; choices timed for the tile form that
+    // preceded it do not apply)
+    std::string k = std::string(pr.name) + "/" + std::to_string(pr.multiProcessorCount) + "/r2/m" + std::to_string(b->mode);
     for (size_t j = 0; j < b->ctx.size(); ++j) {
         const ovl::Geom& g = b->ctx[j]->g;
         k += "/" + std::to_string(g.L[0]) + "x" + std::to_string(g.L[1]) + "x" + std::to_string(g.L[2]) + "x" +
@@ -1315,15 +1622,19 @@ int autotune(ovl_batch* b, double mu, double kappa, int flags, cudaStream_t st) 
     struct Cand {
         int shape, minb, pair;
     };
+    // the double-float regeneration has two forms (3 or 4 times 128 threads per SM), the FP64 one seven
     const Cand cands[] = {{0, 3, 0}, {1, 4, 0}, {2, 5, 0}, {1, 6, 0}, {1, 2, 1}, {1, 3, 1}, {1, 4, 1}};
-    const int ncand = (int)(sizeof(cands) / sizeof(cands[0]));
+    const Cand cands_df[] = {{0, 3, 0}, {1, 4, 0}, {2, 4, 0}};
+    const bool dfm = b->mode == 1 && !(flags & OVL_PASS2_F64);
+    const Cand* cand = dfm ? cands_df : cands;
+    const int ncand = dfm ? (int)(sizeof(cands_df) / sizeof(cands_df[0])) : (int)(sizeof(cands) / sizeof(cands[0]));
     float best1 = 1e30f, best2 = 1e30f;
     int bs = saved_shape, bm = saved_minb, bp = b->regen_pair;
     for (int rep = 0; rep < 2; ++rep)  // the first round warms caches and instruction memory
         for (int c = 0; c < ncand; ++c) {
-            b->shape = cands[c].shape;
-            b->regen_minb = cands[c].minb;
-            b->regen_pair = cands[c].pair;
+            b->shape = cand[c].shape;
+            b->regen_minb = cand[c].minb;
+            b->regen_pair = cand[c].pair;
             const int r = enqueue_batch(b, TUNE_K, mu, kappa, (flags | OVL_PROFILE) & ~OVL_NO_GRAPH, st);
             if (r) return r;
             if (cudaStreamSynchronize(st) != cudaSuccess) return bfail(b, OVL_ECUDA, "tuning solve");
@@ -1331,8 +1642,8 @@ int autotune(ovl_batch* b, double mu, double kappa, int flags, cudaStream_t st) 
             cudaEventElapsedTime(&t1, b->ev[0], b->ev[1]);
             cudaEventElapsedTime(&t2, b->ev[2], b->ev[3]);
             if (rep == 1) {
-                if (t1 < best1) best1 = t1, bs = cands[c].shape;
-                if (t2 < best2) best2 = t2, bm = cands[c].minb, bp = cands[c].pair;
+                if (t1 < best1) best1 = t1, bs = cand[c].shape;
+                if (t2 < best2) best2 = t2, bm = cand[c].minb, bp = cand[c].pair;
             }
         }
     b->shape = bs;

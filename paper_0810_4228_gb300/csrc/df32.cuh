@@ -198,6 +198,92 @@ __device__ __forceinline__ void load_link_df(const dfc* __restrict__ U, int V, i
     }
 }
 
+// Two independent double-float numbers side by side (the two spins of a half spinor): every operation
+// is one packed FP32x2 instruction, so a warp issues half the instructions of the scalar form.  The
+// FP32 pipe's rate is the same either way (measured on chains of link products: 30.9 Top/s scalar,
+// 30.2 packed); what the packing frees is issue slots and latency, which loads and address arithmetic
+// otherwise compete for.  Each half is computed as the scalar operation would compute it.
+#if defined(__CUDA_ARCH__) && __CUDA_ARCH__ >= 1000
+#define OVL_F32X2 1
+#endif
+OVL_HD float2 f2_add(float2 a, float2 b) {
+#ifdef OVL_F32X2
+    return __fadd2_rn(a, b);
+#else
+    return make_float2(DF_ADD(a.x, b.x), DF_ADD(a.y, b.y));
+#endif
+}
+OVL_HD float2 f2_sub(float2 a, float2 b) { return f2_add(a, make_float2(-b.x, -b.y)); }
+OVL_HD float2 f2_mul(float2 a, float2 b) {
+#ifdef OVL_F32X2
+    return __fmul2_rn(a, b);
+#else
+    return make_float2(DF_MUL(a.x, b.x), DF_MUL(a.y, b.y));
+#endif
+}
+OVL_HD float2 f2_fma(float2 a, float2 b, float2 c) {
+#ifdef OVL_F32X2
+    return __ffma2_rn(a, b, c);
+#else
+    return make_float2(DF_FMA(a.x, b.x, c.x), DF_FMA(a.y, b.y, c.y));
+#endif
+}
+OVL_HD float2 f2_dup(float a) { return make_float2(a, a); }
+OVL_HD float2 f2_neg(float2 a) { return make_float2(-a.x, -a.y); }
+
+// pair of unevaluated sums s + e
+struct dfacc2 {
+    float2 s, e;
+};
+// A = a b, a = ah + al and b = bh + bl double-float
+OVL_HD void dfacc2_first(dfacc2& A, float2 ah, float2 al, float2 bh, float2 bl) {
+    const float2 p = f2_mul(ah, bh);
+    float2 pe = f2_fma(ah, bh, f2_neg(p));
+    pe = f2_fma(ah, bl, pe);
+    A.s = p;
+    A.e = f2_fma(al, bh, pe);
+}
+// A += a b (as dfacc_add)
+OVL_HD void dfacc2_add(dfacc2& A, float2 ah, float2 al, float2 bh, float2 bl) {
+    const float2 p = f2_mul(ah, bh);
+    float2 pe = f2_fma(ah, bh, f2_neg(p));
+    pe = f2_fma(ah, bl, pe);
+    pe = f2_fma(al, bh, pe);
+    const float2 s = f2_add(A.s, p);
+    const float2 bb = f2_sub(s, A.s);
+    const float2 t = f2_add(f2_sub(A.s, f2_sub(s, bb)), f2_sub(p, bb));
+    A.s = s;
+    A.e = f2_add(A.e, f2_add(t, pe));
+}
+// A += sg x for sg = +-1 in each half: TwoSum of the leading parts, the sign applied exactly by the
+// fused multiply-adds
+OVL_HD void dfacc2_add_signed(dfacc2& A, float2 sg, float2 xs, float2 xe) {
+    const float2 s = f2_fma(sg, xs, A.s);
+    const float2 bb = f2_sub(s, A.s);
+    const float2 t = f2_add(f2_sub(A.s, f2_sub(s, bb)), f2_fma(sg, xs, f2_neg(bb)));
+    A.s = s;
+    A.e = f2_add(f2_fma(sg, xe, A.e), t);
+}
+// A += x with the low parts summed without loss before the last addition: one rounding at the scale of
+// A.e instead of two, for sums of many terms that are kept renormalised (the solution vector)
+OVL_HD void dfacc2_add_tight(dfacc2& A, float2 xs, float2 xe) {
+    const float2 s = f2_add(A.s, xs);
+    const float2 bb = f2_sub(s, A.s);
+    const float2 t = f2_add(f2_sub(A.s, f2_sub(s, bb)), f2_sub(xs, bb));
+    const float2 g = f2_add(A.e, t);
+    const float2 gb = f2_sub(g, A.e);
+    const float2 d = f2_add(f2_sub(A.e, f2_sub(g, gb)), f2_sub(t, gb));
+    A.s = s;
+    A.e = f2_add(g, f2_add(d, xe));
+}
+// renormalised value: hi = s + e, lo the rounding error (Fast2Sum)
+OVL_HD dfacc2 dfacc2_value(const dfacc2& A) {
+    dfacc2 r;
+    r.s = f2_add(A.s, A.e);
+    r.e = f2_sub(A.e, f2_sub(r.s, A.s));
+    return r;
+}
+
 // in-block accumulators: compensated FP32 pairs for FP32 data, plain FP64 for FP64 data.
 // AccF adds each exact product p + pe (TwoProduct by FMA) with TwoSum into hi and collects the
 // rounding errors and the pe terms in lo (the compensated dot product of Ogita, Rump and Oishi,

@@ -39,7 +39,6 @@ void launch_pack_gauge(const double2* U_canon, double2* U64, float4* U12, float2
                        cudaStream_t st);
 // in place: FP64 vectors (double2) -> double-float (float4 {hi, lo, hi, lo}), n complex each; and back
 void launch_f64_to_df(void* x, size_t n, cudaStream_t st);
-void launch_df_to_f64(void* x, size_t n, cudaStream_t st);
 void launch_pack_spinor(const double2* canon, void* native, int prec, const Geom& g, cudaStream_t st);
 // out_canon = b_canon (if given) + (g5 ? gamma5 : 1) * native
 void launch_unpack_spinor(const void* native, int prec, double2* canon, const double2* b_canon, int g5,

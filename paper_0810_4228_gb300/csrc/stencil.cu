@@ -598,17 +598,8 @@ __global__ void k_f64_to_df(void* x, size_t n) {
         reinterpret_cast<dfc*>(x)[e] = c2dfc(d2df(v));
     }
 }
-__global__ void k_df_to_f64(void* x, size_t n) {
-    for (size_t e = blockIdx.x * (size_t)blockDim.x + threadIdx.x; e < n; e += (size_t)gridDim.x * blockDim.x) {
-        const dfc v = reinterpret_cast<dfc*>(x)[e];
-        reinterpret_cast<double2*>(x)[e] = df2d(dfc2c(v));
-    }
-}
 void launch_f64_to_df(void* x, size_t n, cudaStream_t st) {
     k_f64_to_df<<<(int)std::min<size_t>((n + 255) / 256, 2048), 256, 0, st>>>(x, n);
-}
-void launch_df_to_f64(void* x, size_t n, cudaStream_t st) {
-    k_df_to_f64<<<(int)std::min<size_t>((n + 255) / 256, 2048), 256, 0, st>>>(x, n);
 }
 
 void launch_pack_gauge(const double2* U_canon, double2* U64, float4* U12, float2* U18, float4* Udf, const Geom& g,
