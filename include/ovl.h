@@ -90,8 +90,8 @@ typedef struct ovl_ctx ovl_ctx;
 /* OVL_REPROJ applied every p-th step only (1 <= p <= 127): the pass-1 vectors of the steps i with
  * (i + 1) % p == 0 are projected; p = 1 is OVL_REPROJ.  p > 1 runs the stepwise kernels. */
 #define OVL_REPROJ_PERIOD(p) (OVL_REPROJ | (((p) & 0x7f) << 24))
-#define OVL_STEPWISE     0x40000 /* sign_krylov MIXED: one kernel per recurrence step instead of the
-                                    persistent cooperative kernels (default on small lattices)   */
+#define OVL_STEPWISE     0x40000 /* sign_krylov LANCZOS2 (MIXED or FP64): one kernel per recurrence step instead
+                                    of the persistent cooperative kernels (default on small lattices) */
 #define OVL_PASS2_F64    0x80000 /* MIXED: regeneration pass in native FP64                       */
 #define OVL_NO_TUNE      0x200000 /* batch_solve: keep the current launch shapes, no autotuning     */
 #define OVL_ARNOLDI_CGS2 0x400000 /* sign_krylov ARNOLDI with MIXED: classical Gram-Schmidt applied

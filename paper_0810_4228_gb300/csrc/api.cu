@@ -356,7 +356,20 @@ int enqueue_solve(ovl_ctx* c, int method, int k, double mu, double kappa, int fl
             if (lr) return fail(c, OVL_ECUDA, std::string("persistent pass 1 launch: ") +
                                                    cudaGetErrorString((cudaError_t)lr));
         }
-        for (int i = 0; i < (persist ? 0 : k); ++i) {
+        // FP64 on lattices that fit the SMs' shared memory: the whole process in one launch as well
+        const bool persist64 = !mixed && !(flags & OVL_STEPWISE) && ovl::l2_f64_ok(g, c->num_sms);
+        if (persist64) {
+            cudaMemsetAsync(c->bar, 0, 64, st);
+            int lr = 0;
+            prof(c, KC_PASS1, [&] {
+                double2* vv[3] = {twopass ? c->R64[0] : c->V64, c->R64[1], c->R64[2]};
+                lr = ovl::launch_l2_f64(c->U64, c->nbr, vv, twopass ? 0 : n, c->W64, 0, ks, c->alpha, c->beta,
+                                        c->gamma, c->vscale, mu, kappa, k, part, c->bar, g, c->num_sms, st);
+            });
+            if (lr) return fail(c, OVL_ECUDA, std::string("persistent FP64 process launch: ") +
+                                                   cudaGetErrorString((cudaError_t)lr));
+        }
+        for (int i = 0; i < (persist || persist64 ? 0 : k); ++i) {
             if (mixed) {
                 prof(c, KC_PAIR, [&] {
                     ovl::launch_dslash_pair(c->U12, 1, c->v32[i % 3], c->w32[i % 3], c->t32, c->s32, mu, kappa, ks,
@@ -418,7 +431,7 @@ int enqueue_solve(ovl_ctx* c, int method, int k, double mu, double kappa, int fl
             prof(c, KC_PASS2, [&] {
                 double2* rr[3] = {c->R64[0], c->R64[1], c->R64[2]};
                 const float4* udf = (mixed && (flags & OVL_PASS2_DF)) ? c->Udf : nullptr;
-                lr = ovl::launch_pass2_persistent(c->U64, udf, rr, c->y64, ks, c->alpha, c->beta, c->gamma, c->cvec,
+                lr = ovl::launch_pass2_persistent(c->U64, c->nbr, udf, rr, c->y64, ks, c->alpha, c->beta, c->gamma, c->cvec,
                                                   c->H, c->kcap, mu, kappa, c->bar, &ks->timeout, g, c->num_sms,
                                                   st);
             });

@@ -733,6 +733,12 @@ extern "C" int ovl_sign_grad(ovl_ctx* c, int k, double mu, double kappa, const v
         }
         ovl::launch_native_f32_to_f64(V32, V, g, k, st);
         ovl::launch_native_f32_to_f64(W32, W, g, k, st);
+    } else if (ovl::l2_f64_ok(g, c->num_sms)) {
+        OVL_CUDA_TRY(c, cudaMemsetAsync(c->bar, 0, 64, st));
+        double2 *vv[3] = {V, nullptr, nullptr}, *ww[3] = {W, nullptr, nullptr};
+        if (ovl::launch_l2_f64(c->U64, c->nbr, vv, n, ww, n, ks, c->alpha, c->beta, c->gamma, c->vscale, mu, kappa, k,
+                               part, c->bar, g, c->num_sms, st))
+            return fail(c, OVL_ECUDA, "persistent FP64 process launch");
     } else {
         for (int i = 0; i < k; ++i) {
             const double2* vi = V + (size_t)i * n;

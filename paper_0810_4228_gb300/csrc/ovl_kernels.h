@@ -157,10 +157,27 @@ int launch_pass1_persistent(const float4* U12, float4* const v[3], float4* const
 // coef_work: 4 (kmax + 1) double2 of scratch for the per-step regeneration coefficients.
 // Udf non-null: double-float arithmetic (links Udf; v[] are converted to double-float in place, so
 // v[0] must hold the FP64 start vector and all three are left in double-float); else FP64 (links U64).
-int launch_pass2_persistent(const double2* U64, const float4* Udf, double2* const v[3], double2* y, const KState* ks,
+int launch_pass2_persistent(const double2* U64, const int* nbr, const float4* Udf, double2* const v[3], double2* y,
+                            const KState* ks,
                             const double2* alpha, const double2* beta, const double2* gamma, const double2* c,
                             double2* coef_work, int kmax, double mu, double kappa, unsigned int* bar, int* err,
                             const Geom& g, int num_sms, cudaStream_t st);
+
+// ---- persistent64.cu
+// The FP64 two-sided Lanczos process in one cooperative launch, on lattices whose own-site state fits the
+// SMs' shared memory (l2_f64_ok).  v, w: rings of three vectors, or the first vector of a stored basis
+// (v[0], w[0]) with vstep, wstep complex elements between vectors.  partials: 8 x num_sms doubles; bar:
+// arrival counter, zero at launch.  Scales of the stored vectors to vscale (may be null).
+bool l2_f64_ok(const Geom& g, int num_sms);
+int launch_l2_f64(const double2* U64, const int* nbr, double2* const v[3], size_t vstep, double2* const w[3],
+                  size_t wstep, KState* ks, double2* alpha, double2* beta, double2* gamma, double2* vscale, double mu,
+                  double kappa, int k, double* partials, unsigned int* bar, const Geom& g, int num_sms,
+                  cudaStream_t st);
+// The FP64 regeneration pass in one cooperative launch (lattices of persistent_ok); coef: per step
+// 1 / beta_i, alpha_i / beta_i, gamma_{i-1} / beta_i, c_{i+1}
+int launch_regen_f64(const double2* U64, const int* nbr, double2* const v[3], double2* y, const KState* ks,
+                     const double2* coef, double mu, double kappa, unsigned int* bar, int* err, const Geom& g,
+                     int num_sms, cudaStream_t st);
 
 // ---- inner_sign.cu
 // c[0..n) = nR * sgn(H) e_1 for the upper Hessenberg H (column-major, leading dimension ldH) of

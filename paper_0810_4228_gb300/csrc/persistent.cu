@@ -18,7 +18,8 @@
 // scalars are FP64 and formed by a single warp -- GB300's FP64 pipe is narrow,
 // so scalar algebra repeated by every warp would cost more than the stencil.  Every block adds the per-block partials
 // in the same fixed order, so all blocks hold bit-identical coefficients.
-// Pass 2 regenerates the basis in FP64 with one barrier per step.  The barriers
+// Pass 2 regenerates the basis with one barrier per step: in double-float here, in FP64 (the default) in
+// persistent64.cu.  The barriers
 // count arrivals on a counter zeroed before each launch.
 #include <algorithm>
 
@@ -459,7 +460,7 @@ template <class R> struct P2Args {
     int ntiles;
 };
 
-// FP64 (R = double) or double-float (R = df) pass-2 state: slots 0/1 alternate as v_i and v_{i-1},
+// pass-2 state (R = df): slots 0/1 alternate as v_i and v_{i-1},
 // slot 2 accumulates y
 __device__ __forceinline__ int st2_idx(int jt, int slot, int site, int q) { return ((jt * 3 + slot) * PT + site) * 12 + q; }
 
@@ -643,7 +644,8 @@ static int launch_p2(P2Args<R> a, HopCoef<R> hc, int G, int tpb, cudaStream_t st
     return (int)cudaLaunchKernelEx(&cfg, k_pass2_persistent<R, LF>, a);
 }
 
-int launch_pass2_persistent(const double2* U64, const float4* Udf, double2* const v[3], double2* y, const KState* ks,
+int launch_pass2_persistent(const double2* U64, const int* nbr, const float4* Udf, double2* const v[3], double2* y,
+                            const KState* ks,
                             const double2* alpha, const double2* beta, const double2* gamma, const double2* c,
                             double2* coef_work, int kmax, double mu, double kappa, unsigned int* bar, int* err,
                             const Geom& g, int num_sms, cudaStream_t st) {
@@ -674,9 +676,7 @@ int launch_pass2_persistent(const double2* U64, const float4* Udf, double2* cons
     k_pass2_coef<double2><<<(kmax + 127) / 128, 128, 0, st>>>(ks, alpha, beta, gamma, c,
                                                                reinterpret_cast<RegenCoef<double2>*>(coef_work), kmax,
                                                                bar);
-    P2Args<double> a;
-    fill(a);
-    return launch_p2<double, LINK_F64>(a, make_coef<double>(mu, kappa), G, tpb, st);
+    return launch_regen_f64(U64, nbr, v, y, ks, coef_work, mu, kappa, bar, err, g, num_sms, st);
 }
 
 }  // namespace ovl
