@@ -736,10 +736,14 @@ int ovl_apply_Dw(ovl_ctx* c, double mu, double kappa, const void* x, void* y, in
         xin = c->stage_in;
     }
     const int vprec = prec == 0 ? 0 : 1;
-    ovl::launch_pack_spinor(xin, c->nat_a, vprec, c->g, c->st);
-    ovl::launch_dslash(U, prec, c->nat_a, c->nat_b, m, kappa, g5, c->g, c->st);
     double2* yout = (flags & OVL_HOST) ? c->stage_out : (double2*)y;
-    ovl::launch_unpack_spinor(c->nat_b, vprec, yout, nullptr, 0, c->g, c->st);
+    if (prec == 0 && !(flags & (OVL_STENCIL_SITE | OVL_STENCIL_SPLIT))) {  // straight on canonical vectors
+        ovl::launch_dslash_canon(c->U64, xin, yout, m, kappa, g5, c->g, c->st);
+    } else {
+        ovl::launch_pack_spinor(xin, c->nat_a, vprec, c->g, c->st);
+        ovl::launch_dslash(U, prec, c->nat_a, c->nat_b, m, kappa, g5, c->g, c->st);
+        ovl::launch_unpack_spinor(c->nat_b, vprec, yout, nullptr, 0, c->g, c->st);
+    }
     CUDA_TRY(c, cudaGetLastError());
     if (flags & OVL_HOST) {
         CUDA_TRY(c, cudaMemcpyAsync(y, c->stage_out, cb, cudaMemcpyDeviceToHost, c->st));

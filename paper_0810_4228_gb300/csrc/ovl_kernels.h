@@ -47,6 +47,9 @@ void launch_unpack_spinor(const void* native, int prec, double2* canon, const do
 // skipped when ks is given and the solve is finished.
 void launch_dslash(const void* U, int prec, const void* x, void* y, double mu, double kappa, int gamma5,
                    const Geom& g, cudaStream_t st, const KState* ks = nullptr);
+// the FP64 application on canonical vectors (no conversion to the device layout)
+void launch_dslash_canon(const double2* U64, const double2* x, double2* y, double mu, double kappa, int gamma5,
+                         const Geom& g, cudaStream_t st);
 // pair: t = sv * A v~, s = sw * A^dag w~, alpha[step] = w^dag t (fused grid reduction),
 // kused = step + 1, done after step klast.
 void launch_dslash_pair(const void* U, int prec, const void* v, const void* w, void* t, void* s,

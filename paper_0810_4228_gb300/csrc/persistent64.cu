@@ -13,8 +13,7 @@
 // hop of a lane is a runtime value: address offsets and sign-bit masks select the spin projection, the
 // adjoint and the phase, so every lane runs the same instructions and none of them is an FP64 negation.
 // The half spinors meet in the warp's own shared memory (no block barrier); then the same lanes take
-// (spin, real or imaginary part) and sum the eight hops with the hop coefficient folded into the fused
-// multiply-adds: 84 + 24 FP64 instructions per lane and unit instead of 120 + 36.  Units go round-robin
+// (spin, real or imaginary part) and sum the eight hops, signs and e^{+-mu} in the fused multiply-adds: 84 + 24 FP64 instructions per lane and unit instead of 120 + 36.  Units go round-robin
 // to the blocks and then to their warps, one block per SM.  Own-site vectors stay in shared memory;
 // neighbours are read through L2 (.cg), as other blocks write them.
 //
@@ -28,7 +27,7 @@
 // of the busiest SM quarter is busy 11); regeneration on 8^4 15.5 -> 12.0 us per step (FP64 pipe 8.5).
 #include <algorithm>
 
-#include "stencil_impl.cuh"
+#include "hop64.cuh"
 
 namespace ovl {
 namespace {
@@ -36,86 +35,6 @@ namespace {
 constexpr int LW = 16;             // warps per block
 constexpr int LT = 32 * LW;
 constexpr long long LSPIN = 20000000;  // polls before a barrier wait gives up (sets ks->timeout)
-
-// chunk stride of a warp's half spinors: four groups (sites, or sites x inputs) of eight hops at a stride of
-// nine slots, plus one, so that the epilogue's lanes fall into different banks
-constexpr int HP_ST = 4 * 9 + 1;
-
-// x with its sign bit flipped by mask (0 or 0x80000000): an integer operation (FP64 negation of a value
-// that is not an operand of arithmetic runs on the FP64 pipe)
-__device__ __forceinline__ double flip(double x, unsigned mask) {
-    return __hiloint2double(__double2hiint(x) ^ (int)mask, __double2loint(x));
-}
-constexpr unsigned SIGN = 0x80000000u;
-
-// Hop h (direction h & 3, forward for h < 4) of one site from x: U (or U^dag) times the projected half
-// spinor, without the hop coefficient; both spin rows (RS = 1: o[0..2] row 0, o[3..5] row 1) or row `row`
-// (RS = 2: o[0..2]); ne: neighbour table entry.
-template <int RS>
-__device__ __forceinline__ void hop_lane(int h, int row, int site, int ne, size_t V, const double2* __restrict__ U,
-                                         const double2* x, cx<double> (&o)[6 / RS]) {
-    const int nu = h & 3;
-    const bool fwd = h < 4;
-    const int nb = ne < 0 ? ~ne : ne;
-    const double2* xb = x + nb;
-    const double2* ub = U + (size_t)nu * 9 * V + (fwd ? site : nb);
-    const bool im = (nu & 1) == 0;
-    cx<double> hh[2 / RS][3];
-#pragma unroll
-    for (int r = 0; r < 2 / RS; ++r) {
-        const int rw = RS == 2 ? row : r;
-        // row 0 takes spins 0 and 2 (nu >= 2) or 3, row 1 spins 1 and 3 or 2
-        const double2* pb = xb + (size_t)(3 * rw) * V;
-        const double2* qb = xb + (size_t)((nu >= 2) == (rw == 0) ? 6 : 9) * V;
-        const bool neg = rw == 0 ? ((nu == 3) ? !fwd : fwd) : ((nu == 0) ? fwd : !fwd);
-        const double s = neg ? -1.0 : 1.0, sr = neg != im ? -1.0 : 1.0;
-#pragma unroll
-        for (int a = 0; a < 3; ++a) {
-            const double2 p = __ldcg(pb + a * V), q = __ldcg(qb + a * V);
-            hh[r][a] = mk(fma(sr, im ? q.y : q.x, p.x), fma(s, im ? q.x : q.y, p.y));
-        }
-    }
-    const size_t srow = fwd ? 3 * V : V, scol = fwd ? V : 3 * V;
-    const unsigned pm = ne < 0 ? SIGN : 0u, cm = fwd ? pm : pm ^ SIGN;  // antiperiodic phase, conjugate
-#pragma unroll
-    for (int a = 0; a < 3; ++a) {
-#pragma unroll
-        for (int k = 0; k < 3; ++k) {
-            const double2 v = __ldg(ub + a * srow + k * scol);
-            const cx<double> u = mk(flip(v.x, pm), flip(v.y, cm));
-#pragma unroll
-            for (int r = 0; r < 2 / RS; ++r) {
-                if (k == 0) o[3 * r + a] = u * hh[r][0];
-                else cfma(o[3 * r + a], u, hh[r][k]);
-            }
-        }
-    }
-}
-
-// What the lane of (spin sp, part: 0 real, 1 imaginary) takes from hop w: slot of its half-spinor chunk
-// (colour 0) and the signed coefficient, gamma5 included.
-__device__ __forceinline__ void epilogue_lane(int sp, int part, const HopCoef<double>& hc, int (&off)[8],
-                                              double (&cw)[8]) {
-#pragma unroll
-    for (int w = 0; w < 8; ++w) {
-        const int nu = w & 3;
-        const bool fwd = w < 4, hi2 = nu >= 2, im = (nu & 1) == 0;
-        int row = sp, pp = part;
-        double c = fwd ? hc.f[nu] : hc.b[nu];
-        if (sp >= 2) {
-            row = hi2 ? sp - 2 : 3 - sp;
-            const bool nA = !fwd, nB = (nu == 0 || nu == 3) ? !fwd : fwd;
-            if (sp == 2 ? nA : nB) c = -c;
-            if (im) {
-                if (part == 0) c = -c;
-                pp = 1 - part;
-            }
-            c = -c;  // gamma5
-        }
-        off[w] = (row * 3 * HP_ST + w) * 2 + pp;
-        cw[w] = c;
-    }
-}
 
 // Sums over the lanes of one input (lane bit NB = 8 RS): v0 and v1 each, valid in the lane of that input
 // whose lower bits are 0 (v0) or 4 (v1).  First step: the lane bit above or below NB.
@@ -186,7 +105,7 @@ struct L2Args {
     double* partA;        // [G][4]
     double* partC;        // [G][4]
     unsigned int* bar;
-    HopCoef<double> hv, hw;
+    double kappa, emu, emum;
     int V, k, npass;
 };
 
@@ -223,9 +142,10 @@ __global__ void __launch_bounds__(LT) k_l2_f64(L2Args a) {
     const int nw = min(LW, (nunits - (int)blockIdx.x + G - 1) / G);
     int off[8];
     double cw[8];
-    epilogue_lane(sp, part, n ? a.hw : a.hv, off, cw);
+    epilogue_lane(sp, part, n ? a.emum : a.emu, n ? a.emu : a.emum, off, cw);  // A^dag = gamma5 D_w(-mu)
     const int grp = (sub * 2 + n) * 9;
     const unsigned g5 = sp >= 2 ? SIGN : 0u, pneg = part ? 0u : SIGN;
+    const double mk_ = flip(a.kappa, g5 ^ SIGN);
     int* err = &ks->timeout;
     for (int p = 0; p < a.npass; ++p) {
         const int u = blockIdx.x + G * (wid + LW * p);
@@ -263,7 +183,9 @@ __global__ void __launch_bounds__(LT) k_l2_f64(L2Args a) {
                 if (u >= nunits) break;  // uniform over the warp
                 const int site = SPW * u + sub;
                 cx<double> o[6 / RS];
-                hop_lane<RS>(hop, half, site, __ldg(a.nbr + hop * V + site), V, a.U, x, o);
+                const int ne = __ldg(a.nbr + hop * V + site), nb = ne < 0 ? ~ne : ne;
+                hop_lane<RS, true>(hop, half, x + nb, V, a.U + (size_t)(hop & 3) * 9 * V + (hop < 4 ? site : nb), V,
+                                   ne < 0, o);
 #pragma unroll
                 for (int c = 0; c < 6 / RS; ++c) hp[(c + 3 * half) * HP_ST + grp + hop] = c2d(o[c]);
                 __syncwarp();
@@ -272,9 +194,7 @@ __global__ void __launch_bounds__(LT) k_l2_f64(L2Args a) {
 #pragma unroll
                 for (int c = 0; c < NC; ++c) {
                     const int col = RS == 1 ? c : min(col0 + c, 2);
-                    z[c] = flip(*slot(p, cur, c), g5);
-#pragma unroll
-                    for (int w = 0; w < 8; ++w) z[c] = fma(cw[w], hd[off[w] + 2 * col * HP_ST], z[c]);
+                    z[c] = fma(mk_, hop_sum(hd + 2 * col * HP_ST, off, cw), flip(*slot(p, cur, c), g5));
                 }
 #pragma unroll
                 for (int c = 0; c < NC; ++c) {
@@ -437,7 +357,7 @@ struct R64Args {
     const double2* cf;  // [k][4]
     unsigned int* bar;
     int* err;
-    HopCoef<double> hc;
+    double kappa, emu, emum;
     int V, npass;
 };
 
@@ -458,9 +378,10 @@ __global__ void __launch_bounds__(LT) k_regen_f64(R64Args a) {
     const int G = gridDim.x, nunits = (a.V + SPW - 1) / SPW;
     int off[8];
     double cw[8];
-    epilogue_lane(sp, part, a.hc, off, cw);
+    epilogue_lane(sp, part, a.emu, a.emum, off, cw);
     const int grp = sub * 9;
     const unsigned g5 = sp >= 2 ? SIGN : 0u, pneg = part ? 0u : SIGN;
+    const double mk_ = flip(a.kappa, g5 ^ SIGN);
     const int po = part ? -1 : 1;
     for (int p = 0; p < a.npass; ++p) {
         const int site = SPW * (blockIdx.x + G * (wid + LW * p)) + sub;
@@ -489,7 +410,9 @@ __global__ void __launch_bounds__(LT) k_regen_f64(R64Args a) {
             const bool ok = SPW * u + sub < a.V;
             const int site = ok ? SPW * u + sub : a.V - 1;
             cx<double> o[6 / RS];
-            hop_lane<RS>(hop, half, site, __ldg(a.nbr + hop * V + site), V, a.U, x, o);
+            const int ne = __ldg(a.nbr + hop * V + site), nb = ne < 0 ? ~ne : ne;
+            hop_lane<RS, true>(hop, half, x + nb, V, a.U + (size_t)(hop & 3) * 9 * V + (hop < 4 ? site : nb), V, ne < 0,
+                               o);
 #pragma unroll
             for (int c = 0; c < 6 / RS; ++c) hp[(c + 3 * half) * HP_ST + grp + hop] = c2d(o[c]);
             __syncwarp();
@@ -499,9 +422,7 @@ __global__ void __launch_bounds__(LT) k_regen_f64(R64Args a) {
             for (int c = 0; c < NC; ++c) {
                 const int col = RS == 1 ? c : min(col0 + c, 2);
                 const double self = *slot(p, cur, c);
-                z[c] = flip(self, g5);
-#pragma unroll
-                for (int w = 0; w < 8; ++w) z[c] = fma(cw[w], hd[off[w] + 2 * col * HP_ST], z[c]);
+                z[c] = fma(mk_, hop_sum(hd + 2 * col * HP_ST, off, cw), flip(self, g5));
                 z[c] = fma(car, self, ib * z[c]);
                 z[c] = fma(cai, slot(p, cur, c)[po], z[c]);
                 z[c] = fma(cgr, *slot(p, prv, c), z[c]);
@@ -595,8 +516,7 @@ int launch_l2_f64(const double2* U64, const int* nbr, double2* const v[3], size_
     a.partA = partials;
     a.partC = partials + 4 * (size_t)sp.G;
     a.bar = bar;
-    a.hv = make_coef<double>(mu, kappa);
-    a.hw = make_coef<double>(-mu, kappa);
+    a.kappa = kappa, a.emu = exp(mu), a.emum = exp(-mu);
     a.V = g.V, a.k = k, a.npass = sp.npass;
     static unsigned long long dev1 = 0, dev2 = 0;
     return sp.rs == 1 ? launch_coop(k_l2_f64<1>, a, sp, dev1, st) : launch_coop(k_l2_f64<2>, a, sp, dev2, st);
@@ -616,7 +536,7 @@ int launch_regen_f64(const double2* U64, const int* nbr, double2* const v[3], do
     a.cf = coef;
     a.bar = bar;
     a.err = err;
-    a.hc = make_coef<double>(mu, kappa);
+    a.kappa = kappa, a.emu = exp(mu), a.emum = exp(-mu);
     a.V = g.V, a.npass = sp.npass;
     static unsigned long long dev1 = 0, dev2 = 0;
     return sp.rs == 1 ? launch_coop(k_regen_f64<1>, a, sp, dev1, st) : launch_coop(k_regen_f64<2>, a, sp, dev2, st);

@@ -18,6 +18,7 @@
 #include <algorithm>
 #include <type_traits>
 
+#include "hop64.cuh"
 #include "stencil_impl.cuh"
 
 namespace ovl {
@@ -273,6 +274,99 @@ __global__ void __launch_bounds__(128, MINB) k_dslash(const void* __restrict__ U
     store_spinor(y, g.V, i, acc[0]);
 }
 
+// FP64 application with a site shared by eight lanes (RS = 1) or sixteen (RS = 2): see hop64.cuh.  CANON:
+// x and y in the canonical layout ([site][12], sites in canonical order), otherwise the device layout.
+// A warp takes 4 / RS consecutive sites; the half spinors meet in its own shared memory.  Bound by the FP64
+// pipe: 108 FP64 instructions per four sites (RS = 1) at 19 cycles each and SM.  Measured against one thread
+// per site (large lattices) and per site and direction (small ones), device layout: 4^4 15.0 -> 6.7 us,
+// 8^4 14.9 -> 13.8, 12^4 57.6 -> 45.4, 24^4 695 -> 617, 32^4 2080 -> 1930.  Canonical vectors, which went
+// through the device layout (three launches): 4^4 22.9 -> 6.9 us, 24^4 776 -> 617.
+template <int RS, bool CANON>
+__global__ void __launch_bounds__(128) k_dslash_hl(const double2* __restrict__ U, const double2* __restrict__ x,
+                                                   double2* __restrict__ y, double kappa, double emu, double emum,
+                                                   int g5, const KState* ks, Geom g) {
+    constexpr int SPW = 4 / RS;
+    __shared__ __align__(16) double2 hps[4][6 * HP_ST];
+    if (ks && (ks->done || ks->status)) return;
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    const int hop = lane & 7, half = RS == 2 ? (lane >> 3) & 1 : 0, sub = lane / (8 * RS);
+    const int s0 = (blockIdx.x * 4 + wid) * SPW + sub;
+    if (s0 - sub >= g.V) return;  // the warp's first site (uniform over the warp)
+    const bool ok = s0 < g.V;
+    const int s = ok ? s0 : g.V - 1;
+    const size_t V = (size_t)g.V;
+    int c[4];
+    if (CANON) {
+        int r = s;
+        c[3] = r % g.L[3];
+        r /= g.L[3];
+        c[2] = r % g.L[2];
+        r /= g.L[2];
+        c[1] = r % g.L[1];
+        c[0] = r / g.L[1];
+    } else {
+        const Coord cc = site_coord(g, s);
+#pragma unroll
+        for (int d = 0; d < 4; ++d) c[d] = cc.x[d];
+    }
+    const int nu = hop & 3;
+    const bool fwd = hop < 4;
+    const bool edge = nu == 3 && g.bc_t < 0 && (fwd ? c[3] == g.L[3] - 1 : c[3] == 0);
+    int nc[4];
+#pragma unroll
+    for (int d = 0; d < 4; ++d) {
+        int v = c[d];
+        if (d == nu) {
+            v += fwd ? 1 : -1;
+            if (v == g.L[d]) v = 0;
+            if (v < 0) v = g.L[d] - 1;
+        }
+        nc[d] = v;
+    }
+    const int ni = internal_index(g, nc);
+    const int li = fwd ? (CANON ? internal_index(g, c) : s) : ni;  // the link's site
+    const double2* xb = CANON ? x + (size_t)canon_index(g, nc) * 12 : x + ni;
+    cx<double> o[6 / RS];
+    hop_lane<RS, false>(hop, half, xb, CANON ? 1 : V, U + (size_t)nu * 9 * V + li, V, edge, o);
+    double2* hp = hps[wid];
+#pragma unroll
+    for (int q = 0; q < 6 / RS; ++q) hp[(q + 3 * half) * HP_ST + sub * 9 + hop] = c2d(o[q]);
+    const int sp = hop >> 1, part = hop & 1;
+    int off[8];
+    double cw[8];
+    epilogue_lane(sp, part, emu, emum, off, cw);
+    const unsigned sg = sp >= 2 && g5 ? SIGN : 0u;
+    const double mk_ = flip(kappa, sg ^ SIGN);
+    __syncwarp();
+    const double* hd = reinterpret_cast<const double*>(hp + sub * 9);
+    const double* xd = reinterpret_cast<const double*>(x);
+    double* yd = reinterpret_cast<double*>(y);
+#pragma unroll
+    for (int q = 0; q < (RS == 1 ? 3 : 2); ++q) {
+        const int col = RS == 1 ? q : (half ? 2 : q);
+        if (RS == 2 && half && q) break;
+        const size_t e = CANON ? ((size_t)s * 12 + 3 * sp + col) * 2 + part : ((3 * sp + col) * V + s) * 2 + part;
+        const double z = fma(mk_, hop_sum(hd + 2 * col * HP_ST, off, cw), flip(__ldg(xd + e), sg));
+        if (ok) yd[e] = z;
+    }
+}
+
+template <bool CANON>
+static void launch_hl(const double2* U, const double2* x, double2* y, double mu, double kappa, int gamma5,
+                      const Geom& g, cudaStream_t st, const KState* ks) {
+    const double ef = exp(mu), eb = exp(-mu);
+    // a row of a hop per lane while that leaves at most one unit per SM quarter (4 x 152)
+    if (g.V <= 2 * 608)
+        k_dslash_hl<2, CANON><<<(g.V + 7) / 8, 128, 0, st>>>(U, x, y, kappa, ef, eb, gamma5, ks, g);
+    else
+        k_dslash_hl<1, CANON><<<(g.V + 15) / 16, 128, 0, st>>>(U, x, y, kappa, ef, eb, gamma5, ks, g);
+}
+
+void launch_dslash_canon(const double2* U, const double2* x, double2* y, double mu, double kappa, int gamma5,
+                         const Geom& g, cudaStream_t st) {
+    launch_hl<true>(U, x, y, mu, kappa, gamma5, g, st, nullptr);
+}
+
 // blocks per SM of the FP32 single stencil (128 threads each): 6 measured best on GB300 (48^3 x 64:
 // 8 gave 4571 -> 3966 GB/s with 12-real links)
 #ifndef OVL_DSLASH_F32_MINB
@@ -285,6 +379,10 @@ static bool pick_ds(const Geom& g) { return g_ds_mode < 0 ? use_ds(g) : g_ds_mod
 
 void launch_dslash(const void* U, int prec, const void* x, void* y, double mu, double kappa, int gamma5,
                    const Geom& g, cudaStream_t st, const KState* ks) {
+    if (prec == 0 && g_ds_mode < 0) {
+        launch_hl<false>((const double2*)U, (const double2*)x, (double2*)y, mu, kappa, gamma5, g, st, ks);
+        return;
+    }
     if (pick_ds(g)) {
         if (prec == 0)
             k_dslash_ds<LINK_F64><<<ds_grid(g), 128, ds_smem(16, 1), st>>>(U, (const double2*)x, (double2*)y,
