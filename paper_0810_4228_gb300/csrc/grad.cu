@@ -11,140 +11,77 @@
 //        (1 otherwise), ph the antiperiodic phase of a hop across the time edge;
 //   dl/dmu        = Re <g, (dA/dmu) x>,  dA/dmu = -kappa gamma5 (e^mu T_4^+ - e^-mu T_4^-).
 // Every link receives the forward hop of its own site and the backward hop of
-// the site it points to.  One thread per site, canonical layouts in and out.
+// the site it points to.  Canonical layouts in and out.
+#include <cmath>
+
 #include "ctx.h"
-#include "stencil_impl.cuh"
+#include "force.cuh"
 
 namespace ovl {
 namespace {
 
-// canonical spinor access: psi[s][12]
-__device__ __forceinline__ void load_canon(const double2* __restrict__ p, int s, Spinor<double>& o) {
+// One link per thread, a warp per direction (32 consecutive sites of each of the four directions per block;
+// the direction of a warp rotates with the block, so that the temporal links' extra work spreads over the
+// SM quarters).  R = float: the spatial links in FP32 (OVL_F32); the temporal ones, whose forces also give
+// d/dmu, stay FP64.  Bound by the FP64 pipe: 192 operations per link (force.cuh) and 54 for d/dmu; 24^4:
+// 1490 -> 571 us against one thread per site with four-spin products and the temporal hops applied again.
+template <class R, int NU>
+__device__ __forceinline__ void link_grad(const double2* gx, const double2* gy, const double2* px, const double2* py,
+                                          double2* o, double kappa, double ph) {
+    cx<R> z[9];
 #pragma unroll
-    for (int q = 0; q < 12; ++q) {
-        const double2 v = p[(size_t)s * 12 + q];
-        o.s[q / 3][q % 3] = mk(v.x, v.y);
-    }
-}
-
-// (1 + S gamma_nu) gamma5 g as a full spinor
-template <int NU, int S, class R>
-__device__ __forceinline__ void proj_g5(const Spinor<R>& g, Spinor<R>& o) {
-    Spinor<R> g5 = g;
+    for (int e = 0; e < 9; ++e) z[e] = mk(R(0), R(0));
+    half_force<R, NU>(gx, gy, px, py, 1, z, z);
+    const R f = -(R)kappa * (R)ph;
 #pragma unroll
-    for (int a = 0; a < 3; ++a) {
-        g5.s[2][a] = -g.s[2][a];
-        g5.s[3][a] = -g.s[3][a];
-    }
-    Half<R> h;
-    project<NU, S>(g5, h);
-#pragma unroll
-    for (int sp = 0; sp < 4; ++sp)
-#pragma unroll
-        for (int a = 0; a < 3; ++a) o.s[sp][a] = mk(R(0), R(0));
-    recon_acc<NU, S>(o, h, R(1));
-}
-
-// canonical spinor in precision R
-template <class R>
-__device__ __forceinline__ void load_canon_r(const double2* __restrict__ p, int s, Spinor<R>& o) {
-#pragma unroll
-    for (int q = 0; q < 12; ++q) {
-        const double2 v = p[(size_t)s * 12 + q];
-        o.s[q / 3][q % 3] = mk((R)v.x, (R)v.y);
-    }
-}
-
-// (R = float: the FP32 form of OVL_F32, every product and sum in FP32)
-template <int NU, class R>
-__device__ __forceinline__ void link_grad(const Geom& g, const Coord& c, int s, const double2* __restrict__ x,
-                                          const double2* __restrict__ gr, double2* __restrict__ gU, double cf,
-                                          double cb) {
-    int y[4] = {c.x[0], c.x[1], c.x[2], c.x[3]};
-    y[NU] = (y[NU] + 1) % g.L[NU];
-    const int sf = canon_index(g, y);
-    const R ph = (NU == 3 && c.x[3] == g.L[3] - 1) ? (R)g.bc_t : R(1);
-    Spinor<R> gx, gy, px, py, gt, gh;
-    load_canon_r(gr, s, gx);
-    load_canon_r(gr, sf, gy);
-    load_canon_r(x, s, px);
-    load_canon_r(x, sf, py);
-    proj_g5<NU, +1>(gx, gt);
-    proj_g5<NU, -1>(gy, gh);
-    const R af = -(R)cf * ph, ab = -(R)cb * ph;
-#pragma unroll
-    for (int i = 0; i < 3; ++i)
-#pragma unroll
-        for (int j = 0; j < 3; ++j) {
-            cx<R> z = mk(R(0), R(0));
-#pragma unroll
-            for (int sp = 0; sp < 4; ++sp) {
-                z = z + af * cdot(py.s[sp][j], gt.s[sp][i]);  // g~_i conj(psi(x+nu)_j)
-                z = z + ab * cdot(gh.s[sp][j], px.s[sp][i]);  // psi(x)_i conj(g^_j)
-            }
-            gU[((size_t)s * 4 + NU) * 9 + 3 * i + j] = make_double2((double)z.r, (double)z.i);
-        }
+    for (int e = 0; e < 9; ++e) o[e] = make_double2((double)(f * z[e].r), (double)(f * z[e].i));
 }
 
 template <class R>
-__global__ void __launch_bounds__(128) k_dw_grad(const double2* __restrict__ U, const double2* __restrict__ x,
+__global__ void __launch_bounds__(128, 4) k_dw_grad(const double2* __restrict__ U, const double2* __restrict__ x,
                                                  const double2* __restrict__ gr, double2* __restrict__ gU,
-                                                 double kappa, double mu, Geom g, double* partials,
+                                                 double kappa, double emu, double emum, Geom g, double* partials,
                                                  unsigned int* counter, double* gmu) {
     __shared__ double red[32];
-    const int s = blockIdx.x * blockDim.x + threadIdx.x;
+    const int nu = ((threadIdx.x >> 5) + blockIdx.x) & 3;
+    const int s = blockIdx.x * 32 + (threadIdx.x & 31);
     double part[1] = {0.0};
-    if (s < g.V) {
-        Coord c;
-        {
-            int r = s;
-            c.x[3] = r % g.L[3];
-            r /= g.L[3];
-            c.x[2] = r % g.L[2];
-            r /= g.L[2];
-            c.x[1] = r % g.L[1];
-            c.x[0] = r / g.L[1];
-            c.par = (c.x[0] + c.x[1] + c.x[2] + c.x[3]) & 1;
-        }
-        if (gU) {
-            link_grad<0, R>(g, c, s, x, gr, gU, kappa, kappa);
-            link_grad<1, R>(g, c, s, x, gr, gU, kappa, kappa);
-            link_grad<2, R>(g, c, s, x, gr, gU, kappa, kappa);
-            link_grad<3, R>(g, c, s, x, gr, gU, kappa * exp(mu), kappa * exp(-mu));
-        }
-        // Re <g, dA/dmu x> at this site: the temporal hops with e^mu and -e^-mu
-        const int i = internal_index(g, c.x);
-        Spinor<double> acc, xs;
+    if (s < g.V && (gU || nu == 3)) {
+        int c[4], r = s;
+        c[3] = r % g.L[3];
+        r /= g.L[3];
+        c[2] = r % g.L[2];
+        r /= g.L[2];
+        c[1] = r % g.L[1];
+        c[0] = r / g.L[1];
+        int y[4];
 #pragma unroll
-        for (int sp = 0; sp < 4; ++sp)
+        for (int d = 0; d < 4; ++d) y[d] = d == nu ? (c[d] + 1 == g.L[d] ? 0 : c[d] + 1) : c[d];
+        const size_t i = (size_t)s * 12, f = (size_t)canon_index(g, y) * 12;
+        const double2 *gx = gr + i, *gy = gr + f, *px = x + i, *py = x + f;
+        double2* o = gU + ((size_t)s * 4 + nu) * 9;
+        switch (nu) {  // uniform per warp
+            case 0: link_grad<R, 0>(gx, gy, px, py, o, kappa, 1.0); break;
+            case 1: link_grad<R, 1>(gx, gy, px, py, o, kappa, 1.0); break;
+            case 2: link_grad<R, 2>(gx, gy, px, py, o, kappa, 1.0); break;
+            default: {
+                cx<double> zf[9], zb[9];
 #pragma unroll
-            for (int a = 0; a < 3; ++a) acc.s[sp][a] = mk(0.0, 0.0);
-        Link<double> L;
-        Spinor<double> p;
-        Half<double> h, uh;
-        int y[4] = {c.x[0], c.x[1], c.x[2], c.x[3]};
-        y[3] = (c.x[3] + 1) % g.L[3];
-        load_canon(x, canon_index(g, y), p);
-        const double phf = (c.x[3] == g.L[3] - 1) ? (double)g.bc_t : 1.0;
-        load_link(U, g.V, 3, i, L);
-        project<3, +1>(p, h);
-        mul_link(L, h, uh);
-        recon_acc<3, +1>(acc, uh, -kappa * exp(mu) * phf);
-        y[3] = (c.x[3] - 1 + g.L[3]) % g.L[3];
-        load_canon(x, canon_index(g, y), p);
-        const double phb = (c.x[3] == 0) ? (double)g.bc_t : 1.0;
-        load_link(U, g.V, 3, internal_index(g, y), L);
-        project<3, -1>(p, h);
-        mul_link_dag(L, h, uh);
-        recon_acc<3, -1>(acc, uh, kappa * exp(-mu) * phb);
-        load_canon(gr, s, xs);
+                for (int e = 0; e < 9; ++e) zf[e] = zb[e] = mk(0.0, 0.0);
+                half_force<double, 3>(gx, gy, px, py, 1, zf, zb);
+                const double ph = c[3] == g.L[3] - 1 ? (double)g.bc_t : 1.0;
+                const double af = -kappa * emu * ph, ab = -kappa * emum * ph;
+                const double2* u = U + (size_t)27 * g.V + internal_index(g, c);
 #pragma unroll
-        for (int sp = 0; sp < 4; ++sp)
-#pragma unroll
-            for (int a = 0; a < 3; ++a) {
-                const cx<double> e = sp >= 2 ? -acc.s[sp][a] : acc.s[sp][a];
-                part[0] += cdot(xs.s[sp][a], e).r;
+                for (int e = 0; e < 9; ++e) {
+                    const cx<double> F = af * zf[e];
+                    if (gU) o[e] = make_double2(fma(ab, zb[e].r, F.r), fma(ab, zb[e].i, F.i));
+                    const double2 v = __ldg(u + (size_t)e * g.V);
+                    part[0] = fma(v.x, fma(-ab, zb[e].r, F.r), part[0]);
+                    part[0] = fma(v.y, fma(-ab, zb[e].i, F.i), part[0]);
+                }
             }
+        }
     }
     double out[1];
     if (grid_sum_last<1>(part, partials, counter, out, red))
@@ -165,13 +102,13 @@ extern "C" int ovl_dw_grad(ovl_ctx* c, double mu, double kappa, const void* x, c
     int r = ensure_solve(c, std::max(c->kcap, 1));
     if (r) return r;
     double* gmu = reinterpret_cast<double*>(c->h2);
-    const int T = 128, B = (c->g.V + T - 1) / T;
+    const int T = 128, B = (c->g.V + 31) / 32;
     if (flags & OVL_F32)
         ovl::k_dw_grad<float><<<B, T, 0, c->st>>>(c->U64, (const double2*)x, (const double2*)g, (double2*)grad_U,
-                                                  kappa, mu, c->g, c->partials, c->counter, gmu);
+                                                  kappa, exp(mu), exp(-mu), c->g, c->partials, c->counter, gmu);
     else
         ovl::k_dw_grad<double><<<B, T, 0, c->st>>>(c->U64, (const double2*)x, (const double2*)g, (double2*)grad_U,
-                                                   kappa, mu, c->g, c->partials, c->counter, gmu);
+                                                   kappa, exp(mu), exp(-mu), c->g, c->partials, c->counter, gmu);
     OVL_CUDA_TRY(c, cudaGetLastError());
     if (grad_mu) {
         OVL_CUDA_TRY(c, cudaMemcpyAsync(grad_mu, gmu, sizeof(double), cudaMemcpyDeviceToHost, c->st));

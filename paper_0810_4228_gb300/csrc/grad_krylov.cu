@@ -29,6 +29,7 @@
 
 #include "ctx.h"
 #include "df32.cuh"
+#include "force.cuh"
 #include "stencil_impl.cuh"
 
 namespace ovl {
@@ -324,23 +325,6 @@ __global__ void __launch_bounds__(256) k_gq_combine(const double2* __restrict__ 
 }
 
 // (1 + S gamma_nu) gamma5 x as a full spinor
-template <int NU, int S>
-__device__ __forceinline__ void proj_g5_full(const Spinor<double>& x, Spinor<double>& o) {
-    Spinor<double> g5 = x;
-#pragma unroll
-    for (int a = 0; a < 3; ++a) {
-        g5.s[2][a] = -x.s[2][a];
-        g5.s[3][a] = -x.s[3][a];
-    }
-    Half<double> h;
-    project<NU, S>(g5, h);
-#pragma unroll
-    for (int sp = 0; sp < 4; ++sp)
-#pragma unroll
-        for (int a = 0; a < 3; ++a) o.s[sp][a] = mk(0.0, 0.0);
-    recon_acc<NU, S>(o, h, 1.0);
-}
-
 template <int NU, int S, class R>
 __device__ __forceinline__ void proj_g5_full_r(const Spinor<R>& x, Spinor<R>& o) {
     Spinor<R> g5 = x;
@@ -357,37 +341,6 @@ __device__ __forceinline__ void proj_g5_full_r(const Spinor<R>& x, Spinor<R>& o)
         for (int a = 0; a < 3; ++a) o.s[sp][a] = mk(R(0), R(0));
     recon_acc<NU, S>(o, h, R(1));
 }
-
-// link force of y = gamma5 D_w(m) x for the adjoint gr of y, added into gU (device link layout):
-// gU[x, nu] += -kappa ph (cf g~ (x) conj(x(x+nu)) + cb x(x) (x) conj(g^)),
-// g~ = (1 + gamma_nu) gamma5 gr(x), g^ = (1 - gamma_nu) gamma5 gr(x + nu)
-template <int NU>
-__device__ __forceinline__ void link_force(const Geom& g, const Coord& c, int s, const double2* x,
-                                           const double2* gr, double cf, double cb, cx<double> (&z)[9]) {
-    const int f = neighbour(g, c, NU, +1);
-    const double ph = (NU == 3 && c.x[3] == g.L[3] - 1) ? (double)g.bc_t : 1.0;
-    Spinor<double> gx, gy, px, py, gt, gh;
-    load_spinor(gr, g.V, s, gx);
-    load_spinor(gr, g.V, f, gy);
-    load_spinor(x, g.V, s, px);
-    load_spinor(x, g.V, f, py);
-    proj_g5_full<NU, +1>(gx, gt);
-    proj_g5_full<NU, -1>(gy, gh);
-    const double af = -cf * ph, ab = -cb * ph;
-#pragma unroll
-    for (int i = 0; i < 3; ++i)
-#pragma unroll
-        for (int j = 0; j < 3; ++j) {
-            cx<double> w = z[3 * i + j];
-#pragma unroll
-            for (int sp = 0; sp < 4; ++sp) {
-                w = w + af * cdot(py.s[sp][j], gt.s[sp][i]);
-                w = w + ab * cdot(gh.s[sp][j], px.s[sp][i]);
-            }
-            z[3 * i + j] = w;
-        }
-}
-
 
 // Re <gr, dA/dmu x> at site s, dA/dmu = -kappa gamma5 (e^mu T_4^+ - e^-mu T_4^-)
 __device__ __forceinline__ double dmu_site(const Geom& g, const Coord& c, int s, const double2* U,
@@ -607,42 +560,84 @@ __global__ void __launch_bounds__(GT) k_force_sum_f32(const double2* __restrict_
     }
 }
 
-__global__ void __launch_bounds__(GT) k_force_sum(const double2* __restrict__ U, const double2* __restrict__ V,
-                                                  const double2* __restrict__ Z, int k, double2* __restrict__ gU,
-                                                  double kappa, double mu, Geom g, double* partials,
-                                                  unsigned int* counter, double* gmu) {
-    __shared__ double red[32];
-    const int s = blockIdx.x * blockDim.x + threadIdx.x;
-    const int nu = blockIdx.y;  // 0..3 links, 4: the mu derivative
-    const size_t n = (size_t)12 * g.V;
-    double part[1] = {0.0};
-    if (s < g.V) {
-        const Coord c = site_coord(g, s);
-        if (nu < 4) {
-            cx<double> z[9];
+// FP64 link force summed over the pairs (v~_q, Z_q): block = 32 sites, a warp per direction (rotating with
+// the block), pairs q0 .. q1 of blockIdx.y's share, so that small lattices fill the SM quarters (a warp
+// issues one FP64 instruction per 64 cycles).  6^4, 480 pairs: 8.5 -> 1.05 ms against one warp per 32 links
+// with four-spin products and the mu derivative's hops.
+// part[(split * 45 + e) * V + s]: e = 9 nu + ij for nu < 3, then forward and backward terms of nu = 3.
+__global__ void __launch_bounds__(128) k_force_part(const double2* __restrict__ V, const double2* __restrict__ Z, int k,
+                                                    double2* __restrict__ part, Geom g) {
+    const int nu = ((threadIdx.x >> 5) + blockIdx.x + blockIdx.y) & 3;
+    const int s = blockIdx.x * 32 + (threadIdx.x & 31);
+    if (s >= g.V) return;
+    const size_t n = (size_t)12 * g.V, st = g.V;
+    const int q0 = (int)((long long)k * blockIdx.y / gridDim.y), q1 = (int)((long long)k * (blockIdx.y + 1) / gridDim.y);
+    const int f = neighbour(g, site_coord(g, s), nu, +1);
+    cx<double> zf[9], zb[9];
 #pragma unroll
-            for (int q = 0; q < 9; ++q) z[q] = mk(0.0, 0.0);
-            const double cf = nu == 3 ? kappa * exp(mu) : kappa, cb = nu == 3 ? kappa * exp(-mu) : kappa;
-            for (int q = 0; q < k; ++q) {
-                const double2* x = V + (size_t)q * n;
-                const double2* gr = Z + (size_t)q * n;
-                switch (nu) {
-                    case 0: link_force<0>(g, c, s, x, gr, cf, cb, z); break;
-                    case 1: link_force<1>(g, c, s, x, gr, cf, cb, z); break;
-                    case 2: link_force<2>(g, c, s, x, gr, cf, cb, z); break;
-                    default: link_force<3>(g, c, s, x, gr, cf, cb, z); break;
-                }
-            }
-#pragma unroll
-            for (int q = 0; q < 9; ++q) gU[((size_t)nu * 9 + q) * g.V + s] = c2d(z[q]);
-        } else {
-            for (int q = 0; q < k; ++q) part[0] += dmu_site(g, c, s, U, V + (size_t)q * n, Z + (size_t)q * n, kappa, mu);
+    for (int e = 0; e < 9; ++e) zf[e] = zb[e] = mk(0.0, 0.0);
+    for (int q = q0; q < q1; ++q) {
+        const double2 *x = V + q * n, *gr = Z + q * n;
+        switch (nu) {  // uniform per warp
+            case 0: half_force<double, 0>(gr + s, gr + f, x + s, x + f, st, zf, zf); break;
+            case 1: half_force<double, 1>(gr + s, gr + f, x + s, x + f, st, zf, zf); break;
+            case 2: half_force<double, 2>(gr + s, gr + f, x + s, x + f, st, zf, zf); break;
+            default: half_force<double, 3>(gr + s, gr + f, x + s, x + f, st, zf, zb); break;
         }
     }
-    if (nu == 4) {
-        double out[1];
-        if (grid_sum_last<1>(part, partials, counter, out, red) && threadIdx.x == 0) *gmu = out[0];
+    double2* o = part + ((size_t)blockIdx.y * 45 + 9 * nu) * st + s;
+#pragma unroll
+    for (int e = 0; e < 9; ++e) {
+        o[e * st] = c2d(zf[e]);
+        if (nu == 3) o[(9 + e) * st] = c2d(zb[e]);
     }
+}
+
+// Sum of the shares (fixed order), the hop coefficients, the canonical layout; d/dmu from the temporal links'
+// terms: Re sum_ij U_ij conj(F_ij) (force.cuh).
+__global__ void __launch_bounds__(128) k_force_reduce(const double2* __restrict__ U, const double2* __restrict__ part,
+                                                      int nsplit, double2* __restrict__ gU, double kappa, double emu,
+                                                      double emum, Geom g, double* partials, unsigned int* counter,
+                                                      double* gmu) {
+    __shared__ double red[32];
+    const int nu = ((threadIdx.x >> 5) + blockIdx.x) & 3;
+    const int s = blockIdx.x * 32 + (threadIdx.x & 31);
+    const size_t st = g.V;
+    double dm[1] = {0.0};
+    if (s < g.V) {
+        const Coord c = site_coord(g, s);
+        const double ph = nu == 3 && c.x[3] == g.L[3] - 1 ? (double)g.bc_t : 1.0;
+        const double af = -kappa * (nu == 3 ? emu : 1.0) * ph, ab = -kappa * emum * ph;
+        double2* o = gU + ((size_t)canon_index(g, c.x) * 4 + nu) * 9;
+        for (int e = 0; e < 9; ++e) {
+            double2 f = make_double2(0.0, 0.0), b = f;
+            for (int q = 0; q < nsplit; ++q) {
+                const double2* p = part + ((size_t)q * 45 + 9 * nu + e) * st + s;
+                f.x += p[0].x;
+                f.y += p[0].y;
+                if (nu == 3) {
+                    b.x += p[9 * st].x;
+                    b.y += p[9 * st].y;
+                }
+            }
+            f.x *= af;
+            f.y *= af;
+            if (gU) o[e] = make_double2(fma(ab, b.x, f.x), fma(ab, b.y, f.y));
+            if (nu == 3) {
+                const double2 v = __ldg(U + ((size_t)27 + e) * st + s);
+                dm[0] = fma(v.x, fma(-ab, b.x, f.x), dm[0]);
+                dm[0] = fma(v.y, fma(-ab, b.y, f.y), dm[0]);
+            }
+        }
+    }
+    double out[1];
+    if (grid_sum_last<1>(dm, partials, counter, out, red) && threadIdx.x == 0) *gmu = out[0];
+}
+
+// shares of the pairs: three warps per SM quarter where the lattice alone does not give them
+int force_splits(const Geom& g, int k, int num_sms) {
+    const int warps = 4 * ((g.V + 31) / 32);
+    return std::max(1, std::min(std::min(16, k), (12 * num_sms + warps - 1) / warps));
 }
 
 // device link layout -> canonical [site][nu][3][3]
@@ -684,8 +679,10 @@ extern "C" int ovl_sign_grad(ovl_ctx* c, int k, double mu, double kappa, const v
     // ---- workspace: W (k + 1 vectors), Z (k vectors), g_y packed, link gradient, scalars
     const size_t kk1 = (size_t)k + 1;
     // (mixed: the FP32 bases, (k + 1) vectors of n complex64 each, after the FP64 ones)
+    // (FP64: the shares of the link force after everything else)
+    const int nsplit = mixed ? 0 : ovl::force_splits(g, k, c->num_sms);
     const size_t need = ((2 * kk1 + 1 + 3 + 1) * n + 4 * kk1 + (size_t)k * k + 64) * sizeof(double2) +
-                        (mixed ? 2 * kk1 * n * sizeof(float2) : 0);
+                        (mixed ? 2 * kk1 * n * sizeof(float2) : (size_t)nsplit * 45 * g.V * sizeof(double2));
     if (c->gwork_bytes < need) {
         if (c->gwork) cudaFree(c->gwork);
         c->gwork = nullptr;
@@ -833,9 +830,13 @@ extern "C" int ovl_sign_grad(ovl_ctx* c, int k, double mu, double kappa, const v
                                                                  gmu_acc);
         } else {
             ovl::k_gq_combine_df<<<gz, 256, 0, st>>>(W, M, Z, kk, n);
-            ovl::k_force_sum<<<dim3(B, 5), ovl::GT, 0, st>>>(c->U64, V, Z, kk, gUd, kappa, mu, g, part, cnt, gmu_acc);
+            const int B32 = (g.V + 31) / 32, nsp = std::min(nsplit, kk);
+            double2* shares = misc + 32;
+            ovl::k_force_part<<<dim3(B32, nsp), 128, 0, st>>>(V, Z, kk, shares, g);
+            ovl::k_force_reduce<<<B32, 128, 0, st>>>(c->U64, shares, nsp, (double2*)grad_U, kappa, std::exp(mu),
+                                                     std::exp(-mu), g, part, cnt, gmu_acc);
         }
-        if (grad_U) ovl::k_links_to_canon<<<B, ovl::GT, 0, st>>>(gUd, (double2*)grad_U, g);
+        if (grad_U && mixed) ovl::k_links_to_canon<<<B, ovl::GT, 0, st>>>(gUd, (double2*)grad_U, g);
     }
     if (grad_b) {
         OVL_CUDA_TRY(c, cudaMemsetAsync(tmp, 0, vb, st));

@@ -279,8 +279,8 @@ __global__ void __launch_bounds__(128, MINB) k_dslash(const void* __restrict__ U
 // A warp takes 4 / RS consecutive sites; the half spinors meet in its own shared memory.  Bound by the FP64
 // pipe: 108 FP64 instructions per four sites (RS = 1) at 19 cycles each and SM.  Measured against one thread
 // per site (large lattices) and per site and direction (small ones), device layout: 4^4 15.0 -> 6.7 us,
-// 8^4 14.9 -> 13.8, 12^4 57.6 -> 45.4, 24^4 695 -> 617, 32^4 2080 -> 1930.  Canonical vectors, which went
-// through the device layout (three launches): 4^4 22.9 -> 6.9 us, 24^4 776 -> 617.
+// 24^4 695 -> 481 us.  Canonical vectors, which went through the device layout (three launches): 4^4 22.9 ->
+// 6.2 us, 24^4 776 -> 481.
 template <int RS, bool CANON>
 __global__ void __launch_bounds__(128) k_dslash_hl(const double2* __restrict__ U, const double2* __restrict__ x,
                                                    double2* __restrict__ y, double kappa, double emu, double emum,
@@ -669,25 +669,30 @@ void launch_build_nbr(int* nbr, const Geom& g, cudaStream_t st) {
 }
 
 // ---------------------------------------------------------------- layouts --
-__global__ void k_pack_gauge(const double2* __restrict__ Uc, double2* __restrict__ U64, float4* __restrict__ U12,
-                             float2* __restrict__ U18, float4* __restrict__ Udf, Geom g) {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+// One link per thread: a block is 32 sites (device order) x 4 directions, a warp per direction, so that every
+// store is one coalesced transaction and the four warps share the sites' 576-byte canonical records in L1.
+// Bound by HBM (2208 bytes per site in and out).  24^4: 186 -> 177 us against one site per thread.
+__global__ void __launch_bounds__(128) k_pack_gauge(const double2* __restrict__ Uc, double2* __restrict__ U64,
+                                                    float4* __restrict__ U12, float2* __restrict__ U18,
+                                                    float4* __restrict__ Udf, Geom g) {
+    const int i = blockIdx.x * 32 + (threadIdx.x & 31), nu = threadIdx.x >> 5;
     if (i >= g.V) return;
     const Coord c = site_coord(g, i);
-    const int s = canon_index(g, c.x);
-    for (int nu = 0; nu < 4; ++nu) {
-        double2 e[9];
-        for (int q = 0; q < 9; ++q) e[q] = Uc[((size_t)s * 4 + nu) * 9 + q];
-        for (int q = 0; q < 9; ++q) {
-            U64[((size_t)nu * 9 + q) * g.V + i] = e[q];
-            U18[((size_t)nu * 9 + q) * g.V + i] = make_float2((float)e[q].x, (float)e[q].y);
-            const dfc d = c2dfc(d2df(e[q]));
-            Udf[((size_t)nu * 9 + q) * g.V + i] = make_float4(d.rh, d.rl, d.ih, d.il);
-        }
-        U12[((size_t)nu * 3 + 0) * g.V + i] = make_float4(e[0].x, e[0].y, e[1].x, e[1].y);
-        U12[((size_t)nu * 3 + 1) * g.V + i] = make_float4(e[2].x, e[2].y, e[3].x, e[3].y);
-        U12[((size_t)nu * 3 + 2) * g.V + i] = make_float4(e[4].x, e[4].y, e[5].x, e[5].y);
+    const double2* u = Uc + ((size_t)canon_index(g, c.x) * 4 + nu) * 9;
+    double2 e[9];
+#pragma unroll
+    for (int q = 0; q < 9; ++q) e[q] = __ldg(u + q);
+#pragma unroll
+    for (int q = 0; q < 9; ++q) {
+        const size_t o = ((size_t)nu * 9 + q) * g.V + i;
+        U64[o] = e[q];
+        U18[o] = make_float2((float)e[q].x, (float)e[q].y);
+        const dfc d = c2dfc(d2df(e[q]));
+        Udf[o] = make_float4(d.rh, d.rl, d.ih, d.il);
     }
+    U12[((size_t)nu * 3 + 0) * g.V + i] = make_float4(e[0].x, e[0].y, e[1].x, e[1].y);
+    U12[((size_t)nu * 3 + 1) * g.V + i] = make_float4(e[2].x, e[2].y, e[3].x, e[3].y);
+    U12[((size_t)nu * 3 + 2) * g.V + i] = make_float4(e[4].x, e[4].y, e[5].x, e[5].y);
 }
 
 __global__ void k_f64_to_df(void* x, size_t n) {
@@ -702,7 +707,7 @@ void launch_f64_to_df(void* x, size_t n, cudaStream_t st) {
 
 void launch_pack_gauge(const double2* U_canon, double2* U64, float4* U12, float2* U18, float4* Udf, const Geom& g,
                        cudaStream_t st) {
-    k_pack_gauge<<<(g.V + 127) / 128, 128, 0, st>>>(U_canon, U64, U12, U18, Udf, g);
+    k_pack_gauge<<<(g.V + 31) / 32, 128, 0, st>>>(U_canon, U64, U12, U18, Udf, g);
 }
 
 __global__ void k_pack_spinor(const double2* __restrict__ canon, void* __restrict__ native, int prec, Geom g) {
