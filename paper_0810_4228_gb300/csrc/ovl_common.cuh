@@ -5,6 +5,7 @@
 #pragma once
 
 #include <cuda_runtime.h>
+#include <math.h>
 #include <stdint.h>
 
 #ifndef OVL_HD
@@ -44,15 +45,19 @@ template <class R> OVL_HD R norm2(cx<R> a) { return a.r * a.r + a.i * a.i; }
 template <class R> OVL_HD cx<R> cdot(cx<R> a, cx<R> b) {
     return mk(a.r * b.r + a.i * b.i, a.r * b.i - a.i * b.r);
 }
+// one rounding per product (a.r += b.r c.r - b.i c.i as an expression is a product, a fused multiply-add and
+// an addition: three instructions and three roundings instead of two)
+OVL_HD double mad(double a, double b, double c) { return fma(a, b, c); }
+OVL_HD float mad(float a, float b, float c) { return fmaf(a, b, c); }
 // a += b * c
 template <class R> OVL_HD void cfma(cx<R>& a, cx<R> b, cx<R> c) {
-    a.r += b.r * c.r - b.i * c.i;
-    a.i += b.r * c.i + b.i * c.r;
+    a.r = mad(-b.i, c.i, mad(b.r, c.r, a.r));
+    a.i = mad(b.i, c.r, mad(b.r, c.i, a.i));
 }
 // a += conj(b) * c
 template <class R> OVL_HD void cfmac(cx<R>& a, cx<R> b, cx<R> c) {
-    a.r += b.r * c.r + b.i * c.i;
-    a.i += b.r * c.i - b.i * c.r;
+    a.r = mad(b.i, c.i, mad(b.r, c.r, a.r));
+    a.i = mad(-b.i, c.r, mad(b.r, c.i, a.i));
 }
 OVL_HD cx<double> up(cx<float> a) { return mk<double>(a.r, a.i); }
 OVL_HD cx<double> up(cx<double> a) { return a; }
