@@ -108,7 +108,7 @@ int ensure_solve(ovl_ctx* c, int k) {
     int r = ensure_base(c);
     if (r) return r;
     const int mdb = ovl::multidot_blocks(c->n);
-    const size_t need_part = std::max<size_t>((size_t)(k + 2 + 2 * std::max(c->m, 1)) * mdb * sizeof(double2),
+    const size_t need_part = std::max<size_t>((size_t)(k + 2 + 2 * std::max(c->m, 1)) * (mdb + 1) * sizeof(double2),
                                               (size_t)1 << 19);
     if (k <= c->kcap && c->partials_bytes >= need_part) return OVL_OK;
     drop_graph(c);
@@ -469,9 +469,9 @@ int enqueue_solve(ovl_ctx* c, int method, int k, double mu, double kappa, int fl
                 float4* un = Vd + (size_t)(j + 1) * n;
                 prof(c, KC_ADSLASH, [&] { ovl::launch_dslash(c->U64, 0, x64, c->t64, mu, kappa, 1, g, st, ks); });
                 prof(c, KC_ADOT, [&] {
-                    ovl::launch_adf_dot2(Vd, n, j + 1, uj, c->t64, c->h1, c->h2, part, n, c->num_sms, ks, st);
+                    ovl::launch_adf_dot2(Vd, n, j + 1, uj, c->t64, c->h1, c->h2, h1d, h2d, c->H, ldH, part, cnt, n,
+                                         c->num_sms, ks, st);
                 }, 2);
-                prof(c, KC_ANORM, [&] { ovl::launch_adf_dcgs(c->H, ldH, c->h1, c->h2, h1d, h2d, ks, j, 0, st); });
                 prof(c, KC_AAXPY, [&] {
                     ovl::launch_adf_update2(Vd, n, j, h1d, h2d, uj, un, c->t64, x64, c->H, ldH, c->h1, c->h2, n, ks,
                                             st);
@@ -481,7 +481,7 @@ int enqueue_solve(ovl_ctx* c, int method, int k, double mu, double kappa, int fl
             prof(c, KC_ADOT, [&] {
                 ovl::launch_adf_dot(Vd, n, k + 1, Vd + (size_t)k * n, c->h1, h1d, part, n, c->num_sms, ks, st);
             }, 2);
-            prof(c, KC_ANORM, [&] { ovl::launch_adf_dcgs(c->H, ldH, c->h1, c->h2, h1d, h2d, ks, k, 1, st); });
+            prof(c, KC_ANORM, [&] { ovl::launch_adf_dcgs(c->H, ldH, c->h1, c->h2, ks, k, 1, st); });
         } else
         for (int j = 0; j < k; ++j) {
             float4* t = Vd + (size_t)(j + 1) * n;
@@ -569,18 +569,18 @@ int enqueue_restarted(ovl_ctx* c, int rs, int cycles, double mu, double kappa, i
             float4* un = Vd + (size_t)(j + 1) * n;
             prof(c, KC_ADSLASH, [&] { ovl::launch_dslash(c->U64, 0, x64, c->t64, mu, kappa, 1, g, st, ks); });
             prof(c, KC_ADOT, [&] {
-                ovl::launch_adf_dot2(Vd, n, j + 1, uj, c->t64, c->h1, c->h2, part, n, c->num_sms, ks, st);
+                ovl::launch_adf_dot2(Vd, n, j + 1, uj, c->t64, c->h1, c->h2, h1d, h2d, Hc, ldH, part, cnt, n,
+                                     c->num_sms, ks, st);
             }, 2);
-            prof(c, KC_ANORM, [&] { ovl::launch_adf_dcgs(Hc, ldH, c->h1, c->h2, h1d, h2d, ks, j, 0, st); });
             prof(c, KC_AAXPY, [&] {
                 ovl::launch_adf_update2(Vd, n, j, h1d, h2d, uj, un, c->t64, x64, Hc, ldH, c->h1, c->h2, n, ks, st);
             });
         }
         // re-orthogonalise u_rs: finishes the cycle's last column and its coupling entry
         prof(c, KC_ADOT, [&] {
-            ovl::launch_adf_dot(Vd, n, rs + 1, Vd + (size_t)rs * n, c->h1, h2d, part, n, c->num_sms, ks, st);
+            ovl::launch_adf_dot(Vd, n, rs + 1, Vd + (size_t)rs * n, c->h1, h1d, part, n, c->num_sms, ks, st);
         }, 2);
-        prof(c, KC_ANORM, [&] { ovl::launch_adf_dcgs(Hc, ldH, c->h1, c->h2, h1d, h2d, ks, rs, 2, st); });
+        prof(c, KC_ANORM, [&] { ovl::launch_adf_dcgs(Hc, ldH, c->h1, c->h2, ks, rs, 2, st); });
         prof(c, KC_SETUP, [&] { ovl::launch_rs_mid(ks, st); });
         // inner sign of the accumulated matrix, then this cycle's share of the combination
         int r = 0;

@@ -12,6 +12,8 @@
 // bound.  The coefficients h, H and the inner sign stay FP64; every product enters its sum through
 // the exact FMA split (dfacc), and every sum of per-lane, per-warp and per-block partials is
 // deterministic (fixed order).
+#include <algorithm>
+
 #include "ovl_kernels.h"
 #include "df32.cuh"
 
@@ -21,8 +23,33 @@ static constexpr int AD_T = 256;    // threads per block
 static constexpr int AD_W = AD_T / 32;
 static constexpr int AD_CH = 1024;  // elements of x per block in the many-vector dot
 
-__device__ __forceinline__ float4 to_f4(cx<df> z) { return make_float4(z.r.hi, z.r.lo, z.i.hi, z.i.lo); }
-__device__ __forceinline__ cx<df> from_f4(float4 v) { return mk(df(v.x, v.y), df(v.z, v.w)); }
+// Storage of one complex number here: {re.hi, im.hi, re.lo, im.lo}, so that the leading and the trailing
+// parts are the operand pairs of the packed FP32x2 arithmetic (df32.cuh) as loaded.
+__device__ __forceinline__ float4 to_f4(cx<df> z) { return make_float4(z.r.hi, z.i.hi, z.r.lo, z.i.lo); }
+__device__ __forceinline__ cx<df> from_f4(float4 v) { return mk(df(v.x, v.z), df(v.y, v.w)); }
+
+// Complex sums of products in packed form: A collects (a.r v.r, a.i v.i), B (a.r v.i, a.i v.r); the two
+// halves of each are combined once at the end, so a term is 24 packed instructions and four moves (the
+// swapped v) instead of 48 scalar ones.
+struct PAcc {
+    dfacc2 A, B;
+};
+__device__ __forceinline__ void pacc_zero(PAcc& p) {
+    p.A.s = p.A.e = p.B.s = p.B.e = make_float2(0.f, 0.f);
+}
+__device__ __forceinline__ void pacc_add(PAcc& p, const float4& a, const float4& v) {
+    const float2 ah = make_float2(a.x, a.y), al = make_float2(a.z, a.w);
+    dfacc2_add(p.A, ah, al, make_float2(v.x, v.y), make_float2(v.z, v.w));
+    dfacc2_add(p.B, ah, al, make_float2(v.y, v.x), make_float2(v.w, v.z));
+}
+// sum a v
+__device__ __forceinline__ cx<df> pacc_product(const PAcc& p) {
+    return mk(df(p.A.s.x, p.A.e.x) - df(p.A.s.y, p.A.e.y), df(p.B.s.x, p.B.e.x) + df(p.B.s.y, p.B.e.y));
+}
+// sum conj(v) a
+__device__ __forceinline__ cx<df> pacc_dot(const PAcc& p) {
+    return mk(df(p.A.s.x, p.A.e.x) + df(p.A.s.y, p.A.e.y), df(p.B.s.y, p.B.e.y) - df(p.B.s.x, p.B.e.x));
+}
 
 // sum over the 32 lanes of a warp (butterfly; every lane ends with the same value)
 __device__ __forceinline__ df warp_sum_df(df a) {
@@ -70,24 +97,31 @@ __device__ __forceinline__ void cp_async16(float4* smem, const float4* gmem) {
     const unsigned s = (unsigned)__cvta_generic_to_shared(smem);
     asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(s), "l"(gmem) : "memory");
 }
+// Vectors of the basis that two consecutive sweeps cannot both find in L2 are read as evict-first, so that
+// the last ones (AD_KEEP bytes of 129 MB) stay there from sweep to sweep: k = 450 on 8^4 (a basis of up to
+// 354 MB) 54.2 -> 52.1 ms.  A shorter basis has none of them.
+static constexpr size_t AD_KEEP = (size_t)88 << 20;
+__device__ __forceinline__ unsigned long long evict_first_policy() {
+    unsigned long long p;
+    asm("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(p));
+    return p;
+}
+__device__ __forceinline__ void cp_async16_hint(float4* smem, const float4* gmem, unsigned long long pol) {
+    const unsigned s = (unsigned)__cvta_generic_to_shared(smem);
+    asm volatile("cp.async.cg.shared.global.L2::cache_hint [%0], [%1], 16, %2;" ::"r"(s), "l"(gmem), "l"(pol)
+                 : "memory");
+}
+__device__ __forceinline__ float4 ldg_hint(const float4* p, unsigned long long pol) {
+    float4 v;
+    asm("ld.global.nc.L2::cache_hint.v4.f32 {%0, %1, %2, %3}, [%4], %5;"
+        : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w)
+        : "l"(p), "l"(pol));
+    return v;
+}
+static int adf_cold(int nvec, size_t n) { return (int)std::max<long long>(0, nvec - (long long)(AD_KEEP / (n * sizeof(float4)))); }
 __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
 template <int N> __device__ __forceinline__ void cp_async_wait() {
     asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory");
-}
-
-// re + i im += conj(v) x
-__device__ __forceinline__ void adf_dot_term(dfacc& re, dfacc& im, const cx<df>& v, const cx<df>& xx) {
-    dfacc_add(re, v.r, xx.r, false);
-    dfacc_add(re, v.i, xx.i, false);
-    dfacc_add(im, v.r, xx.i, false);
-    dfacc_add(im, v.i, xx.r, true);
-}
-// re + i im += h v
-__device__ __forceinline__ void adf_axpy_term(dfacc& re, dfacc& im, const cx<df>& h, const cx<df>& v) {
-    dfacc_add(re, h.r, v.r, false);
-    dfacc_add(re, h.i, v.i, true);
-    dfacc_add(im, h.r, v.i, false);
-    dfacc_add(im, h.i, v.r, false);
 }
 
 // stage 1, grid (chunks, vector groups): block (c, g) stages elements [c*AD_CH, (c+1)*AD_CH) of
@@ -126,7 +160,8 @@ __global__ void __launch_bounds__(AD_T) k_adf_dot(const float4* __restrict__ V, 
         cp_async_commit();
     };
     if (total > 0) issue(0);
-    dfacc re = {0.f, 0.f}, im = {0.f, 0.f};
+    PAcc acc;
+    pacc_zero(acc);
     for (int it = 0; it < total; ++it) {
         if (it + 1 < total) {
             issue(it + 1);
@@ -139,14 +174,12 @@ __global__ void __launch_bounds__(AD_T) k_adf_dot(const float4* __restrict__ V, 
         const float4* cur = wb + (it & 1) * AD_SUB;
         const float4* xt = xs + si * AD_SUB;
         const int cnt = min(AD_SUB, lim - si * AD_SUB);
-        if (si == 0) {
-            re = {0.f, 0.f};
-            im = {0.f, 0.f};
-        }
+        if (si == 0) pacc_zero(acc);
 #pragma unroll 4
-        for (int u = lane; u < cnt; u += 32) adf_dot_term(re, im, from_f4(cur[u]), from_f4(xt[u]));
+        for (int u = lane; u < cnt; u += 32) pacc_add(acc, xt[u], cur[u]);
         if (si == ntile - 1) {
-            const df sr = warp_sum_df(dfacc_value(re)), si2 = warp_sum_df(dfacc_value(im));
+            const cx<df> d = pacc_dot(acc);
+            const df sr = warp_sum_df(d.r), si2 = warp_sum_df(d.i);
             if (lane == 0)
                 part[(size_t)(l0 + a * AD_W) * gridDim.x + blockIdx.x] = make_double2(sr.to_double(), si2.to_double());
         }
@@ -182,26 +215,22 @@ __global__ void k_adf_dot_reduce(const double2* __restrict__ part, int nblk, int
 __device__ __forceinline__ void adf_lincomb(const float4* __restrict__ V, size_t ld, int nvec,
                                             const float4* __restrict__ c, size_t e, bool in, int wid, int lane,
                                             float4 (&red)[AD_W][32], cx<df>& sum) {
-    dfacc re = {0.f, 0.f}, im = {0.f, 0.f};
+    PAcc acc;
+    pacc_zero(acc);
     if (in) {
 #pragma unroll 4
         for (int l = wid; l < nvec; l += AD_W) {
             if ((lane & 7) == 0 && l + AD_PFV * AD_W < nvec)  // one lane per 128-byte line
                 prefetch_l2(V + (size_t)(l + AD_PFV * AD_W) * ld + e);
-            adf_axpy_term(re, im, from_f4(__ldg(c + l)), from_f4(__ldg(V + (size_t)l * ld + e)));
+            pacc_add(acc, __ldg(c + l), __ldg(V + (size_t)l * ld + e));
         }
     }
-    red[wid][lane] = make_float4(re.s, re.e, im.s, im.e);
+    red[wid][lane] = to_f4(pacc_product(acc));
     __syncthreads();
     if (wid == 0) {
-        df sr = df_fast2sum(red[0][lane].x, red[0][lane].y), si = df_fast2sum(red[0][lane].z, red[0][lane].w);
+        sum = from_f4(red[0][lane]);
 #pragma unroll
-        for (int w = 1; w < AD_W; ++w) {
-            const float4 p = red[w][lane];
-            sr = sr + df_fast2sum(p.x, p.y);
-            si = si + df_fast2sum(p.z, p.w);
-        }
-        sum = mk(sr, si);
+        for (int w = 1; w < AD_W; ++w) sum = sum + from_f4(red[w][lane]);
     }
 }
 
@@ -324,42 +353,69 @@ __global__ void __launch_bounds__(AD_T) k_adf_combine(const float4* __restrict__
 // one more dot sweep re-orthogonalises u_k and finishes column k-1.  In exact arithmetic this is
 // the Arnoldi process of Sec. 2 (Eq. 2.2-2.3).
 
-static size_t adf_dot2_smem() { return sizeof(float4) * (2 * (size_t)AD_CH + (size_t)AD_W * 2 * AD_SUB); }
+// Bound by the FP32 pipe (24 packed operations per term, 58 % of its rate) beside 16 bytes of basis per term.
+// All sweeps of k = 450 on 8^4: 29 ms in scalar arithmetic, 24.4 ms packed.
+// Chunks of 512 elements and staging tiles of 128: 48 KB per block, four blocks (32 warps) per SM, and tasks
+// (one vector over one chunk) small enough that the last round of warps costs little.
+static constexpr int D2_CH = 512, D2_SUB = 128;
+static size_t adf_dot2_smem() { return sizeof(float4) * (2 * (size_t)D2_CH + (size_t)AD_W * 2 * D2_SUB); }
+
+// Warp sums of the four real numbers of two complex ones, transposed (6 double-float additions instead of
+// 20): lanes 0, 8, 16, 24 end with a.r, a.i, b.r, b.i.
+__device__ __forceinline__ df warp_sum4_df(const cx<df>& a, const cx<df>& b) {
+    const int lane = threadIdx.x & 31;
+    auto xchg = [](df x, int o) {
+        return df(__shfl_xor_sync(0xffffffffu, x.hi, o), __shfl_xor_sync(0xffffffffu, x.lo, o));
+    };
+    const bool u16 = lane & 16, u8 = lane & 8;
+    const df p = (u16 ? b.r : a.r) + xchg(u16 ? a.r : b.r, 16);
+    const df q = (u16 ? b.i : a.i) + xchg(u16 ? a.i : b.i, 16);
+    df r = (u8 ? q : p) + xchg(u8 ? p : q, 8);
+    r = r + xchg(r, 4);
+    r = r + xchg(r, 2);
+    return r + xchg(r, 1);
+}
 
 // stage 1 of the two-vector dot, grid (chunks, vector groups): V_l^dag x1 and V_l^dag x2 for every
 // l < nvec over the block's chunk; x1 is a double-float vector, x2 an FP64 one (split on staging).
 // Partials: part[(2 l + q) * gridDim.x + chunk], q = 0 for x1, 1 for x2.
-__global__ void __launch_bounds__(AD_T) k_adf_dot2(const float4* __restrict__ V, size_t ld, int nvec, int vpb,
+__global__ void __launch_bounds__(AD_T, 4) k_adf_dot2(const float4* __restrict__ V, size_t ld, int nvec, int vpb, int cold,
                                                    const float4* __restrict__ x1, const double2* __restrict__ x2,
                                                    double2* __restrict__ part, size_t n, const KState* ks) {
     extern __shared__ float4 adf_sm[];
     float4* xs1 = adf_sm;
-    float4* xs2 = adf_sm + AD_CH;
+    float4* xs2 = adf_sm + D2_CH;
     if (ks->done || ks->status) return;
-    const size_t base = (size_t)blockIdx.x * AD_CH;
-    const int lim = (int)(n - base < (size_t)AD_CH ? n - base : (size_t)AD_CH);
+    const size_t base = (size_t)blockIdx.x * D2_CH;
+    const int lim = (int)(n - base < (size_t)D2_CH ? n - base : (size_t)D2_CH);
     for (int q = threadIdx.x; q < lim; q += AD_T) {
         xs1[q] = x1[base + q];
         xs2[q] = to_f4(d2df(x2[base + q]));
     }
     __syncthreads();
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    float4* wb = adf_sm + 2 * AD_CH + (size_t)wid * 2 * AD_SUB;
+    float4* wb = adf_sm + 2 * D2_CH + (size_t)wid * 2 * D2_SUB;
     const int l0 = blockIdx.y * vpb + wid;
     const int l1 = min(nvec, blockIdx.y * vpb + vpb);
     const int nv = l0 < l1 ? (l1 - l0 + AD_W - 1) / AD_W : 0;
-    const int ntile = (lim + AD_SUB - 1) / AD_SUB;
+    const int ntile = (lim + D2_SUB - 1) / D2_SUB;
     const int total = nv * ntile;
+    const unsigned long long pol = evict_first_policy();
     auto issue = [&](int it) {
         const int a = it / ntile, si = it - a * ntile;
-        const float4* src = V + (size_t)(l0 + a * AD_W) * ld + base + (size_t)si * AD_SUB;
-        float4* dst = wb + (it & 1) * AD_SUB;
-        const int cnt = min(AD_SUB, lim - si * AD_SUB);
-        for (int u = lane; u < cnt; u += 32) cp_async16(dst + u, src + u);
+        const float4* src = V + (size_t)(l0 + a * AD_W) * ld + base + (size_t)si * D2_SUB;
+        float4* dst = wb + (it & 1) * D2_SUB;
+        const int cnt = min(D2_SUB, lim - si * D2_SUB);
+        if (l0 + a * AD_W < cold)
+            for (int u = lane; u < cnt; u += 32) cp_async16_hint(dst + u, src + u, pol);
+        else
+            for (int u = lane; u < cnt; u += 32) cp_async16(dst + u, src + u);
         cp_async_commit();
     };
     if (total > 0) issue(0);
-    dfacc re1 = {0.f, 0.f}, im1 = {0.f, 0.f}, re2 = {0.f, 0.f}, im2 = {0.f, 0.f};
+    PAcc a1, a2;
+    pacc_zero(a1);
+    pacc_zero(a2);
     for (int it = 0; it < total; ++it) {
         if (it + 1 < total) {
             issue(it + 1);
@@ -369,144 +425,199 @@ __global__ void __launch_bounds__(AD_T) k_adf_dot2(const float4* __restrict__ V,
         }
         __syncwarp();
         const int a = it / ntile, si = it - a * ntile;
-        const float4* cur = wb + (it & 1) * AD_SUB;
-        const int cnt = min(AD_SUB, lim - si * AD_SUB);
-        if (si == 0) re1 = im1 = re2 = im2 = {0.f, 0.f};
+        const float4* cur = wb + (it & 1) * D2_SUB;
+        const int cnt = min(D2_SUB, lim - si * D2_SUB);
+        if (si == 0) {
+            pacc_zero(a1);
+            pacc_zero(a2);
+        }
 #pragma unroll 4
         for (int u = lane; u < cnt; u += 32) {
-            const cx<df> v = from_f4(cur[u]);
-            adf_dot_term(re1, im1, v, from_f4(xs1[si * AD_SUB + u]));
-            adf_dot_term(re2, im2, v, from_f4(xs2[si * AD_SUB + u]));
+            const float4 v = cur[u];
+            pacc_add(a1, xs1[si * D2_SUB + u], v);
+            pacc_add(a2, xs2[si * D2_SUB + u], v);
         }
         if (si == ntile - 1) {
-            const df s1r = warp_sum_df(dfacc_value(re1)), s1i = warp_sum_df(dfacc_value(im1));
-            const df s2r = warp_sum_df(dfacc_value(re2)), s2i = warp_sum_df(dfacc_value(im2));
-            if (lane == 0) {
+            const cx<df> d1 = pacc_dot(a1), d2 = pacc_dot(a2);
+            const df r = warp_sum4_df(d1, d2);
+            if ((lane & 7) == 0) {
                 const size_t l = (size_t)(l0 + a * AD_W);
-                part[(2 * l) * gridDim.x + blockIdx.x] = make_double2(s1r.to_double(), s1i.to_double());
-                part[(2 * l + 1) * gridDim.x + blockIdx.x] = make_double2(s2r.to_double(), s2i.to_double());
+                reinterpret_cast<double*>(part + (2 * l + (lane >> 4)) * gridDim.x + blockIdx.x)[(lane >> 3) & 1] =
+                    r.to_double();
             }
         }
         __syncwarp();  // this tile's buffer receives the copy issued two iterations on
     }
 }
 
-// stage 2: one warp per (vector, operand) sums its chunk partials in FP64 (fixed order):
-// h1[l] = V_l^dag x1, h2[l] = V_l^dag x2
-__global__ void k_adf_dot2_reduce(const double2* __restrict__ part, int nblk, int nvec, double2* __restrict__ h1,
-                                  double2* __restrict__ h2, const KState* ks) {
-    if (ks->done || ks->status) return;
-    const int lane = threadIdx.x & 31;
-    const int p = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
-    if (p >= 2 * nvec) return;
-    double re = 0.0, im = 0.0;
-    for (int b = lane; b < nblk; b += 32) {
-        const double2 v = part[(size_t)p * nblk + b];
-        re += v.x;
-        im += v.y;
-    }
-    re = warp_sum(re);
-    im = warp_sum(im);
-    if (lane == 0) ((p & 1) ? h2 : h1)[p >> 1] = make_double2(re, im);
-}
-
-// (2): one block.  h1 = (c, rho^2) and h2 = (d, e) of step j (h2 unused when fin).  Finishes
-// column j-1 of H (j >= 1), decides a lucky breakdown (nu <= bdtol |H|), and for the update writes
-// cdf = c, qdf = d / nu (double-float), ks->red[1] = (1 / nu, nu), ks->red[2] = r.  fin = 1 after
-// the last step (j = k): only column k-1 is finished and the solve is marked done.  fin = 2 at the
-// end of a restart cycle: column k-1 is finished, cdf = c and ks->red[1] are written for the next
-// cycle's start vector (u_k - V c) / nu, and the solve goes on unless the Krylov space is invariant.
-__global__ void __launch_bounds__(1024) k_adf_dcgs(double2* __restrict__ H, int ldH, const double2* __restrict__ h1,
-                                                   const double2* __restrict__ h2, float4* __restrict__ cdf,
-                                                   float4* __restrict__ qdf, KState* ks, int j, int fin,
-                                                   double bdtol) {
-    __shared__ double red[4 * 32];  // block_sum<4>: 32 doubles per value
-    __shared__ double s_nu;
-    __shared__ int s_stop;
-    if (ks->done || ks->status) return;
+// (2), one block of 256 threads.  h1 = (c, rho^2) and h2 = (d, e) of step j (h2 unused when fin).  Finishes
+// column j-1 of H (j >= 1), decides a lucky breakdown (nu <= bdtol |H|) and for the update writes
+// ks->red[1] = (1 / nu, nu), ks->red[2] = r, ks->red[3].x != 0 where |c| <= 2^-30 rho.  fin = 1 after the
+// last step (j = k): only column k-1 is finished and the solve is marked done.  fin = 2 at the end of a
+// restart cycle: column k-1 is finished and ks->red[1] written for the next cycle's start vector
+// (u_k - V c) / nu, and the solve goes on unless the Krylov space is invariant.
+// FP64 instructions take 64 cycles of their warp each: the four sums are transposed over the warp (6
+// additions instead of 20), nu comes from one reciprocal square root, and the column norm's own square root
+// is taken by another warp.
+static constexpr int DC_T = 256;
+__device__ __forceinline__ void dcgs_block(double2* __restrict__ H, int ldH, const double2* h1, const double2* h2,
+                                           KState* ks, int j, int fin, double bdtol) {
+    __shared__ double red[DC_T / 32][4];
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     // |c|^2, c^dag d, |H[<j, j-1] + c|^2
-    double acc[4] = {0.0, 0.0, 0.0, 0.0};
-    for (int l = threadIdx.x; l < j; l += blockDim.x) {
-        const double2 c = h1[l];
-        acc[0] += c.x * c.x + c.y * c.y;
+    double a0 = 0.0, a1 = 0.0, a2 = 0.0, a3 = 0.0;
+    for (int l = threadIdx.x; l < j; l += DC_T) {
+        const double2 c = __ldcg(h1 + l);
+        a0 = fma(c.x, c.x, fma(c.y, c.y, a0));
         if (!fin) {
-            const double2 d = h2[l];
-            acc[1] += c.x * d.x + c.y * d.y;
-            acc[2] += c.x * d.y - c.y * d.x;
+            const double2 d = __ldcg(h2 + l);
+            a1 = fma(c.x, d.x, fma(c.y, d.y, a1));
+            a2 = fma(c.x, d.y, fma(-c.y, d.x, a2));
         }
-        const double2 hv = H[l + (size_t)(j - 1) * ldH];
-        const double hr = hv.x + c.x, hi = hv.y + c.y;
-        acc[3] += hr * hr + hi * hi;
+        double2* hp = H + l + (size_t)(j - 1) * ldH;
+        double2 hv = *hp;
+        hv.x += c.x;
+        hv.y += c.y;
+        *hp = hv;
+        a3 = fma(hv.x, hv.x, fma(hv.y, hv.y, a3));
     }
-    block_sum<4>(acc, red);
-    if (threadIdx.x == 0) {
-        const double rho2 = h1[j].x;
-        const double nu2 = rho2 - acc[0];
-        const double nu = nu2 > 0.0 ? sqrt(nu2) : 0.0;
-        int stop = 0;
-        if (j >= 1) {
-            H[j + (size_t)(j - 1) * ldH] = make_double2(nu, 0.0);
-            const double colnorm = sqrt(acc[3] + nu * nu);
-            if (colnorm > ks->anorm) ks->anorm = colnorm;
-            ks->kused = j;
-            if (fin == 1 || nu <= bdtol * fmax(ks->anorm, 1e-300)) stop = 1;  // last column, or K_j invariant
-        } else if (!(nu > 0.0)) {
-            stop = 1;  // zero start vector (cannot happen after the deflation split's check)
-        }
-        if (stop) {
-            ks->done = 1;
-        } else {
-            const double inu = 1.0 / nu;
-            ks->red[1] = make_double2(inu, nu);
-            if (!fin) {  // r = (e - c^dag d) / nu^2
-                const double2 e = h2[j];
-                ks->red[2] = make_double2((e.x - acc[1]) * inu * inu, (e.y - acc[2]) * inu * inu);
-            }
-        }
-        s_nu = nu;
-        s_stop = stop;
+    {
+        const bool u16 = lane & 16, u8 = lane & 8;
+        const double b0 = (u16 ? a2 : a0) + __shfl_xor_sync(0xffffffffu, u16 ? a0 : a2, 16);
+        const double b1 = (u16 ? a3 : a1) + __shfl_xor_sync(0xffffffffu, u16 ? a1 : a3, 16);
+        double r = (u8 ? b1 : b0) + __shfl_xor_sync(0xffffffffu, u8 ? b0 : b1, 8);
+        r += __shfl_xor_sync(0xffffffffu, r, 4);
+        r += __shfl_xor_sync(0xffffffffu, r, 2);
+        r += __shfl_xor_sync(0xffffffffu, r, 1);
+        if ((lane & 7) == 0) red[wid][lane >> 3] = r;  // lanes 0, 8, 16, 24: values 0, 1, 2, 3
     }
     __syncthreads();
-    const double inu = s_stop ? 0.0 : 1.0 / s_nu;
-    for (int l = threadIdx.x; l < j; l += blockDim.x) {
-        const double2 c = h1[l];
-        const double2 hv = H[l + (size_t)(j - 1) * ldH];
-        H[l + (size_t)(j - 1) * ldH] = make_double2(hv.x + c.x, hv.y + c.y);
-        if (!s_stop) {
-            cdf[l] = to_f4(d2df(c));
-            if (!fin) {
-                const double2 d = h2[l];
-                qdf[l] = to_f4(d2df(make_double2(d.x * inu, d.y * inu)));
-            }
+    if (wid >= 2) return;
+    double t = red[lane >> 2][lane & 3];
+    t += __shfl_xor_sync(0xffffffffu, t, 16);
+    t += __shfl_xor_sync(0xffffffffu, t, 8);
+    t += __shfl_xor_sync(0xffffffffu, t, 4);
+    const double c2 = __shfl_sync(0xffffffffu, t, 0), er = __shfl_sync(0xffffffffu, t, 1);
+    const double ei = __shfl_sync(0xffffffffu, t, 2), hn2 = __shfl_sync(0xffffffffu, t, 3);
+    if (lane) return;
+    const double rho2 = __ldcg(&h1[j].x), nu2 = rho2 - c2;
+    if (wid == 1) {  // |H| so far, in the record of the next steps (warp 0 works with its square)
+        if (j >= 1) {
+            const double an = sqrt(hn2 + (nu2 > 0.0 ? nu2 : 0.0));
+            if (an > ks->red[0].y) ks->red[0].y = an;
+            ks->anorm = ks->red[0].y;
         }
+        return;
+    }
+    const double inu = nu2 > 0.0 ? rsqrt(nu2) : 0.0, nu = nu2 > 0.0 ? nu2 * inu : 0.0;
+    int stop = 0;
+    if (j >= 1) {
+        H[j + (size_t)(j - 1) * ldH] = make_double2(nu, 0.0);
+        const double an2 = fmax(fmax(ks->red[0].x, hn2 + nu * nu), 1e-300);  // largest column so far, squared
+        ks->red[0].x = an2;
+        ks->kused = j;
+        if (fin == 1 || nu * nu <= bdtol * bdtol * an2) stop = 1;  // last column, or K_j invariant
+    } else if (!(nu > 0.0)) {
+        stop = 1;  // zero start vector (cannot happen after the deflation split's check)
+    }
+    if (stop) {
+        ks->done = 1;
+        return;
+    }
+    ks->red[1] = make_double2(inu, nu);
+    if (!fin) {  // r = (e - c^dag d) / nu^2
+        const double2 e = __ldcg(h2 + j);
+        const double i2 = inu * inu;
+        ks->red[2] = make_double2((e.x - er) * i2, (e.y - ei) * i2);
+        ks->red[3] = make_double2(c2 <= 0x1p-60 * rho2 ? 1.0 : 0.0, 0.0);
     }
 }
 
-// (3): per element e, over the final vectors V_0..V_{j-1}: s1 = sum_l c_l V_l[e], s2 = sum_l
-// (d_l / nu) V_l[e]; then v_j = (u_j - s1) / nu into slot j (in place of u_j) and u_{j+1} =
-// w / nu - s2 - r v_j into slot j + 1 and, as FP64, into x64 (the next stencil's input).  Blocks
-// 0..j also write the tentative column j of H: H[i, j] = d_i / nu - g_i (i < j), r - c_{j-1}
-// (i = j), g_i = sum_{l >= i-1} H[i, l] c_l / nu (upper Hessenberg rows of the final columns).
-__global__ void __launch_bounds__(AD_T) k_adf_update2(const float4* __restrict__ V, size_t ld, int j,
-                                                      const float4* __restrict__ cdf, const float4* __restrict__ qdf,
-                                                      float4* __restrict__ uj, float4* __restrict__ unext,
-                                                      const double2* __restrict__ w, double2* __restrict__ x64,
-                                                      double2* __restrict__ H, int ldH, const double2* __restrict__ h1,
-                                                      const double2* __restrict__ h2, size_t n, KState* ks) {
+__global__ void __launch_bounds__(DC_T) k_adf_dcgs(double2* __restrict__ H, int ldH, const double2* __restrict__ h1,
+                                                   const double2* __restrict__ h2, KState* ks, int j, int fin,
+                                                   double bdtol) {
+    if (ks->done || ks->status) return;
+    dcgs_block(H, ldH, h1, h2, ks, j, fin, bdtol);
+}
+
+// stage 2 of the two-vector dot: one warp per (vector, operand) sums its chunk partials in FP64 (fixed
+// order): h1[l] = V_l^dag x1, h2[l] = V_l^dag x2, and their double-float splits for the update; the last
+// block to finish goes on with (2) (a launch of its own, a chain of FP64 instructions in one block, took 16 us of each step; in all
+// 7.2 ms of k = 450 on 8^4, now 4.7 ms with the dot's second stage).
+__global__ void __launch_bounds__(DC_T) k_adf_dot2_reduce(const double2* __restrict__ part, int nblk, int nvec,
+                                                          double2* h1, double2* h2, float4* __restrict__ h1d,
+                                                          float4* __restrict__ h2d, double2* __restrict__ H, int ldH,
+                                                          KState* ks, double bdtol, unsigned int* counter) {
+    __shared__ bool last;
+    if (ks->done || ks->status) return;
+    const int lane = threadIdx.x & 31;
+    const int p = blockIdx.x * (DC_T / 32) + (threadIdx.x >> 5);
+    if (p < 2 * nvec) {
+        double re = 0.0, im = 0.0;
+        for (int b = lane; b < nblk; b += 32) {
+            const double2 v = part[(size_t)p * nblk + b];
+            re += v.x;
+            im += v.y;
+        }
+        // even lanes end with the real part's sum, odd lanes with the imaginary part's
+        const bool odd = lane & 1;
+        double r = (odd ? im : re) + __shfl_xor_sync(0xffffffffu, odd ? re : im, 1);
+#pragma unroll
+        for (int o = 2; o < 32; o <<= 1) r += __shfl_xor_sync(0xffffffffu, r, o);
+        const double ri = __shfl_sync(0xffffffffu, r, 1);
+        if (lane == 0) {
+            ((p & 1) ? h2 : h1)[p >> 1] = make_double2(r, ri);
+            ((p & 1) ? h2d : h1d)[p >> 1] = to_f4(d2df(make_double2(r, ri)));
+        }
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        __threadfence();
+        last = atomicAdd(counter, 1u) == gridDim.x - 1;
+    }
+    __syncthreads();
+    if (!last) return;
+    __threadfence();
+    if (threadIdx.x == 0) *counter = 0u;
+    dcgs_block(H, ldH, h1, h2, ks, nvec - 1, 0, bdtol);
+}
+
+// (3): per element e, over the final vectors V_0..V_{j-1}: s1 = sum_l c_l V_l[e], s2 = sum_l d_l V_l[e];
+// then v_j = (u_j - s1) / nu into slot j (in place of u_j) and u_{j+1} = (w - s2) / nu - r v_j into slot
+// j + 1 and, as FP64, into x64 (the next stencil's input).  The first hb blocks write the tentative column j
+// of H, a warp per row: H[i, j] = d_i / nu - g_i (i < j), r - c_{j-1} (i = j), g_i = sum_{l >= i-1} H[i, l] c_l / nu (upper
+// Hessenberg rows of the final columns).
+// Bound by loads in flight (3.8 TB/s of basis).  All sweeps of k = 450 on 8^4: 30.1 ms with both sums scalar,
+// 21.4 ms so.
+// c is what the first projection left behind, 2^-40 of u_j or less while Gram-Schmidt works: with
+// |c| <= 2^-30 rho (ks->red[3], the same in every block) s1 is formed in FP32 from the leading parts, which
+// leaves an error below 2^-50 of u_j, under the double-float rounding of u_j itself; otherwise in
+// double-float like s2.
+static constexpr int UP_CH = 512;  // coefficients staged in shared memory at a time
+__global__ void __launch_bounds__(AD_T, 3) k_adf_update2(const float4* __restrict__ V, size_t ld, int j, int cold, int hb,
+                                                         const float4* __restrict__ cdf, const float4* __restrict__ ddf,
+                                                         float4* __restrict__ uj, float4* __restrict__ unext,
+                                                         const double2* __restrict__ w, double2* __restrict__ x64,
+                                                         double2* __restrict__ H, int ldH,
+                                                         const double2* __restrict__ h1, const double2* __restrict__ h2,
+                                                         size_t n, KState* ks) {
     __shared__ float4 red1[AD_W][32];
     __shared__ float4 red2[AD_W][32];
+    __shared__ float4 dsm[UP_CH];
+    __shared__ float2 csm[UP_CH];
     if (ks->done || ks->status) return;
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    const double2 sc = ks->red[1];
-    const double inu = sc.x;
+    const double inu = ks->red[1].x;
     const double2 r = ks->red[2];
-    if ((int)blockIdx.x <= j && wid == 0) {
-        const int i = blockIdx.x;
+    const bool small = ks->red[3].x != 0.0;
+    if ((int)blockIdx.x < hb) {  // a warp per row of H
+        const int i = blockIdx.x * AD_W + wid;
+        if (i > j) return;
         double gr = 0.0, gi = 0.0;
         for (int l = max(i - 1, 0) + lane; l < j; l += 32) {
             const double2 hv = H[i + (size_t)l * ldH], c = h1[l];
-            gr += hv.x * c.x - hv.y * c.y;
-            gi += hv.x * c.y + hv.y * c.x;
+            gr = fma(hv.x, c.x, fma(-hv.y, c.y, gr));
+            gi = fma(hv.x, c.y, fma(hv.y, c.x, gi));
         }
         gr = warp_sum(gr) * inu;
         gi = warp_sum(gi) * inu;
@@ -521,43 +632,84 @@ __global__ void __launch_bounds__(AD_T) k_adf_update2(const float4* __restrict__
             }
             H[i + (size_t)j * ldH] = hv;
         }
+        return;
     }
     const df dinu(inu);
     const cx<df> rr = d2df(r);
     const size_t ntile = (n + 31) / 32;
-    for (size_t tile = blockIdx.x; tile < ntile; tile += gridDim.x) {
+    const unsigned long long pol = evict_first_policy();
+    for (size_t tile = blockIdx.x - hb; tile < ntile; tile += gridDim.x - hb) {
         const size_t e = tile * 32 + lane;
         const bool in = e < n;
-        dfacc a1r = {0.f, 0.f}, a1i = {0.f, 0.f}, a2r = {0.f, 0.f}, a2i = {0.f, 0.f};
-        if (in) {
-#pragma unroll 4
-            for (int l = wid; l < j; l += AD_W) {
-                if ((lane & 7) == 0 && l + AD_PFV * AD_W < j)  // one lane per 128-byte line
-                    prefetch_l2(V + (size_t)(l + AD_PFV * AD_W) * ld + e);
-                const cx<df> v = from_f4(__ldg(V + (size_t)l * ld + e));
-                adf_axpy_term(a1r, a1i, from_f4(__ldg(cdf + l)), v);
-                adf_axpy_term(a2r, a2i, from_f4(__ldg(qdf + l)), v);
+        PAcc a2;
+        pacc_zero(a2);
+        cx<df> s1 = mk(df(0), df(0));
+        if (small) {
+            float2 fa = make_float2(0.f, 0.f), fb = fa;
+            // four vectors of this warp per round, the next round's loads in flight meanwhile
+            const float4 zero = make_float4(0.f, 0.f, 0.f, 0.f);
+            const float4* Ve = V + e;
+            auto load4 = [&](int l, float4 (&v)[4]) {
+#pragma unroll
+                for (int q = 0; q < 4; ++q) {
+                    const float4* p = Ve + (size_t)(l + q * AD_W) * ld;
+                    v[q] = !in || l + q * AD_W >= j ? zero : l < cold ? ldg_hint(p, pol) : __ldg(p);
+                }
+            };
+            float4 v[4];
+            load4(wid, v);
+            for (int l0 = 0; l0 < j; l0 += UP_CH) {
+                if (l0 > 0 || tile + hb != blockIdx.x) __syncthreads();  // the last chunk has been read
+                for (int l = threadIdx.x; l < UP_CH; l += AD_T) {
+                    const bool ok = l0 + l < j;
+                    dsm[l] = ok ? __ldg(ddf + l0 + l) : zero;
+                    csm[l] = ok ? __ldg(reinterpret_cast<const float2*>(cdf + l0 + l)) : make_float2(0.f, 0.f);
+                }
+                __syncthreads();
+                const int lim = min(UP_CH, j - l0);
+                for (int l = wid; l < lim; l += 4 * AD_W) {
+                    float4 nx[4];
+                    load4(l0 + l + 4 * AD_W, nx);
+#pragma unroll
+                    for (int q = 0; q < 4; ++q) {
+                        const float2 c = csm[l + q * AD_W];
+                        fa = f2_fma(c, make_float2(v[q].x, v[q].y), fa);
+                        fb = f2_fma(c, make_float2(v[q].y, v[q].x), fb);
+                        pacc_add(a2, dsm[l + q * AD_W], v[q]);
+                        v[q] = nx[q];
+                    }
+                }
             }
+            s1 = mk(df(fa.x, 0.f) - df(fa.y, 0.f), df(fb.x, 0.f) + df(fb.y, 0.f));
+        } else {
+            PAcc a1;
+            pacc_zero(a1);
+            if (in) {
+#pragma unroll 2
+                for (int l = wid; l < j; l += AD_W) {
+                    const float4 v = __ldg(V + (size_t)l * ld + e);
+                    pacc_add(a1, __ldg(cdf + l), v);
+                    pacc_add(a2, __ldg(ddf + l), v);
+                }
+            }
+            s1 = pacc_product(a1);
         }
-        red1[wid][lane] = make_float4(a1r.s, a1r.e, a1i.s, a1i.e);
-        red2[wid][lane] = make_float4(a2r.s, a2r.e, a2i.s, a2i.e);
+        red1[wid][lane] = to_f4(s1);
+        red2[wid][lane] = to_f4(pacc_product(a2));
         __syncthreads();
         if (wid == 0 && in) {
-            df s1r = df_fast2sum(red1[0][lane].x, red1[0][lane].y), s1i = df_fast2sum(red1[0][lane].z, red1[0][lane].w);
-            df s2r = df_fast2sum(red2[0][lane].x, red2[0][lane].y), s2i = df_fast2sum(red2[0][lane].z, red2[0][lane].w);
+            s1 = from_f4(red1[0][lane]);
+            cx<df> s2 = from_f4(red2[0][lane]);
 #pragma unroll
             for (int q = 1; q < AD_W; ++q) {
-                const float4 p1 = red1[q][lane], p2 = red2[q][lane];
-                s1r = s1r + df_fast2sum(p1.x, p1.y);
-                s1i = s1i + df_fast2sum(p1.z, p1.w);
-                s2r = s2r + df_fast2sum(p2.x, p2.y);
-                s2i = s2i + df_fast2sum(p2.z, p2.w);
+                s1 = s1 + from_f4(red1[q][lane]);
+                s2 = s2 + from_f4(red2[q][lane]);
             }
             const cx<df> u = from_f4(uj[e]);
-            const cx<df> vj = mk((u.r - s1r) * dinu, (u.i - s1i) * dinu);
+            const cx<df> vj = mk((u.r - s1.r) * dinu, (u.i - s1.i) * dinu);
             const cx<df> ww = d2df(w[e]);
             const cx<df> rv = rr * vj;
-            const cx<df> un = mk(ww.r * dinu - s2r - rv.r, ww.i * dinu - s2i - rv.i);
+            const cx<df> un = mk((ww.r - s2.r) * dinu - rv.r, (ww.i - s2.i) * dinu - rv.i);
             uj[e] = to_f4(vj);
             unext[e] = to_f4(un);
             x64[e] = df2d(un);
@@ -718,11 +870,14 @@ void launch_adf_normalize(float4* t, double2* x64, const KState* ks, size_t n, c
     k_adf_normalize<<<adf_grid(n), 256, 0, st>>>(t, x64, ks, n);
 }
 
+// steps (1) and (2) of step nvec - 1
 void launch_adf_dot2(const float4* V, size_t ld, int nvec, const float4* x1, const double2* x2, double2* h1,
-                     double2* h2, double* partials, size_t n, int num_sms, const KState* ks, cudaStream_t st) {
+                     double2* h2, float4* h1d, float4* h2d, double2* H, int ldH, double* partials,
+                     unsigned int* counter, size_t n, int num_sms, KState* ks, cudaStream_t st) {
     if (nvec <= 0) return;
-    const int nchunk = adf_dot_blocks(n);
-    const long long target = 8ll * (num_sms > 0 ? num_sms : 1);
+    const int nchunk = (int)((n + D2_CH - 1) / D2_CH);
+    // vectors per warp: about 24 blocks per SM in all (six rounds of the four that fit an SM)
+    const long long target = 24ll * (num_sms > 0 ? num_sms : 1);
     long long vpw = ((long long)nvec * nchunk + (long long)AD_W * target - 1) / ((long long)AD_W * target);
     if (vpw < 1) vpw = 1;
     const int vpb = (int)(vpw * AD_W);
@@ -731,22 +886,23 @@ void launch_adf_dot2(const float4* V, size_t ld, int nvec, const float4* x1, con
     static unsigned long long attr_dev = 0;
     if (first_use_on_device(attr_dev))
         cudaFuncSetAttribute(k_adf_dot2, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)adf_dot2_smem());
-    k_adf_dot2<<<dim3(nchunk, ngroup), AD_T, adf_dot2_smem(), st>>>(V, ld, nvec, vpb, x1, x2, part, n, ks);
-    k_adf_dot2_reduce<<<(2 * nvec + 7) / 8, 256, 0, st>>>(part, nchunk, nvec, h1, h2, ks);
-}
-
-void launch_adf_dcgs(double2* H, int ldH, const double2* h1, const double2* h2, float4* cdf, float4* qdf, KState* ks,
-                     int j, int fin, cudaStream_t st) {
+    k_adf_dot2<<<dim3(nchunk, ngroup), AD_T, adf_dot2_smem(), st>>>(V, ld, nvec, vpb, adf_cold(nvec, n), x1, x2, part, n, ks);
     // double-float sweeps: the lucky-breakdown threshold of the double-float CGS2 path (1e-11)
-    k_adf_dcgs<<<1, 1024, 0, st>>>(H, ldH, h1, h2, cdf, qdf, ks, j, fin, 1e-11);
+    k_adf_dot2_reduce<<<(2 * nvec + 7) / 8, DC_T, 0, st>>>(part, nchunk, nvec, h1, h2, h1d, h2d, H, ldH, ks, 1e-11,
+                                                           counter);
 }
 
-void launch_adf_update2(const float4* V, size_t ld, int j, const float4* cdf, const float4* qdf, float4* uj,
+void launch_adf_dcgs(double2* H, int ldH, const double2* h1, const double2* h2, KState* ks, int j, int fin,
+                     cudaStream_t st) {
+    k_adf_dcgs<<<1, DC_T, 0, st>>>(H, ldH, h1, h2, ks, j, fin, 1e-11);
+}
+
+void launch_adf_update2(const float4* V, size_t ld, int j, const float4* cdf, const float4* ddf, float4* uj,
                         float4* unext, const double2* w, double2* x64, double2* H, int ldH, const double2* h1,
                         const double2* h2, size_t n, KState* ks, cudaStream_t st) {
-    unsigned grid = adf_update_grid(n);
-    if (grid < (unsigned)j + 1) grid = (unsigned)j + 1;  // blocks 0..j each write one row of column j
-    k_adf_update2<<<grid, AD_T, 0, st>>>(V, ld, j, cdf, qdf, uj, unext, w, x64, H, ldH, h1, h2, n, ks);
+    const int hb = (j + 1 + AD_W - 1) / AD_W;  // blocks of the rows of H, first
+    k_adf_update2<<<hb + adf_update_grid(n), AD_T, 0, st>>>(V, ld, j, adf_cold(j, n), hb, cdf, ddf, uj, unext, w, x64, H,
+                                                            ldH, h1, h2, n, ks);
 }
 
 void launch_rs_begin(KState* ks, int cyc, cudaStream_t st) { k_rs_begin<<<1, 1, 0, st>>>(ks, cyc); }

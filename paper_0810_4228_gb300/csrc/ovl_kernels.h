@@ -37,7 +37,7 @@ struct Workspace;   // defined in api.cu
 // Udf: the double-float copy of the links (float4 {re.hi, re.lo, im.hi, im.lo} in the FP64 layout)
 void launch_pack_gauge(const double2* U_canon, double2* U64, float4* U12, float2* U18, float4* Udf, const Geom& g,
                        cudaStream_t st);
-// in place: FP64 vectors (double2) -> double-float (float4 {hi, lo, hi, lo}), n complex each; and back
+// in place: FP64 vectors (double2) -> double-float (float4 {hi, lo, hi, lo}), n complex
 void launch_f64_to_df(void* x, size_t n, cudaStream_t st);
 void launch_pack_spinor(const double2* canon, void* native, int prec, const Geom& g, cudaStream_t st);
 // out_canon = b_canon (if given) + (g5 ? gamma5 : 1) * native
@@ -133,11 +133,14 @@ void launch_adf_normalize(float4* t, double2* x64, const KState* ks, size_t n, c
 // y += sum_{l < kused} c_l V_l; cdf: kmax float4 scratch
 // delayed CGS2 (low-synch Arnoldi, csrc/arnoldi_df.cu): h1[l] = V_l^dag x1, h2[l] = V_l^dag x2 for l < nvec in
 // one sweep (x1 double-float, x2 FP64); the step's scalar work; the fused update of v_j and u_{j+1}
+// (h1d, h2d: the double-float splits of h1, h2; H, ks: column nvec - 2 is finished and the scalars of the
+// update set by the last block; counter: a ticket, zero between uses); the scalar work alone (fin = 1, 2)
 void launch_adf_dot2(const float4* V, size_t ld, int nvec, const float4* x1, const double2* x2, double2* h1,
-                     double2* h2, double* partials, size_t n, int num_sms, const KState* ks, cudaStream_t st);
-void launch_adf_dcgs(double2* H, int ldH, const double2* h1, const double2* h2, float4* cdf, float4* qdf, KState* ks,
-                     int j, int fin, cudaStream_t st);
-void launch_adf_update2(const float4* V, size_t ld, int j, const float4* cdf, const float4* qdf, float4* uj,
+                     double2* h2, float4* h1d, float4* h2d, double2* H, int ldH, double* partials,
+                     unsigned int* counter, size_t n, int num_sms, KState* ks, cudaStream_t st);
+void launch_adf_dcgs(double2* H, int ldH, const double2* h1, const double2* h2, KState* ks, int j, int fin,
+                     cudaStream_t st);
+void launch_adf_update2(const float4* V, size_t ld, int j, const float4* cdf, const float4* ddf, float4* uj,
                         float4* unext, const double2* w, double2* x64, double2* H, int ldH, const double2* h1,
                         const double2* h2, size_t n, KState* ks, cudaStream_t st);
 // restarted Arnoldi (csrc/arnoldi_df.cu): cycle bookkeeping, the cycle's combination y += V c[off ..] and the next
