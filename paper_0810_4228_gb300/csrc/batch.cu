@@ -29,6 +29,11 @@
 #include <string>
 #include <vector>
 
+// Two-sided Lanczos passes near a breakdown for about one source in a hundred, and the result at a given k
+// then hangs on pass 1's roundings: between two orders of the FP32 products such a source's results differ by
+// 1e-9 to 1e-4 where all others agree to 1e-13.  A batch holds many sources, so its FP32 pass keeps the rounding
+// that it always had (chained multiply-adds would take 2 % off a batch of 48).
+#define OVL_F32_PRODUCTS_FIRST 1
 #include "ctx.h"
 #include "stencil_impl.cuh"
 

@@ -59,6 +59,17 @@ template <class R> OVL_HD void cfmac(cx<R>& a, cx<R> b, cx<R> c) {
     a.r = mad(b.i, c.i, mad(b.r, c.r, a.r));
     a.i = mad(-b.i, c.r, mad(b.r, c.i, a.i));
 }
+#ifdef OVL_F32_PRODUCTS_FIRST
+// The same with b c (or conj(b) c) formed first and added then, as batch.cu wants its FP32 products rounded.
+OVL_HD void cfma(cx<float>& a, cx<float> b, cx<float> c) {
+    a.r += b.r * c.r - b.i * c.i;
+    a.i += b.r * c.i + b.i * c.r;
+}
+OVL_HD void cfmac(cx<float>& a, cx<float> b, cx<float> c) {
+    a.r += b.r * c.r + b.i * c.i;
+    a.i += b.r * c.i - b.i * c.r;
+}
+#endif
 OVL_HD cx<double> up(cx<float> a) { return mk<double>(a.r, a.i); }
 OVL_HD cx<double> up(cx<double> a) { return a; }
 OVL_HD cx<double> d2c(double2 a) { return mk(a.x, a.y); }
