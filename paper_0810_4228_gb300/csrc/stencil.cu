@@ -23,12 +23,13 @@
 
 namespace ovl {
 
-__device__ __forceinline__ int site_of_thread(const Geom& g) {
+__device__ __forceinline__ int site_of_block(const Geom& g, int block) {
     const int half = blockDim.x >> 1;
     const int par = threadIdx.x >= half;
-    const int cb = blockIdx.x * half + (threadIdx.x - par * half);
+    const int cb = block * half + (threadIdx.x - par * half);
     return cb < g.Vh ? par * g.Vh + cb : -1;
 }
+__device__ __forceinline__ int site_of_thread(const Geom& g) { return site_of_block(g, blockIdx.x); }
 
 int dslash_grid(const Geom& g, int threads) { return (g.Vh + threads / 2 - 1) / (threads / 2); }
 
@@ -250,7 +251,7 @@ __global__ void __launch_bounds__(128) k_dslash_regen_ds(const double2* __restri
 static size_t ds_smem(int bytes_per_cx, int nin) { return (size_t)4 * nin * DS_SITES * 12 * bytes_per_cx; }
 static int ds_grid(const Geom& g) { return (g.V + DS_SITES - 1) / DS_SITES; }
 
-// one thread per site fills the GPU from about this many sites up
+// one thread per site fills the GPU with the FP64 regeneration step from about this many sites up
 static bool use_ds(const Geom& g) { return g.V < 152 * 1024; }
 
 // ------------------------------------------------------------ single apply --
@@ -383,7 +384,10 @@ void launch_dslash(const void* U, int prec, const void* x, void* y, double mu, d
         launch_hl<false>((const double2*)U, (const double2*)x, (double2*)y, mu, kappa, gamma5, g, st, ks);
         return;
     }
-    if (pick_ds(g)) {
+    // FP32: one thread per site is the faster form from about 2^15 sites (measured, 12-real / 18-real links:
+    // 20736 sites 6.4 / 6.7 us against 6.3 / 6.2 split, 36864 7.6 / 8.3 against 8.3 / 8.3, 65536 8.5 / 8.7 against
+    // 10.3 / 10.4, 276480 28.5 / 32.9 against 32.9 / 45.2)
+    if (g_ds_mode < 0 ? g.V < (1 << 15) : g_ds_mode == 1) {
         if (prec == 0)
             k_dslash_ds<LINK_F64><<<ds_grid(g), 128, ds_smem(16, 1), st>>>(U, (const double2*)x, (double2*)y,
                                                                           make_coef<double>(mu, kappa), gamma5, ks, g);
@@ -426,9 +430,11 @@ void launch_dslash(const void* U, int prec, const void* x, void* y, double mu, d
 // t = sv * gamma5 D_w(mu) v~,  s = sw * gamma5 D_w(-mu) w~,  alpha[step] = w^dag t
 // with w = sw w~.  Skipped (uniformly) once the solve is done or failed.
 // The two stencils go to two sets of blocks (which = 0: t and the alpha partials; 1: s), so a thread
-// carries one accumulator spinor (half the registers: more warps per SM); which is blockIdx.y on a
-// one-dimensional grid, the low bit of blockIdx.x on the row-grouped grid.  Only the t blocks take
-// part in the reduction.
+// carries one accumulator spinor (half the registers: more warps per SM); which is the low bit of
+// blockIdx.x, so that both find the links in L2.  Only the t blocks take part in the reduction.
+// Both kinds of block run the same copy of the stencil (34 KB of instructions): with a copy each, warps of
+// the two kinds on one SM waited for instructions a quarter of the time (32^4, FP32: 296 -> 230 us; 48^3 x 64:
+// 1843 -> 1387 us).  Bound by issue slots and load latency, at 2.8 TB/s of its own operands.
 template <int LF, bool ROWS>
 __global__ void __launch_bounds__(128, LF == LINK_F64 ? 2 : OVL_DSLASH_F32_MINB) k_dslash_pair(const void* __restrict__ U,
                                                      const typename VecT<typename LinkReal<LF>::R>::T* __restrict__ v,
@@ -443,48 +449,39 @@ __global__ void __launch_bounds__(128, LF == LINK_F64 ? 2 : OVL_DSLASH_F32_MINB)
     __shared__ double red[3 * 32];  // grid_sum_last<3>: 32 doubles per value
     if (ks->done || ks->status) return;
     const double2 sv = ks->sv, sw = ks->sw;
-    const int which = ROWS ? (int)(blockIdx.x & 1u) : (int)blockIdx.y;
-    const int i = ROWS ? site_of_rows(g, blockIdx.x >> 1, gridDim.x >> 1) : site_of_thread(g);
-    if (which == 1) {  // s = sw A^dag w~
-        if (i >= 0) {
-            const typename VecT<R>::T* const xs[1] = {w};
-            Spinor<R> acc[1], self;
-            const HopCoef<R> hcs[1] = {hw};
-            apply_site<LF, R, 1>(g, i, U, xs, acc, hcs);
-            load_spinor(w, g.V, i, self);
-            finish_site(acc[0], self, true);
-            const cx<R> csw = mk(R(sw.x), R(sw.y));
-#pragma unroll
-            for (int sp = 0; sp < 4; ++sp)
-#pragma unroll
-                for (int a = 0; a < 3; ++a) acc[0].s[sp][a] = csw * acc[0].s[sp][a];
-            store_spinor(s, g.V, i, acc[0]);
-        }
-        return;
-    }
+    const int which = (int)(blockIdx.x & 1u);
+    const int i = ROWS ? site_of_rows(g, blockIdx.x >> 1, gridDim.x >> 1) : site_of_block(g, blockIdx.x >> 1);
     // per-thread sums: FP64 for FP64 data; for FP32 data exact FP32 products summed as compensated
     // FP32 pairs (TwoSum) on the FP32 pipe, widened to FP64 for the block and grid sums
     using A = typename std::conditional<sizeof(R) == 4, AccF, AccD>::type;
     A pa[3];
-    if (i >= 0) {  // t = sv A v~, partials of w~^dag t and |t|^2
-        const typename VecT<R>::T* const xs[1] = {v};
+    if (i >= 0) {  // t = sv A v~, partials of w~^dag t and |t|^2; or s = sw A^dag w~
+        const typename VecT<R>::T* const xs[1] = {which ? w : v};
         Spinor<R> acc[1], self;
-        const HopCoef<R> hcs[1] = {hv};
+        HopCoef<R> hcs[1] = {hv};
+        hcs[0].f[3] = which ? hw.f[3] : hv.f[3];
+        hcs[0].b[3] = which ? hw.b[3] : hv.b[3];
         apply_site<LF, R, 1>(g, i, U, xs, acc, hcs);
-        load_spinor(v, g.V, i, self);
+        load_spinor(xs[0], g.V, i, self);
         finish_site(acc[0], self, true);
-        load_spinor(w, g.V, i, self);
-        const cx<R> csv = mk(R(sv.x), R(sv.y));
+        const cx<R> cs = which ? mk(R(sw.x), R(sw.y)) : mk(R(sv.x), R(sv.y));
 #pragma unroll
         for (int sp = 0; sp < 4; ++sp)
 #pragma unroll
-            for (int a = 0; a < 3; ++a) {
-                acc[0].s[sp][a] = csv * acc[0].s[sp][a];
-                acc_cdot(pa, self.s[sp][a], acc[0].s[sp][a]);  // w~^dag t
-                acc_norm2(pa[2], acc[0].s[sp][a]);
-            }
-        store_spinor(t, g.V, i, acc[0]);
+            for (int a = 0; a < 3; ++a) acc[0].s[sp][a] = cs * acc[0].s[sp][a];
+        store_spinor(which ? s : t, g.V, i, acc[0]);
+        if (!which) {
+            load_spinor(w, g.V, i, self);
+#pragma unroll
+            for (int sp = 0; sp < 4; ++sp)
+#pragma unroll
+                for (int a = 0; a < 3; ++a) {
+                    acc_cdot(pa, self.s[sp][a], acc[0].s[sp][a]);  // w~^dag t
+                    acc_norm2(pa[2], acc[0].s[sp][a]);
+                }
+        }
     }
+    if (which) return;
     double part[3];
 #pragma unroll
     for (int j = 0; j < 3; ++j) {
@@ -492,8 +489,7 @@ __global__ void __launch_bounds__(128, LF == LINK_F64 ? 2 : OVL_DSLASH_F32_MINB)
         else part[j] = pa[j].v;
     }
     double out[3];
-    const unsigned nx = ROWS ? gridDim.x >> 1 : gridDim.x;
-    const unsigned bx = ROWS ? blockIdx.x >> 1 : blockIdx.x;
+    const unsigned nx = gridDim.x >> 1, bx = blockIdx.x >> 1;
     const unsigned blk = ROWS ? bx + nx * (blockIdx.y + gridDim.y * blockIdx.z) : bx;
     const unsigned nblk = ROWS ? nx * gridDim.y * gridDim.z : nx;
     if (grid_sum_last<3>(part, partials, counter, out, red, blk, nblk)) {
@@ -509,13 +505,19 @@ __global__ void __launch_bounds__(128, LF == LINK_F64 ? 2 : OVL_DSLASH_F32_MINB)
     }
 }
 
-int dslash_pair_blocks(const Geom& g) { return pick_ds(g) ? ds_grid(g) : dslash_grid(g, 128); }
+// The pair's two stencils run in one launch, so one thread per site and stencil is the faster form from few
+// sites on (us of the call, FP32 / FP64, against the direction split: 4096 sites 30.6 / 66.7 against 31.0 / 48.2,
+// 8748 31.1 / 67.7 against 34.7 / 67.7, 20736 34.8 / 130 against 52.9 / 131, 65536 43.8 / 270 against 80.3 / 308).
+// The FP32 form sums alpha in compensated pairs (48 bits; the FP32 rounding of t itself, which both forms share,
+// is what alpha's error is made of).
+static bool pair_ds(const Geom& g) { return g_ds_mode < 0 ? g.V < (1 << 13) : g_ds_mode == 1; }
+int dslash_pair_blocks(const Geom& g) { return pair_ds(g) ? ds_grid(g) : dslash_grid(g, 128); }
 
 void launch_dslash_pair(const void* U, int prec, const void* v, const void* w, void* t, void* s, double mu,
                         double kappa, KState* ks, double2* alpha, int step, int klast, double* partials,
                         unsigned int* counter, const Geom& g, cudaStream_t st) {
     const int B = dslash_pair_blocks(g);  // the partial-sum slots the fused reduction writes
-    if (pick_ds(g)) {
+    if (pair_ds(g)) {
         static unsigned long long attr_dev = 0;
         if (first_use_on_device(attr_dev))
             cudaFuncSetAttribute(k_dslash_pair_ds<LINK_F64>, cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -535,7 +537,7 @@ void launch_dslash_pair(const void* U, int prec, const void* v, const void* w, v
     const int T = 128;
     RowGrid rg = row_grid(g, T);
     rg.grid.x *= 2;  // the two stencils
-    const dim3 g1(B, 2);
+    const dim3 g1(2 * B);
     if (prec == 0) {
         if (rg.ok)
             k_dslash_pair<LINK_F64, true><<<rg.grid, T, 0, st>>>(
