@@ -68,6 +68,8 @@ struct BSeq {
     double2* gamma;
     double2* cvec;
     double2* vscale;
+    double2* cf;              // recurrence coefficients of the step: alpha sv, conj(alpha) sw, gamma_{i-1} svp,
+                              // conj(beta_{i-1}) swp
     double2* part;            // [nblk][4] block partials of the batched kernels
     unsigned int* cnt;        // ticket of this sequence
     int blk0[3], nblk[3];     // block range in the pass-1 launches, per site-block shape (64, 128, 256 sites)
@@ -123,7 +125,7 @@ __device__ __forceinline__ AccD acc_load(double2 v, AccD) {
 // Per-sequence reduction of NQ accumulators (in their own arithmetic: compensated FP32 pairs for FP32
 // data, FP64 otherwise): warp trees, the block's warps in a fixed order into part[local], then the
 // last block of the sequence (ticket) adds the partials of its nblk blocks in a fixed order.
-// Returns true in the last block; out[] (FP64) is valid in thread 0 there.
+// Returns true in the last block; out[] (FP64) is valid in every lane of warp 0 there.
 template <int NQ, int NW, class A>
 __device__ bool seq_reduce(A (&v)[NQ], double2* part, unsigned int* cnt, int local, int nblk, double (&out)[NQ]) {
     __shared__ double2 red[NQ][NW];
@@ -162,11 +164,55 @@ __device__ bool seq_reduce(A (&v)[NQ], double2* part, unsigned int* cnt, int loc
         if (lane == 0) red[qv][0] = acc_store(acc);
     }
     __syncthreads();
-    if (threadIdx.x == 0) {
-        for (int q = 0; q < NQ; ++q) out[q] = red[q][0].x + red[q][0].y;
-        *cnt = 0u;
+    if (wid == 0) {
+        const double2 r = red[lane < NQ ? lane : 0][0];
+        const double s = r.x + r.y;
+#pragma unroll
+        for (int q = 0; q < NQ; ++q) out[q] = __shfl_sync(0xffffffffu, s, q);
+        if (lane == 0) *cnt = 0u;
     }
     return true;
+}
+
+// ---- the scalars of a step, by one warp (every lane gets the sums).  An FP64 instruction takes 64 cycles of
+// its warp however few lanes take part, a library division 430 and a square root 680, and these chains are
+// the tail of every step: real and imaginary parts go to lanes side by side, and the norms, their
+// reciprocals and the divisions come from one reciprocal square root.
+__device__ __forceinline__ double flip_sign(double x) {
+    return __hiloint2double(__double2hiint(x) ^ (int)0x80000000u, __double2loint(x));
+}
+// alpha = conj(sw) w~^dag t from (re, im) = w~^dag t (sv is real): even lanes return its real part, odd lanes
+// its imaginary part; r: lanes 0, 1 conj(alpha) sw, lanes 2, 3 alpha sv
+__device__ __forceinline__ double alpha_scalars(double re, double im, double svr, double swr, double swi, double& r) {
+    const int lane = threadIdx.x & 31;
+    const bool q = lane & 1, first = lane < 2;
+    const double al = fma(swr, q ? im : re, swi * (q ? flip_sign(re) : im));
+    const double ao = __shfl_xor_sync(0xffffffffu, al, 1);
+    const double ar = q ? ao : al, ai = q ? al : ao;
+    const double m1 = first ? (q ? swi : swr) : svr, m2 = first ? (q ? flip_sign(swr) : swi) : 0.0;
+    r = fma(first ? ar : al, m1, ai * m2);
+    return al;
+}
+// beta = |v^|, gamma = delta / beta, sv' = 1 / beta, sw' = 1 / conj(gamma) = delta beta / |delta|^2 from
+// delta = (re, im) and nv2 = |v^|^2: nv, rnv in every lane, g: lanes 0, 1 gamma, lanes 2, 3 sw';
+// cn: lanes 0, 1 gamma sv, lanes 2, 3 beta sw (the next step's coefficients of the previous vectors)
+__device__ __forceinline__ void beta_scalars(double re, double im, double nv2, double svr, double swr, double swi,
+                                             double& nv, double& rnv, double& g, double& cn) {
+    const int lane = threadIdx.x & 31;
+    const bool q = lane & 1;
+    const double nd2 = fma(im, im, re * re);
+    const double r = rsqrt(q ? nd2 : nv2);  // even lanes 1 / |v^|, odd lanes 1 / |delta|
+    const double r2 = r * (q ? r : nv2);    // |v^|, 1 / |delta|^2
+    rnv = __shfl_sync(0xffffffffu, r, 0);
+    nv = __shfl_sync(0xffffffffu, r2, 0);
+    const double f = nv * __shfl_sync(0xffffffffu, r2, 1);
+    g = (q ? im : re) * (lane < 2 ? rnv : f);
+    cn = (lane < 2 ? g : nv) * (lane < 2 ? svr : (q ? swi : swr));
+}
+// lucky (1) or serious (2) breakdown from the squared norms; an2: largest |A v_i|^2 so far
+__device__ __forceinline__ int breakdown(double re, double im, double nv2, double nw2, double an2) {
+    if (nv2 <= 1e-26 * fmax(an2, 1e-300)) return 1;  // |v^| <= 1e-13 max |A v_i|
+    return fma(im, im, re * re) <= 1e-28 * nv2 * nw2 ? 2 : 0;  // |w^^dag v^| <= 1e-14 |v^| |w^|
 }
 
 // Programmatic dependent launch: the batched kernels of one solve follow each other on one
@@ -237,12 +283,17 @@ __global__ void __launch_bounds__(SHAPE_SITES[SH], LF == LINK_F64 ? 1 : 768 / SH
     }
     if (second) return;
     double o[3];
-    if (seq_reduce<3, BT / 32>(a, q.part, q.cnt, local, q.nblk[SH], o) && threadIdx.x == 0) {
-        const cx<double> alpha = cdot(d2c(ks->sw), mk(o[0], o[1]));  // conj(sw) w~^dag t
-        q.alpha[i] = c2d(alpha);
-        ks->anorm = fmax(ks->anorm, sqrt(o[2]));
-        ks->kused = i + 1;
-        if (i >= klast) ks->done = 1;
+    if (seq_reduce<3, BT / 32>(a, q.part, q.cnt, local, q.nblk[SH], o) && threadIdx.x < 32) {
+        const int lane = threadIdx.x;
+        double r;
+        const double al = alpha_scalars(o[0], o[1], ks->sv.x, ks->sw.x, ks->sw.y, r);
+        if (lane < 4) reinterpret_cast<double*>(q.cf + (lane < 2 ? 1 : 0))[lane & 1] = r;
+        if (lane < 2) reinterpret_cast<double*>(q.alpha + i)[lane] = al;
+        if (lane == 0) {
+            ks->red[0].x = fmax(ks->red[0].x, o[2]);  // max |A v_i|^2
+            ks->kused = i + 1;
+            if (i >= klast) ks->done = 1;
+        }
     }
 }
 
@@ -280,15 +331,9 @@ __global__ void __launch_bounds__(SHAPE_SITES[SH], sizeof(R) == 4 ? 1536 / SHAPE
     pdl_wait_and_release();
     if (ks->done || ks->status) return;
     __shared__ cx<R> cf[4];
-    if (threadIdx.x == 0) {
-        const cx<double> a = d2c(q.alpha[i]);
-        const cx<double> ca = a * d2c(ks->sv), da = conj(a) * d2c(ks->sw);
-        const cx<double> cg = i > 0 ? d2c(q.gamma[i - 1]) * d2c(ks->svp) : mk(0.0, 0.0);
-        const cx<double> db = i > 0 ? conj(d2c(q.beta[i - 1])) * d2c(ks->swp) : mk(0.0, 0.0);
-        cf[0] = mk((R)ca.r, (R)ca.i);
-        cf[1] = mk((R)da.r, (R)da.i);
-        cf[2] = mk((R)cg.r, (R)cg.i);
-        cf[3] = mk((R)db.r, (R)db.i);
+    if (threadIdx.x < 4) {
+        const double2 c = q.cf[threadIdx.x];
+        cf[threadIdx.x] = mk((R)c.x, (R)c.y);
     }
     __syncthreads();
     constexpr int BT = SHAPE_SITES[SH];
@@ -337,23 +382,28 @@ __global__ void __launch_bounds__(SHAPE_SITES[SH], sizeof(R) == 4 ? 1536 / SHAPE
         }
     }
     double o[4];
-    if (seq_reduce<4, BT / 32>(a, q.part, q.cnt, local, q.nblk[SH], o) && threadIdx.x == 0) {
-        const double nv = sqrt(o[2]), nw = sqrt(o[3]);
-        const cx<double> delta = mk(o[0], o[1]);
-        if (nv <= 1e-13 * fmax(ks->anorm, 1e-300)) {
-            ks->done = 1;  // lucky breakdown
-        } else if (sqrt(norm2(delta)) <= 1e-14 * nv * nw) {
-            ks->done = 1;  // serious breakdown
-            ks->bdstep = i + 1;
+    if (seq_reduce<4, BT / 32>(a, q.part, q.cnt, local, q.nblk[SH], o) && threadIdx.x < 32) {
+        const int lane = threadIdx.x;
+        const int bk = breakdown(o[0], o[1], o[2], o[3], ks->red[0].x);
+        if (bk) {
+            if (lane == 0) {
+                ks->done = 1;
+                if (bk == 2) ks->bdstep = i + 1;
+            }
         } else {
-            const cx<double> gm = mk(o[0] / nv, o[1] / nv);
-            q.beta[i] = make_double2(nv, 0.0);
-            q.gamma[i] = c2d(gm);
-            ks->svp = ks->sv;
-            ks->swp = ks->sw;
-            ks->sv = make_double2(1.0 / nv, 0.0);
-            ks->sw = c2d(cdiv(mk(1.0, 0.0), conj(gm)));
-            q.vscale[i + 1] = ks->sv;
+            const double2 sv = ks->sv, sw = ks->sw;
+            double nv, rnv, g, cn;
+            beta_scalars(o[0], o[1], o[2], sv.x, sw.x, sw.y, nv, rnv, g, cn);
+            __syncwarp();
+            if (lane < 2) reinterpret_cast<double*>(q.gamma + i)[lane] = g;
+            else if (lane < 4) reinterpret_cast<double*>(&ks->sw)[lane & 1] = g;
+            if (lane < 4) reinterpret_cast<double*>(q.cf + 2)[lane] = cn;
+            if (lane == 0) {
+                q.beta[i] = make_double2(nv, 0.0);
+                ks->svp = sv;
+                ks->swp = sw;
+                ks->sv = q.vscale[i + 1] = make_double2(rnv, 0.0);
+            }
         }
     }
 }
@@ -420,12 +470,6 @@ __device__ __forceinline__ void bp1_seq_sum(const double2* part, int nblk, doubl
 
 __device__ __forceinline__ cx<float> f32c(cx<double> z) { return mk((float)z.r, (float)z.i); }
 
-struct BP1Scalars {
-    cx<double> sv, sw, svp, swp, beta_prev, gamma_prev;
-    double anorm;
-    int kused, bd;
-};
-
 template <int LF>
 __global__ void __launch_bounds__(BP1_T, 3) k_bp1(BP1Args a) {
     const int sidx = a.bseq[blockIdx.x];
@@ -444,16 +488,19 @@ __global__ void __launch_bounds__(BP1_T, 3) k_bp1(BP1Args a) {
     int* err = &ks->timeout;
     double2* partA = q.part;
     double2* partC = q.part + (size_t)nblk * 4;
-    // recurrence scalars in FP64, meaningful in thread 0 (identical in every block of the sequence)
-    // recurrence scalars in FP64, used by thread 0 only (shared: no registers in the other threads)
-    __shared__ BP1Scalars sc;
+    // recurrence scalars in FP64 (identical in every block of the sequence; sv is real), in shared memory: no
+    // registers between the uses
+    __shared__ double sc[7];             // sv, sw (re, im), svp, swp (re, im); max |A v_i|^2
+    __shared__ int steps[2];             // steps taken, step of a serious breakdown
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     if (threadIdx.x == 0) {
-        sc.sv = d2c(ks->sv), sc.sw = d2c(ks->sw), sc.svp = d2c(ks->svp), sc.swp = d2c(ks->swp);
-        sc.beta_prev = mk(0.0, 0.0), sc.gamma_prev = mk(0.0, 0.0);
-        sc.anorm = ks->anorm;
-        sc.kused = 0, sc.bd = -1;
-        cs[0] = f32c(sc.sv);
-        cs[1] = f32c(sc.sw);
+        sc[0] = ks->sv.x, sc[1] = ks->sw.x, sc[2] = ks->sw.y;
+        sc[3] = ks->svp.x, sc[4] = ks->swp.x, sc[5] = ks->swp.y;
+        sc[6] = ks->anorm * ks->anorm;
+        steps[0] = 0, steps[1] = -1;
+        cs[0] = mk((float)sc[0], 0.f);
+        cs[1] = mk((float)sc[1], (float)sc[2]);
+        cc[2] = cc[3] = mk(0.f, 0.f);
     }
     __syncthreads();
     unsigned int nb = 0;
@@ -489,15 +536,14 @@ __global__ void __launch_bounds__(BP1_T, 3) k_bp1(BP1Args a) {
         grid_barrier_mono(bar, (unsigned)nblk * (++nb), err, 1, BP1_SPIN);
         if (*(volatile int*)err) return;
         bp1_seq_sum<3>(partA, nblk, osum);
-        if (threadIdx.x == 0) {
-            const cx<double> alpha = cdot(sc.sw, mk(osum[0], osum[1]));  // conj(sw) w~^dag t
-            sc.anorm = fmax(sc.anorm, sqrt(osum[2]));
-            sc.kused = i + 1;
-            if (local == 0) q.alpha[i] = c2d(alpha);
-            cc[0] = f32c(alpha * sc.sv);
-            cc[1] = f32c(conj(alpha) * sc.sw);
-            cc[2] = f32c(i > 0 ? sc.gamma_prev * sc.svp : mk(0.0, 0.0));
-            cc[3] = f32c(i > 0 ? conj(sc.beta_prev) * sc.swp : mk(0.0, 0.0));
+        if (wid == 0) {
+            double r;
+            const double al = alpha_scalars(osum[0], osum[1], sc[0], sc[1], sc[2], r);
+            if (lane < 4) reinterpret_cast<float*>(cc + (lane < 2 ? 1 : 0))[lane & 1] = (float)r;
+            if (local == 0 && lane < 2) reinterpret_cast<double*>(q.alpha + i)[lane] = al;
+        } else if (threadIdx.x == 32) {
+            sc[6] = fmax(sc[6], osum[2]);
+            steps[0] = i + 1;
         }
         if (i == a.k - 1) break;
         __syncthreads();
@@ -535,45 +581,46 @@ __global__ void __launch_bounds__(BP1_T, 3) k_bp1(BP1Args a) {
         grid_barrier_mono(bar, (unsigned)nblk * (++nb), err, 1, BP1_SPIN);
         if (*(volatile int*)err) return;
         bp1_seq_sum<4>(partC, nblk, osum);
-        if (threadIdx.x == 0) {
-            const double nv = sqrt(osum[2]), nw = sqrt(osum[3]);
-            const cx<double> delta = mk(osum[0], osum[1]);
-            int dn = 0;
-            if (nv <= 1e-13 * fmax(sc.anorm, 1e-300)) {
-                dn = 1;  // lucky breakdown
-            } else if (sqrt(norm2(delta)) <= 1e-14 * nv * nw) {
-                dn = 1;  // serious breakdown
-                sc.bd = i + 1;
-            } else {
-                const cx<double> gm = mk(osum[0] / nv, osum[1] / nv);
-                sc.beta_prev = mk(nv, 0.0);
-                sc.gamma_prev = gm;
-                sc.svp = sc.sv;
-                sc.swp = sc.sw;
-                sc.sv = mk(1.0 / nv, 0.0);
-                sc.sw = cdiv(mk(1.0, 0.0), conj(gm));
-                if (local == 0) {
-                    q.beta[i] = make_double2(nv, 0.0);
-                    q.gamma[i] = c2d(gm);
-                    q.vscale[i + 1] = c2d(sc.sv);
-                }
-                cs[0] = f32c(sc.sv);
-                cs[1] = f32c(sc.sw);
+        double nv = 0.0, rnv = 0.0, g = 0.0, cn = 0.0;
+        if (wid == 0) {
+            beta_scalars(osum[0], osum[1], osum[2], sc[0], sc[1], sc[2], nv, rnv, g, cn);
+        } else if (wid == 1) {
+            const int bk = breakdown(osum[0], osum[1], osum[2], osum[3], sc[6]);
+            if (lane == 0) {
+                sdone = bk;
+                if (bk == 2) steps[1] = i + 1;
             }
-            sdone = dn;
         }
         __syncthreads();
         if (sdone) break;
+        if (wid == 0) {
+            const double swr = __shfl_sync(0xffffffffu, g, 2), swi = __shfl_sync(0xffffffffu, g, 3);
+            if (lane < 4) reinterpret_cast<float*>(cc + 2)[lane] = (float)cn;
+            if (lane == 0) {
+                sc[3] = sc[0], sc[4] = sc[1], sc[5] = sc[2];
+                sc[0] = rnv, sc[1] = swr, sc[2] = swi;
+                cs[0] = mk((float)rnv, 0.f);
+                cs[1] = mk((float)swr, (float)swi);
+            }
+            if (local == 0) {
+                if (lane < 2) reinterpret_cast<double*>(q.gamma + i)[lane] = g;
+                if (lane == 0) {
+                    q.beta[i] = make_double2(nv, 0.0);
+                    q.vscale[i + 1] = make_double2(rnv, 0.0);
+                }
+            }
+        }
+        __syncthreads();
     }
-    if (local == 0 && threadIdx.x == 0) {
-        ks->kused = sc.kused;
+    if (local == 0 && threadIdx.x == 32) {
+        ks->sv = make_double2(sc[0], 0.0);
+        ks->sw = make_double2(sc[1], sc[2]);
+        ks->svp = make_double2(sc[3], 0.0);
+        ks->swp = make_double2(sc[4], sc[5]);
+        ks->kused = steps[0];
         ks->done = 1;
-        ks->anorm = sc.anorm;
-        if (sc.bd >= 0) ks->bdstep = sc.bd;
-        ks->sv = c2d(sc.sv);
-        ks->sw = c2d(sc.sw);
-        ks->svp = c2d(sc.svp);
-        ks->swp = c2d(sc.swp);
+        ks->anorm = sqrt(sc[6]);
+        if (steps[1] >= 0) ks->bdstep = steps[1];
     }
 }
 
@@ -1230,7 +1277,7 @@ int balloc(ovl_batch* b, int mode, int kmax) {
         const size_t need = std::max<size_t>((size_t)2 * std::max(c->m, 1) * ovl::multidot_blocks(c->n), 2048);
         pro_off[s + 1] = pro_off[s] + ((need + 31) & ~(size_t)31);
     }
-    total += al(ns * sizeof(ovl::KState)) + 5 * al(ns * kk * sizeof(double2)) +
+    total += al(ns * sizeof(ovl::KState)) + 5 * al(ns * kk * sizeof(double2)) + al(ns * 4 * sizeof(double2)) +
              al((size_t)ns * inner_stride * sizeof(double2)) + al((size_t)ns * qpart_stride * sizeof(double)) +
              al(ns * 64 * sizeof(unsigned int)) + al(ns * sizeof(ovl::BSeq)) + al(nblocks[0] * sizeof(int)) +
              al(nblocks[1] * sizeof(int)) + al(nblocks[2] * sizeof(int)) +
@@ -1250,6 +1297,7 @@ int balloc(ovl_batch* b, int mode, int kmax) {
     b->gamma = (double2*)take(ns * kk * sizeof(double2));
     b->cvec = (double2*)take(ns * kk * sizeof(double2));
     b->vscale = (double2*)take(ns * kk * sizeof(double2));
+    double2* cf = (double2*)take(ns * 4 * sizeof(double2));
     b->inner = (double2*)take((size_t)ns * inner_stride * sizeof(double2));
     b->inner_stride = inner_stride;
     b->qpart = (double*)take((size_t)ns * qpart_stride * sizeof(double));
@@ -1313,6 +1361,7 @@ int balloc(ovl_batch* b, int mode, int kmax) {
         q.gamma = b->gamma + s * kk;
         q.cvec = b->cvec + s * kk;
         q.vscale = b->vscale + s * kk;
+        q.cf = cf + 4 * s;
         for (int h = 0; h < ovl::NSHAPE; ++h) q.nblk[h] = (c->g.V + ovl::SHAPE_SITES[h] - 1) / ovl::SHAPE_SITES[h];
         q.part = (double2*)take((size_t)std::max(q.nblk[0], 2 * q.nblk[1]) * 4 * sizeof(double2));
         b->pq[s] = (double2*)take(128 * sizeof(double2));
