@@ -23,6 +23,9 @@
 // count arrivals on a counter zeroed before each launch.
 #include <algorithm>
 
+// pass 1 keeps the rounding that its FP32 products always had, as batch.cu says (a chained multiply-add would
+// take 1.7 % off an 8^4 solve)
+#define OVL_F32_PRODUCTS_FIRST 1
 #include "stencil_impl.cuh"
 
 namespace ovl {
@@ -158,6 +161,49 @@ __device__ __forceinline__ void warp_sum_partials(const float2* part, int stride
     __syncwarp();
 }
 
+// Called by one full warp: the sums over blocks b < G of the four pairs part[b * stride + q], in a fixed order
+// (identical in every block), rounded to FP64 at the end and valid in every lane.  Each lane loads its
+// blocks' pairs at once (one L2 round trip up to 160 blocks); the warp sum is transposed (6 pair additions).
+__device__ __forceinline__ void warp_sum4_partials(const float2* part, int stride, int G, double (&o)[4]) {
+    const int lane = threadIdx.x & 31;
+    ff s[4] = {{0.f, 0.f}, {0.f, 0.f}, {0.f, 0.f}, {0.f, 0.f}};
+    for (int b0 = lane; b0 < G; b0 += 160) {
+        float4 x[5][2];
+#pragma unroll
+        for (int u = 0; u < 5; ++u) {
+            const bool ok = b0 + 32 * u < G;
+            const float4* p = reinterpret_cast<const float4*>(part + (size_t)(ok ? b0 + 32 * u : b0) * stride);
+            x[u][0] = __ldcg(p);
+            x[u][1] = __ldcg(p + 1);
+        }
+#pragma unroll
+        for (int u = 0; u < 5; ++u)
+            if (b0 + 32 * u < G) {
+                s[0] = ff_add(s[0], ff{x[u][0].x, x[u][0].y});
+                s[1] = ff_add(s[1], ff{x[u][0].z, x[u][0].w});
+                s[2] = ff_add(s[2], ff{x[u][1].x, x[u][1].y});
+                s[3] = ff_add(s[3], ff{x[u][1].z, x[u][1].w});
+            }
+    }
+    auto xchg = [](ff a, int m) {
+        return ff{__shfl_xor_sync(0xffffffffu, a.hi, m), __shfl_xor_sync(0xffffffffu, a.lo, m)};
+    };
+    const bool u16 = lane & 16, u8 = lane & 8;
+    const ff p = ff_add(u16 ? s[2] : s[0], xchg(u16 ? s[0] : s[2], 16));
+    const ff q = ff_add(u16 ? s[3] : s[1], xchg(u16 ? s[1] : s[3], 16));
+    ff r = ff_add(u8 ? q : p, xchg(u8 ? p : q, 8));
+    r = ff_add(r, xchg(r, 4));
+    r = ff_add(r, xchg(r, 2));
+    r = ff_add(r, xchg(r, 1));
+    const double d = (double)r.hi + (double)r.lo;
+#pragma unroll
+    for (int v = 0; v < 4; ++v) o[v] = __shfl_sync(0xffffffffu, d, 8 * v);
+}
+
+__device__ __forceinline__ double flip_sign(double x) {
+    return __hiloint2double(__double2hiint(x) ^ (int)0x80000000u, __double2loint(x));
+}
+
 __device__ __forceinline__ cx<float> down(cx<double> z) { return mk((float)z.r, (float)z.i); }
 
 struct P1Args {
@@ -204,7 +250,6 @@ __global__ void __launch_bounds__(32 * PW1) k_pass1_persistent(P1Args a) {
     cx<float>* st = dirpart + PW1 * 2 * PT * 12;                  // [tpb][3][2][PT][12]
     __shared__ float2 redf[PW1 * 4];
     __shared__ double coef[4 + 4 * PMAX_M];
-    __shared__ double oc[4];
     __shared__ P1Shared sh;
     KState* ks = a.ks;
     int* err = &ks->timeout;
@@ -216,9 +261,11 @@ __global__ void __launch_bounds__(32 * PW1) k_pass1_persistent(P1Args a) {
     const int site = tid >> 3, sp = (tid >> 1) & 3, vw = tid & 1;
     const int m = a.m;
     const int NA = 4 + 4 * m;
-    // recurrence state in FP64, meaningful in warp 0 lane 0
-    cx<double> sv = d2c(ks->sv), sw = d2c(ks->sw), svp = d2c(ks->svp), swp = d2c(ks->swp);
-    cx<double> beta_prev = mk(0.0, 0.0), gamma_prev = mk(0.0, 0.0);
+    // recurrence state in FP64: the scales in every lane of warp 0 (sv is real), what the breakdown checks
+    // need in warp 1.  An FP64 instruction takes 64 cycles of its warp: the real and imaginary parts of a
+    // step's scalars are formed by lanes side by side, and the checks run beside them (one lane doing all of
+    // it took 2 us of a 12 us step).
+    double svr = ks->sv.x, svpr = ks->svp.x, swr = ks->sw.x, swi = ks->sw.y, swpr = ks->swp.x, swpi = ks->swp.y;
     double anorm2 = ks->anorm * ks->anorm;
     int kused = 0, bd = -1;
     unsigned int nbar = 0;
@@ -239,8 +286,9 @@ __global__ void __launch_bounds__(32 * PW1) k_pass1_persistent(P1Args a) {
         }
     }
     if (tid == 0) {
-        sh.cs[0] = down(sv);
-        sh.cs[1] = down(sw);
+        sh.cs[0] = mk((float)svr, 0.f);
+        sh.cs[1] = mk((float)swr, (float)swi);
+        sh.cp[0] = sh.cp[1] = mk(0.f, 0.f);
         sh.done = 0;
     }
     __syncthreads();
@@ -318,25 +366,30 @@ __global__ void __launch_bounds__(32 * PW1) k_pass1_persistent(P1Args a) {
         if (*(volatile int*)err) return;
         // ---- scalars (warp 0): alpha_i, the recurrence coefficients of phase C
         if (wid == 0) {
-            warp_sum_partials(a.partA, NA, 3, G, coef);
+            double o[4];
+            warp_sum4_partials(a.partA, NA, G, o);
             if (m > 0) warp_sum_partials(a.partA + 4, NA, 4 * m, G, coef + 4);
-            if (lane == 0) {
-                const cx<double> alpha = cdot(sw, mk(coef[0], coef[1]));
-                anorm2 = fmax(anorm2, coef[2]);
-                kused = i + 1;
-                if (blockIdx.x == 0) a.alpha[i] = c2d(alpha);
-                sh.ca[0] = down(alpha * sv);
-                sh.ca[1] = down(conj(alpha) * sw);
-                sh.cp[0] = down(i > 0 ? gamma_prev * svp : mk(0.0, 0.0));
-                sh.cp[1] = down(i > 0 ? conj(beta_prev) * swp : mk(0.0, 0.0));
-            }
+            // alpha = conj(sw) w~^dag t: even lanes its real part, odd lanes its imaginary part
+            const bool q = lane & 1;
+            const double al = fma(swr, q ? o[1] : o[0], swi * (q ? flip_sign(o[0]) : o[1]));
+            const double ao = __shfl_xor_sync(0xffffffffu, al, 1);
+            // lanes 0, 1: conj(alpha) sw; lanes 2, 3: alpha sv
+            const double ar = q ? ao : al, ai = q ? al : ao;
+            const bool first = lane < 2;
+            const double m1 = first ? (q ? swi : swr) : svr, m2 = first ? (q ? flip_sign(swr) : swi) : 0.0;
+            const double r = fma(first ? ar : al, m1, ai * m2);
+            if (lane < 4) reinterpret_cast<float*>(sh.ca)[(first ? 2 : 0) + q] = (float)r;
+            if (blockIdx.x == 0 && lane < 2) reinterpret_cast<double*>(a.alpha + i)[lane] = al;
+            if (lane == 0) coef[2] = o[2];
             for (int j = lane; j < m; j += 32) {
                 sh.pq[0][j] = mk((float)coef[4 + 4 * j], (float)coef[4 + 4 * j + 1]);
                 sh.pq[1][j] = mk((float)coef[4 + 4 * j + 2], (float)coef[4 + 4 * j + 3]);
             }
         }
-        if (i == a.k - 1) break;
+        kused = i + 1;
         __syncthreads();
+        if (wid == 1) anorm2 = fmax(anorm2, coef[2]);
+        if (i == a.k - 1) break;
         // ---- phase C: the recurrence on the own sites (Eq. 4.2), reductions for beta, gamma
         ff pc[4] = {{0.f, 0.f}, {0.f, 0.f}, {0.f, 0.f}, {0.f, 0.f}};
         float4* const xn = vw ? a.w[(i + 1) % 3] : a.v[(i + 1) % 3];
@@ -376,48 +429,65 @@ __global__ void __launch_bounds__(32 * PW1) k_pass1_persistent(P1Args a) {
         block_reduce_ff<4, PW1>(pc, redf, a.partC + (size_t)blockIdx.x * 4);
         grid_barrier_mono(a.bar, (unsigned)G * (++nbar) + a.unreach, err, 1, a.spin);
         if (*(volatile int*)err) return;
+        double nv = 0.0, gm = 0.0, rnv = 0.0;
         if (wid == 0) {
-            warp_sum_partials(a.partC, 4, 4, G, oc);
-            if (lane == 0) {
-                const double nv2 = oc[2], nw2 = oc[3];
-                const cx<double> delta = mk(oc[0], oc[1]);
-                int dn = 0;
-                if (nv2 <= 1e-26 * fmax(anorm2, 1e-300)) {
-                    dn = 1;  // lucky breakdown: |v^| <= 1e-13 max |A v_i|
-                } else if (norm2(delta) <= 1e-28 * nv2 * nw2) {
-                    dn = 1;  // serious breakdown: |w^^dag v^| <= 1e-14 |v^| |w^|
-                    bd = i + 1;
-                } else {
-                    const double rnv = rsqrt(nv2), nv = nv2 * rnv;
-                    const cx<double> gm = mk(oc[0] * rnv, oc[1] * rnv);
-                    beta_prev = mk(nv, 0.0);
-                    gamma_prev = gm;
-                    if (blockIdx.x == 0) {
-                        a.beta[i] = c2d(beta_prev);
-                        a.gamma[i] = c2d(gm);
-                    }
-                    svp = sv;
-                    swp = sw;
-                    sv = mk(rnv, 0.0);
-                    sw = (1.0 / norm2(gm)) * gm;  // 1 / conj(gm)
-                    sh.cs[0] = down(sv);
-                    sh.cs[1] = down(sw);
-                }
-                sh.done = dn;
+            // beta = |v^|, gamma = delta / beta, sv = 1 / beta, sw = 1 / conj(gamma) = delta beta / |delta|^2
+            double o[4];
+            warp_sum4_partials(a.partC, 4, G, o);
+            const bool q = lane & 1;
+            const double nd2 = fma(o[1], o[1], o[0] * o[0]);
+            const double r = rsqrt(q ? nd2 : o[2]);  // even lanes 1 / |v^|, odd lanes 1 / |delta|
+            const double r2 = r * (q ? r : o[2]);    // |v^|, 1 / |delta|^2
+            rnv = __shfl_sync(0xffffffffu, r, 0);
+            nv = __shfl_sync(0xffffffffu, r2, 0);
+            const double f = nv * __shfl_sync(0xffffffffu, r2, 1);
+            gm = (q ? o[1] : o[0]) * (lane < 2 ? rnv : f);  // lanes 0, 1: gamma; lanes 2, 3: sw
+            // the next step's gamma_{i-1} svp and conj(beta_{i-1}) swp
+            const double cn = (lane < 2 ? gm : nv) * (lane < 2 ? svr : (q ? swi : swr));
+            if (lane < 4) reinterpret_cast<float*>(sh.cp)[lane] = (float)cn;
+        } else if (wid == 1) {
+            double o[4];
+            warp_sum4_partials(a.partC, 4, G, o);
+            const double nd2 = fma(o[1], o[1], o[0] * o[0]);
+            int dn = 0;
+            if (o[2] <= 1e-26 * fmax(anorm2, 1e-300)) {
+                dn = 1;  // lucky breakdown: |v^| <= 1e-13 max |A v_i|
+            } else if (nd2 <= 1e-28 * o[2] * o[3]) {
+                dn = 1;  // serious breakdown: |w^^dag v^| <= 1e-14 |v^| |w^|
+                bd = i + 1;
             }
+            if (lane == 0) sh.done = dn;
         }
         __syncthreads();
         if (sh.done) break;
+        if (wid == 0) {
+            svpr = svr, swpr = swr, swpi = swi;
+            svr = rnv;
+            swr = __shfl_sync(0xffffffffu, gm, 2);
+            swi = __shfl_sync(0xffffffffu, gm, 3);
+            const double gi = __shfl_sync(0xffffffffu, gm, 1);
+            if (lane == 0) {
+                sh.cs[0] = mk((float)svr, 0.f);
+                sh.cs[1] = mk((float)swr, (float)swi);
+                if (blockIdx.x == 0) {
+                    a.beta[i] = make_double2(nv, 0.0);
+                    a.gamma[i] = make_double2(gm, gi);
+                }
+            }
+        }
+        __syncthreads();
     }
     if (blockIdx.x == 0 && tid == 0) {
+        ks->sv = make_double2(svr, 0.0);
+        ks->sw = make_double2(swr, swi);
+        ks->svp = make_double2(svpr, 0.0);
+        ks->swp = make_double2(swpr, swpi);
+    }
+    if (blockIdx.x == 0 && tid == 32) {
         ks->kused = kused;
         ks->done = 1;
         ks->anorm = sqrt(anorm2);
         if (bd >= 0) ks->bdstep = bd;
-        ks->sv = c2d(sv);
-        ks->sw = c2d(sw);
-        ks->svp = c2d(svp);
-        ks->swp = c2d(swp);
     }
 }
 
