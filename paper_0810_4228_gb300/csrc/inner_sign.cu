@@ -99,6 +99,7 @@ __global__ void k_quad_prep(const double2* alpha, const double2* beta, const dou
         double mm = 0.0;
         for (int w = 0; w < (int)(blockDim.x >> 5); ++w) mm = fmax(mm, red[w]);
         ks->red[7] = make_double2(log(fmax(mm, 1e-300)), 0.0);
+        ks->red[6] = make_double2(0.0, 0.0);  // a singular node of the level solved ahead (k_quad_solve)
         ks->inner_done = 0;
         ks->inner_iters = 0;
         ks->inner_method = 0;
@@ -133,18 +134,26 @@ __device__ __forceinline__ float cabs1f(const cx<df>& z) { return fabsf(z.r.hi) 
 // FP32 pipe: a node's elimination is one dependent chain of complex operations per row, and
 // GB300's FP64 unit would run each of them 64x slower; 48 significant bits keep the quadrature's
 // 1e-14 accuracy.
+// Levels 0 and 1 (as many nodes each) are solved by one launch, blockIdx.z = 1 ahead of level 0's verdict
+// into its own region behind level 0's: a launch is one dependent chain of 2 k rows whatever its nodes, and
+// level 1 is needed more often than not.  The chain waits for no loads: coefficients are loaded a row ahead,
+// the back substitution's rows four ahead.  k = 480: 8^4 solve 11.33 -> 11.14 ms, 6^4 FP64 solve 7.87 -> 7.70 ms.
 __global__ void k_quad_solve(KState* ks, double2* __restrict__ work, size_t coef_off, int level, int nthreads,
                              QStride qs) {
+    const dfc* ca;
     {
         const size_t j = blockIdx.y;
         ks += j;
         work += j * qs.work;
+        ca = reinterpret_cast<const dfc*>(work + coef_off);
     }
     if (ks->inner_done || ks->status || ks->timeout) return;
     const int t = blockIdx.x * blockDim.x + threadIdx.x;
     if (t >= nthreads) return;
+    const bool ahead = blockIdx.z == 1;
+    if (ahead) level = 1;
     const int n = ks->kused;
-    const dfc* ca = reinterpret_cast<const dfc*>(work + coef_off);
+    if (level == 1) work += 3 * (size_t)n * nthreads;
     const dfc* cb = ca + n;
     const dfc* cg = ca + 2 * n;
     const double lo = ks->red[7].x - QUAD_HALFWIDTH;
@@ -165,14 +174,24 @@ __global__ void k_quad_solve(KState* ks, double2* __restrict__ work, size_t coef
     dfc* wd = bd + 2 * (size_t)n * nthreads;
     const dfc zero = {0.f, 0.f, 0.f, 0.f};
 #define IDX(i) ((size_t)(i) * nthreads + t)
+    // (the coefficients are read-only here; a row's are loaded while the one before is eliminated)
+    auto coef = [](const dfc* p, int i) {
+        const float4 v = __ldg(reinterpret_cast<const float4*>(p) + i);
+        return dfc{v.x, v.y, v.z, v.w};
+    };
     // current row i: (d, u) at (i, i+1), rhs rb
-    cx<df> d = dfc2c(ca[0]) + sig;
-    cx<df> uu = n > 1 ? dfc2c(cg[0]) : mk(df(0), df(0));
+    cx<df> d = dfc2c(coef(ca, 0)) + sig;
+    cx<df> uu = n > 1 ? dfc2c(coef(cg, 0)) : mk(df(0), df(0));
     cx<df> rb = mk(df(1), df(0));
+    dfc nl = zero, na = zero, ng = zero;
+    if (n > 1) nl = coef(cb, 0), na = coef(ca, 1);
+    if (n > 2) ng = coef(cg, 1);
     for (int i = 0; i + 1 < n; ++i) {
-        const cx<df> l = dfc2c(cb[i]);                  // row i+1, column i
-        const cx<df> dn = dfc2c(ca[i + 1]) + sig;       // row i+1, column i+1
-        const cx<df> un = (i + 2 < n) ? dfc2c(cg[i + 1]) : mk(df(0), df(0));
+        const cx<df> l = dfc2c(nl);                     // row i+1, column i
+        const cx<df> dn = dfc2c(na) + sig;              // row i+1, column i+1
+        const cx<df> un = (i + 2 < n) ? dfc2c(ng) : mk(df(0), df(0));
+        if (i + 2 < n) nl = coef(cb, i + 1), na = coef(ca, i + 2);
+        if (i + 3 < n) ng = coef(cg, i + 2);
         if (cabs1f(d) >= cabs1f(l)) {
             // no interchange: final row i = (d, uu, 0)
             const cx<df> id = crcp(d);
@@ -196,25 +215,45 @@ __global__ void k_quad_solve(KState* ks, double2* __restrict__ work, size_t coef
             // new rhs of row i+1: rb (old row i) - m * 0
         }
     }
-    if (d.r.hi == 0.f && d.i.hi == 0.f) {
-        atomicExch(&ks->status, 5);  // singular shifted matrix
+    if (d.r.hi == 0.f && d.i.hi == 0.f) {  // singular shifted matrix
+        if (ahead) ks->red[6].x = 1.0;     // counts only if level 1 is used
+        else atomicExch(&ks->status, 5);
         return;
     }
     // back substitution, x overwrites bd
     cx<df> x1 = rb * crcp(d), x2 = mk(df(0), df(0));
     bd[IDX(n - 1)] = c2dfc(mk(tau * x1.r, tau * x1.i));
-    for (int i = n - 2; i >= 0; --i) {
-        const cx<df> x = dfc2c(bd[IDX(i)]) - dfc2c(ud[IDX(i)]) * x1 - dfc2c(wd[IDX(i)]) * x2;
-        bd[IDX(i)] = c2dfc(mk(tau * x.r, tau * x.i));
-        x2 = x1;
-        x1 = x;
+    // (four rows at a time, the next four on their way meanwhile: a row's own loads would each cost the
+    // chain an L2 round trip)
+    constexpr int RP = 4;
+    dfc rbd[RP], rud[RP], rwd[RP];
+    auto rows = [&](int i) {
+#pragma unroll
+        for (int r = 0; r < RP; ++r)
+            if (i - r >= 0) rbd[r] = bd[IDX(i - r)], rud[r] = ud[IDX(i - r)], rwd[r] = wd[IDX(i - r)];
+    };
+    rows(n - 2);
+    for (int i = n - 2; i >= 0; i -= RP) {
+        dfc b4[RP], u4[RP], w4[RP];
+#pragma unroll
+        for (int r = 0; r < RP; ++r) b4[r] = rbd[r], u4[r] = rud[r], w4[r] = rwd[r];
+        rows(i - RP);
+#pragma unroll
+        for (int r = 0; r < RP; ++r) {
+            if (i - r < 0) break;
+            const cx<df> x = dfc2c(b4[r]) - dfc2c(u4[r]) * x1 - dfc2c(w4[r]) * x2;
+            bd[IDX(i - r)] = c2dfc(mk(tau * x.r, tau * x.i));
+            x2 = x1;
+            x1 = x;
+        }
     }
 #undef IDX
 }
 
 // T_l = (l == 0 ? 0 : T_{l-1}/2) + (h_l/pi) sum_threads x ; convergence on |T_l - T_{l-1}|.
 __global__ void k_quad_sum(const double2* __restrict__ work, double2* __restrict__ T, double2* __restrict__ c,
-                           KState* ks, int level, int nthreads, double* partials, unsigned int* counter, QStride qs) {
+                           KState* ks, int level, int nthreads, double* partials, unsigned int* counter, QStride qs,
+                           int tri) {
     __shared__ double red[96];
     {
         const size_t j = blockIdx.y;
@@ -227,6 +266,13 @@ __global__ void k_quad_sum(const double2* __restrict__ work, double2* __restrict
     }
     if (ks->inner_done || ks->status || ks->timeout) return;
     const int n = ks->kused;
+    if (tri && level == 1) {  // solved ahead, behind level 0's region
+        if (ks->red[6].x != 0.0) {
+            if (blockIdx.x == 0 && threadIdx.x == 0) atomicExch(&ks->status, 5);
+            return;
+        }
+        work += 3 * (size_t)n * nthreads;
+    }
     const double hl = QUAD_H0 / (double)(1 << level);
     const double wgt = hl / M_PI;
     double part[2] = {0.0, 0.0};  // |T_l - T_{l-1}|^2, |T_l|^2
@@ -288,10 +334,12 @@ static void quad_launch(const double2* alpha, const double2* beta, const double2
     k_quad_prep<<<nseq, 256, 0, st>>>(alpha, beta, gamma, ks, work, coef_off, qs);
     for (int level = 0; level < QUAD_LEVELS; ++level) {
         const int nt = quad_threads(level);
-        k_quad_solve<<<dim3((nt + 31) / 32, nseq), 32, 0, st>>>(ks, work, coef_off, level, nt, qs);
+        if (level != 1)  // level 1 is solved by level 0's launch
+            k_quad_solve<<<dim3((nt + 31) / 32, nseq, level == 0 ? 2 : 1), 32, 0, st>>>(ks, work, coef_off, level,
+                                                                                        nt, qs);
         int blocks = (kmax + 7) / 8;
         if (blocks > 256) blocks = 256;
-        k_quad_sum<<<dim3(blocks, nseq), 256, 0, st>>>(work, T, c, ks, level, nt, partials, counter, qs);
+        k_quad_sum<<<dim3(blocks, nseq), 256, 0, st>>>(work, T, c, ks, level, nt, partials, counter, qs, 1);
     }
 }
 
@@ -509,7 +557,7 @@ static void hess_quad_launch(const double2* H, int ldH, KState* ks, double2* c, 
         k_hess_solve<<<(nt + wpb - 1) / wpb, 32 * wpb, smem, st>>>(ks, work, hoff, kmax, kmax, level, nt);
         int blocks = (kmax + 7) / 8;
         if (blocks > 256) blocks = 256;
-        k_quad_sum<<<dim3(blocks, 1), 256, 0, st>>>(work, T, c, ks, level, nt, partials, counter, QStride{0, 0, 0});
+        k_quad_sum<<<dim3(blocks, 1), 256, 0, st>>>(work, T, c, ks, level, nt, partials, counter, QStride{0, 0, 0}, 0);
     }
 }
 
