@@ -114,86 +114,110 @@ __global__ void k_tadj_prep(const double2* alpha, const double2* beta, const dou
     }
 }
 
-// Solve M x = rhs for the tridiagonal M (diag d_j + shift, below l_j, above u_j), Gaussian elimination
-// with partial pivoting; rows of the eliminated system in the thread's scratch columns (stride nt).
-// adj = true solves with M = G^dag (diag conj(alpha), below conj(gamma), above conj(beta)).
-// rhs: e_1 if null.  Returns false if singular.  x overwrites bd.
-__device__ bool tri_solve(const double2* alpha, const double2* beta, const double2* gamma, bool adj, cx<double> shift,
-                          const double2* rhs, int n, double2* bd, double2* ud, double2* wd, int nt, int t) {
+// x = scale (M + shift)^-1 e_1 for the tridiagonal M = G, or M = G^dag (ADJ: diagonal conj(alpha), below conj(gamma),
+// above conj(beta)): Gaussian elimination with partial pivoting, rows of the eliminated system in the thread's
+// scratch columns (stride nt).  Returns false if singular.  x overwrites bd.  One dependent chain of FP64
+// operations, 64 cycles each: the loads are kept out of it (coefficients one row ahead, the back substitution's
+// rows four ahead).
+template <bool ADJ>
+__device__ bool tri_solve(const double2* __restrict__ alpha, const double2* __restrict__ beta,
+                          const double2* __restrict__ gamma, cx<double> shift, double scale, int n, double2* bd,
+                          double2* ud, double2* wd, int nt, int t) {
 #define IDX(i) ((size_t)(i) * nt + t)
-    auto D = [&](int j) { const cx<double> a = d2c(alpha[j]); return (adj ? conj(a) : a) + shift; };
-    auto Lw = [&](int j) { return adj ? conj(d2c(gamma[j])) : d2c(beta[j]); };   // row j+1, col j
-    auto Up = [&](int j) { return adj ? conj(d2c(beta[j])) : d2c(gamma[j]); };   // row j, col j+1
-    auto R = [&](int j) { return rhs ? d2c(rhs[j]) : (j == 0 ? mk(1.0, 0.0) : mk(0.0, 0.0)); };
-    cx<double> d = D(0);
-    cx<double> uu = n > 1 ? Up(0) : mk(0.0, 0.0);
-    cx<double> rb = R(0);
+    auto C = [](double2 v) { return ADJ ? conj(d2c(v)) : d2c(v); };
+    const double2* __restrict__ lw = ADJ ? gamma : beta;  // row j+1, column j
+    const double2* __restrict__ up = ADJ ? beta : gamma;  // row j, column j+1
+    const double2 zero = make_double2(0.0, 0.0);
+    cx<double> d = C(__ldg(alpha)) + shift;
+    cx<double> uu = n > 1 ? C(__ldg(up)) : mk(0.0, 0.0);
+    cx<double> rb = mk(1.0, 0.0);
+    double2 nl = zero, na = zero, ng = zero;
+    if (n > 1) nl = __ldg(lw), na = __ldg(alpha + 1);
+    if (n > 2) ng = __ldg(up + 1);
     for (int i = 0; i + 1 < n; ++i) {
-        const cx<double> l = Lw(i), dn = D(i + 1);
-        const cx<double> un = (i + 2 < n) ? Up(i + 1) : mk(0.0, 0.0);
-        const cx<double> rn = R(i + 1);
-        if (norm2(d) >= norm2(l)) {
-            if (norm2(d) == 0.0) return false;
-            const double inv = 1.0 / norm2(d);
+        const cx<double> l = C(nl), dn = C(na) + shift;
+        const cx<double> un = (i + 2 < n) ? C(ng) : mk(0.0, 0.0);
+        if (i + 2 < n) nl = __ldg(lw + i + 1), na = __ldg(alpha + i + 2);
+        if (i + 3 < n) ng = __ldg(up + i + 2);
+        const double d2 = norm2(d), l2 = norm2(l);
+        if (d2 >= l2) {
+            if (d2 == 0.0) return false;
+            const double inv = 1.0 / d2;
             const cx<double> id = mk(d.r * inv, -d.i * inv);
             const cx<double> m = l * id;
             bd[IDX(i)] = c2d(rb * id);
             ud[IDX(i)] = c2d(uu * id);
-            wd[IDX(i)] = make_double2(0.0, 0.0);
+            wd[IDX(i)] = zero;
             d = dn - m * uu;
             uu = un;
-            rb = rn - m * rb;
+            rb = mk(m.i * rb.i - m.r * rb.r, -m.r * rb.i - m.i * rb.r);  // the right-hand side of row i+1 is 0
         } else {
-            const double inv = 1.0 / norm2(l);
+            const double inv = 1.0 / l2;
             const cx<double> il = mk(l.r * inv, -l.i * inv);
             const cx<double> m = d * il;
-            bd[IDX(i)] = c2d(rn * il);
+            bd[IDX(i)] = zero;
             ud[IDX(i)] = c2d(dn * il);
             wd[IDX(i)] = c2d(un * il);
-            const cx<double> nd = uu - m * dn;
-            const cx<double> nu = mk(0.0, 0.0) - m * un;
-            rb = rb - m * rn;
-            d = nd;
-            uu = nu;
+            d = uu - m * dn;
+            uu = mk(m.i * un.i - m.r * un.r, -m.r * un.i - m.i * un.r);
         }
     }
     if (norm2(d) == 0.0) return false;
     cx<double> x1 = cdiv(rb, d), x2 = mk(0.0, 0.0);
-    bd[IDX(n - 1)] = c2d(x1);
-    for (int i = n - 2; i >= 0; --i) {
-        const cx<double> x = d2c(bd[IDX(i)]) - d2c(ud[IDX(i)]) * x1 - d2c(wd[IDX(i)]) * x2;
-        bd[IDX(i)] = c2d(x);
-        x2 = x1;
-        x1 = x;
+    bd[IDX(n - 1)] = c2d(scale * x1);
+    constexpr int RP = 4;
+    double2 rbd[RP], rud[RP], rwd[RP];
+    auto rows = [&](int i) {
+#pragma unroll
+        for (int r = 0; r < RP; ++r)
+            if (i - r >= 0) rbd[r] = bd[IDX(i - r)], rud[r] = ud[IDX(i - r)], rwd[r] = wd[IDX(i - r)];
+    };
+    rows(n - 2);
+    for (int i = n - 2; i >= 0; i -= RP) {
+        double2 b4[RP], u4[RP], w4[RP];
+#pragma unroll
+        for (int r = 0; r < RP; ++r) b4[r] = rbd[r], u4[r] = rud[r], w4[r] = rwd[r];
+        rows(i - RP);
+#pragma unroll
+        for (int r = 0; r < RP; ++r) {
+            if (i - r < 0) break;
+            const cx<double> x = d2c(b4[r]) - d2c(u4[r]) * x1 - d2c(w4[r]) * x2;
+            bd[IDX(i - r)] = c2d(ADJ ? x : scale * x);
+            x2 = x1;
+            x1 = x;
+        }
     }
 #undef IDX
     return true;
 }
 
-
-// one thread per (node, sign s): a = (G + s i e^u)^-1 e_1 and d = (G^dag - s i e^u)^-1 e_1 into the
-// scratch (region 0: a, region 3: d; thread columns)
+// One thread per (node, sign s) and system: e^u a, a = (G + s i e^u)^-1 e_1 (blockIdx.y = 0, region 0 of the scratch;
+// e^u itself into region 1, free after the solve) and d = (G^dag - s i e^u)^-1 e_1 (blockIdx.y = 1, region 3); thread
+// columns.  blockIdx.z = 1: level + 1 into the next six regions (the first two levels have as many nodes and
+// are always both needed).  Bound by the length of the chain, 2 n rows, whatever runs beside it: the four
+// solves side by side took forward and backward on 6^4 (k = 480) from 31.8 to 27.3 ms (two launches of 2.75 ms,
+// each with its two solves one after the other, and a host check in between, before).
 __global__ void k_gq_solve(const double2* alpha, const double2* beta, const double2* gamma, int n,
                            const double* scal, double2* work, int level, int nt, int* status) {
     const int t = blockIdx.x * blockDim.x + threadIdx.x;
     if (t >= nt) return;
+    const size_t reg = (size_t)n * nt;
+    level += blockIdx.z;
+    work += 6 * reg * blockIdx.z;
     const double lo = scal[0] - TADJ_HALFWIDTH;
     const int node = t >> 1;
     const double sg = (t & 1) ? -1.0 : 1.0;
     const double u = level == 0 ? lo + node * TADJ_H0 : lo + (2 * node + 1) * (TADJ_H0 / (double)(1 << level));
     const double tau = exp(u);
-    double2* r = work;
-    double2* d = work + 3 * (size_t)n * nt;
-    if (!tri_solve(alpha, beta, gamma, false, mk(0.0, sg * tau), nullptr, n, r, r + (size_t)n * nt,
-                   r + 2 * (size_t)n * nt, nt, t) ||
-        !tri_solve(alpha, beta, gamma, true, mk(0.0, -sg * tau), nullptr, n, d, d + (size_t)n * nt,
-                   d + 2 * (size_t)n * nt, nt, t)) {
-        atomicExch(status, 5);
-        return;
+    bool ok;
+    if (blockIdx.y == 0) {
+        ok = tri_solve<false>(alpha, beta, gamma, mk(0.0, sg * tau), tau, n, work, work + reg, work + 2 * reg, nt, t);
+        work[reg + t] = make_double2(tau, 0.0);
+    } else {
+        ok = tri_solve<true>(alpha, beta, gamma, mk(0.0, -sg * tau), 1.0, n, work + 3 * reg, work + 4 * reg,
+                             work + 5 * reg, nt, t);
     }
-    // weight e^u folded into a; e^u kept for the d sum (region 1 is free after the solves)
-    for (int j = 0; j < n; ++j) r[(size_t)j * nt + t] = c2d(tau * d2c(r[(size_t)j * nt + t]));
-    work[(size_t)n * nt + t] = make_double2(tau, 0.0);
+    if (!ok) atomicExch(status, 5);
 }
 
 // M_l = M_{l-1}/2 + h_l sum_threads conj(d_p) (e^u a_q), a 16 x 16 tile of (p, q) per block, the
@@ -801,11 +825,14 @@ extern "C" int ovl_sign_grad(ovl_ctx* c, int k, double mu, double kappa, const v
         bool conv = false;
         for (int level = 0; level < ovl::TADJ_LEVELS && !conv; ++level) {
             const int nt = level == 0 ? 2 * m0 : 2 * (m0 << (level - 1));
-            ovl::k_gq_solve<<<(nt + 31) / 32, 32, 0, st>>>(c->alpha, c->beta, c->gamma, kk, tscal, c->tadj, level, nt,
-                                                           tstatus);
+            if (level != 1)  // level 1 is solved with level 0
+                ovl::k_gq_solve<<<dim3((nt + 31) / 32, 2, level == 0 ? 2 : 1), 32, 0, st>>>(
+                    c->alpha, c->beta, c->gamma, kk, tscal, c->tadj, level, nt, tstatus);
+            const double2* sol = c->tadj + (level == 1 ? 6 * (size_t)kk * nt : 0);
             const int ntile = (kk + ovl::GQ_T - 1) / ovl::GQ_T;
-            ovl::k_gq_accum<<<ntile * ntile, 256, 0, st>>>(c->tadj, kk, nt, level, M, part, cnt, dn);
-            ovl::k_gq_dsum<<<(kk + 7) / 8, 256, 0, st>>>(c->tadj, kk, nt, level, sd);
+            ovl::k_gq_accum<<<ntile * ntile, 256, 0, st>>>(sol, kk, nt, level, M, part, cnt, dn);
+            ovl::k_gq_dsum<<<(kk + 7) / 8, 256, 0, st>>>(sol, kk, nt, level, sd);
+            if (level == 0) continue;  // nothing to compare with yet
             double hd[2];
             int hst = 0;
             OVL_CUDA_TRY(c, cudaMemcpyAsync(hd, dn, sizeof(hd), cudaMemcpyDeviceToHost, st));
@@ -814,7 +841,7 @@ extern "C" int ovl_sign_grad(ovl_ctx* c, int k, double mu, double kappa, const v
             if (hst) return fail(c, OVL_ESINGULAR, "shifted projected matrix is singular");
             // geometric convergence: the error of level l is about rel^2
             const double rel = std::sqrt(hd[0]) / std::max(std::sqrt(hd[1]), 1e-300);
-            if (level > 0 && rel <= 1e-6) conv = true;
+            if (rel <= 1e-6) conv = true;
         }
         if (!conv) return fail(c, OVL_ENOCONV, "quadrature of the gradient did not converge");
         const size_t ne = (size_t)kk * kk + kk;
