@@ -135,7 +135,7 @@ __device__ __forceinline__ float cabs1f(const cx<df>& z) { return fabsf(z.r.hi) 
 // GB300's FP64 unit would run each of them 64x slower; 48 significant bits keep the quadrature's
 // 1e-14 accuracy.
 // Levels 0 and 1 (as many nodes each) are solved by one launch, blockIdx.z = 1 ahead of level 0's verdict
-// into its own region behind level 0's: a launch is one dependent chain of 2 k rows whatever its nodes, and
+// into its own region behind level 0's (k_quad_sum reads it there): a launch is one dependent chain of 2 k rows whatever its nodes, and
 // level 1 is needed more often than not.  The chain waits for no loads: coefficients are loaded a row ahead,
 // the back substitution's rows four ahead.  k = 480: 8^4 solve 11.33 -> 11.14 ms, 6^4 FP64 solve 7.87 -> 7.70 ms.
 __global__ void k_quad_solve(KState* ks, double2* __restrict__ work, size_t coef_off, int level, int nthreads,
@@ -252,8 +252,7 @@ __global__ void k_quad_solve(KState* ks, double2* __restrict__ work, size_t coef
 
 // T_l = (l == 0 ? 0 : T_{l-1}/2) + (h_l/pi) sum_threads x ; convergence on |T_l - T_{l-1}|.
 __global__ void k_quad_sum(const double2* __restrict__ work, double2* __restrict__ T, double2* __restrict__ c,
-                           KState* ks, int level, int nthreads, double* partials, unsigned int* counter, QStride qs,
-                           int tri) {
+                           KState* ks, int level, int nthreads, double* partials, unsigned int* counter, QStride qs) {
     __shared__ double red[96];
     {
         const size_t j = blockIdx.y;
@@ -266,7 +265,7 @@ __global__ void k_quad_sum(const double2* __restrict__ work, double2* __restrict
     }
     if (ks->inner_done || ks->status || ks->timeout) return;
     const int n = ks->kused;
-    if (tri && level == 1) {  // solved ahead, behind level 0's region
+    if (level == 1) {  // solved ahead, behind level 0's region
         if (ks->red[6].x != 0.0) {
             if (blockIdx.x == 0 && threadIdx.x == 0) atomicExch(&ks->status, 5);
             return;
@@ -339,7 +338,7 @@ static void quad_launch(const double2* alpha, const double2* beta, const double2
                                                                                         nt, qs);
         int blocks = (kmax + 7) / 8;
         if (blocks > 256) blocks = 256;
-        k_quad_sum<<<dim3(blocks, nseq), 256, 0, st>>>(work, T, c, ks, level, nt, partials, counter, qs, 1);
+        k_quad_sum<<<dim3(blocks, nseq), 256, 0, st>>>(work, T, c, ks, level, nt, partials, counter, qs);
     }
 }
 
@@ -396,6 +395,7 @@ __global__ void __launch_bounds__(256) k_hess_prep(const double2* __restrict__ H
     if (grid_sum_last<1>(part, partials, counter, out, red)) {
         if (threadIdx.x == 0) {
             ks->red[7] = make_double2(log(fmax(sqrt(out[0]), 1e-300)), 0.0);
+            ks->red[6] = make_double2(0.0, 0.0);  // a singular node of the level solved ahead
             ks->inner_done = (n == 0);
             ks->inner_iters = 0;
             ks->inner_method = 0;
@@ -448,6 +448,8 @@ __device__ __forceinline__ cx<df> shfl_cdf(const cx<df>& z, int src) {
 
 static constexpr int HQ_WPB_MAX = 4;  // warps (nodes) per block
 
+// (blockIdx.z = 1: level 1 beside level 0, ahead of its verdict, as k_quad_solve does; the launch is bound by
+// its warps' chains: k = 450, Arnoldi on 8^4 52.1 -> 51.6 ms)
 __global__ void k_hess_solve(KState* ks, double2* __restrict__ work, size_t hoff, int ldd, int kmax, int level,
                              int nthreads) {
     extern __shared__ float4 hq_col[];
@@ -457,6 +459,11 @@ __global__ void k_hess_solve(KState* ks, double2* __restrict__ work, size_t hoff
     if (t >= nthreads) return;  // whole warps
     const int n = ks->kused;
     const dfc* Hd = reinterpret_cast<const dfc*>(work + hoff);
+    const bool ahead = blockIdx.z == 1;
+    if (ahead) {
+        level = 1;
+        work += 3 * (size_t)n * nthreads;
+    }
     float4* col = hq_col + (size_t)wid * kmax;
     const double lo = ks->red[7].x - QUAD_HALFWIDTH;
     const int node = t >> 1;
@@ -499,7 +506,10 @@ __global__ void k_hess_solve(KState* ks, double2* __restrict__ work, size_t hoff
     const float4 r0 = col[0];
     const cx<df> R00 = mk(df(r0.x, r0.y), df(r0.z, r0.w));
     if (R00.r.hi == 0.f && R00.i.hi == 0.f) {
-        if (lane == 0) atomicExch(&ks->status, 5);  // singular shifted matrix
+        if (lane == 0) {  // singular shifted matrix
+            if (ahead) ks->red[6].x = 1.0;  // counts only if level 1 is used
+            else atomicExch(&ks->status, 5);
+        }
         return;
     }
     __syncwarp();  // CA, CB written by lane 0 are read by every lane below
@@ -554,10 +564,12 @@ static void hess_quad_launch(const double2* H, int ldH, KState* ks, double2* c, 
     }
     for (int level = 0; level < QUAD_LEVELS; ++level) {
         const int nt = quad_threads(level);
-        k_hess_solve<<<(nt + wpb - 1) / wpb, 32 * wpb, smem, st>>>(ks, work, hoff, kmax, kmax, level, nt);
+        if (level != 1)  // level 1 is solved by level 0's launch
+            k_hess_solve<<<dim3((nt + wpb - 1) / wpb, 1, level == 0 ? 2 : 1), 32 * wpb, smem, st>>>(ks, work, hoff, kmax,
+                                                                                                   kmax, level, nt);
         int blocks = (kmax + 7) / 8;
         if (blocks > 256) blocks = 256;
-        k_quad_sum<<<dim3(blocks, 1), 256, 0, st>>>(work, T, c, ks, level, nt, partials, counter, QStride{0, 0, 0}, 0);
+        k_quad_sum<<<dim3(blocks, 1), 256, 0, st>>>(work, T, c, ks, level, nt, partials, counter, QStride{0, 0, 0});
     }
 }
 
