@@ -113,7 +113,7 @@ extern "C" int ovl_apply_pair_noalloc(ovl_ctx* c, double mu, double kappa, int p
     double* partials = scratch + (kStateBytes + kCounterBytes) / sizeof(double);
     k_noalloc_reset<<<1, 1, 0, c->st>>>(scratch);
     ovl::launch_dslash_pair(prec == 0 ? (const void*)c->U64 : (const void*)c->U12, prec, v, w, t, s, mu, kappa, ks,
-                            reinterpret_cast<double2*>(alpha_dev), 0, 1 << 30, partials, counter, c->g, c->st);
+                            reinterpret_cast<double2*>(alpha_dev), 0, 1 << 30, partials, counter, c->g, c->st, true);
     const cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return fail(c, OVL_ECUDA, std::string("kernel launch: ") + cudaGetErrorString(e));
     return OVL_OK;

@@ -51,17 +51,18 @@ void launch_dslash(const void* U, int prec, const void* x, void* y, double mu, d
 void launch_dslash_canon(const double2* U64, const double2* x, double2* y, double mu, double kappa, int gamma5,
                          const Geom& g, cudaStream_t st);
 // pair: t = sv * A v~, s = sw * A^dag w~, alpha[step] = w^dag t (fused grid reduction),
-// kused = step + 1, done after step klast.
+// kused = step + 1, done after step klast.  fixed_grid: the grid of dslash_pair_blocks.
 void launch_dslash_pair(const void* U, int prec, const void* v, const void* w, void* t, void* s,
                         double mu, double kappa, KState* ks, double2* alpha, int step, int klast,
-                        double* partials, unsigned int* counter, const Geom& g, cudaStream_t st);
+                        double* partials, unsigned int* counter, const Geom& g, cudaStream_t st,
+                        bool fixed_grid = false);
 // FP64 regeneration step of the two-pass 2sL (Sec. 5): v_{i+1} = ((A - alpha_i) v_i - gamma_{i-1} v_{i-1})
 // / beta_i and y += c_{i+1} v_{i+1}, no reductions.
 void launch_dslash_regen(const double2* U, const double2* vi, const double2* vim1, double2* vip1, double2* y,
                          double mu, double kappa, const KState* ks, const double2* alpha, const double2* beta,
                          const double2* gamma, const double2* c, int step, const Geom& g, cudaStream_t st);
 int dslash_grid(const Geom& g, int threads);
-// thread blocks launch_dslash_pair launches on g (= the partial-sum slots its reduction writes)
+// thread blocks launch_dslash_pair launches on g with fixed_grid (= the partial-sum slots its reduction writes)
 int dslash_pair_blocks(const Geom& g);
 // nvec FP64 device-layout vectors to the FP32 device layout (component pairs in float4)
 void launch_native_f64_to_f32(const double2* x, void* y, const Geom& g, int nvec, cudaStream_t st);

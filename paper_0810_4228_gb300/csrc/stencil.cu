@@ -511,13 +511,15 @@ __global__ void __launch_bounds__(128, LF == LINK_F64 ? 2 : OVL_DSLASH_F32_MINB)
 // The FP32 form sums alpha in compensated pairs (48 bits; the FP32 rounding of t itself, which both forms share,
 // is what alpha's error is made of).
 static bool pair_ds(const Geom& g) { return g_ds_mode < 0 ? g.V < (1 << 13) : g_ds_mode == 1; }
-int dslash_pair_blocks(const Geom& g) { return pair_ds(g) ? ds_grid(g) : dslash_grid(g, 128); }
+// The allocation-free call answers for its grid (ovl_apply_pair_noalloc_blocks) and keeps the one it had.
+int dslash_pair_blocks(const Geom& g) { return pick_ds(g) ? ds_grid(g) : dslash_grid(g, 128); }
 
 void launch_dslash_pair(const void* U, int prec, const void* v, const void* w, void* t, void* s, double mu,
                         double kappa, KState* ks, double2* alpha, int step, int klast, double* partials,
-                        unsigned int* counter, const Geom& g, cudaStream_t st) {
-    const int B = dslash_pair_blocks(g);  // the partial-sum slots the fused reduction writes
-    if (pair_ds(g)) {
+                        unsigned int* counter, const Geom& g, cudaStream_t st, bool fixed_grid) {
+    const bool split = fixed_grid ? pick_ds(g) : pair_ds(g);
+    const int B = split ? ds_grid(g) : dslash_grid(g, 128);  // the partial-sum slots the fused reduction writes
+    if (split) {
         static unsigned long long attr_dev = 0;
         if (first_use_on_device(attr_dev))
             cudaFuncSetAttribute(k_dslash_pair_ds<LINK_F64>, cudaFuncAttributeMaxDynamicSharedMemorySize,
