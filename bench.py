@@ -451,11 +451,11 @@ def batch_launches(nseq, k, m, persistent_pass1=True, fused_start=False):
     of solve + sum) and k - 1 regeneration steps.  755 for 12 sequences, k = 550, m = 20 (the ncu
     launch list of one solve counts the same).  fused_start: the regeneration's start vectors, their
     conversions and the way back in one launch each for all sequences, plus one for the step
-    coefficients, as the library does it now."""
+    coefficients, and the first two quadrature levels' solves in one launch, as the library does it now."""
     per_seq = 1 + 1 + (4 if m > 0 else 0) + 1 + 2 + 2 + 1 + 2 + 1 + 1
     pass1 = 1 if persistent_pass1 else 2 * k - 1
     if fused_start:
-        return nseq * (per_seq - 4) + pass1 + 1 + 2 * 6 + 3 + (k - 1)
+        return nseq * (per_seq - 4) + pass1 + 1 + 2 * 6 - 1 + 3 + (k - 1)
     return nseq * per_seq + pass1 + 1 + 2 * 6 + (k - 1)
 
 
