@@ -23,9 +23,6 @@
 // count arrivals on a counter zeroed before each launch.
 #include <algorithm>
 
-// pass 1 keeps the rounding that its FP32 products always had, as batch.cu says (a chained multiply-add would
-// take 1.7 % off an 8^4 solve)
-#define OVL_F32_PRODUCTS_FIRST 1
 #include "stencil_impl.cuh"
 
 namespace ovl {
