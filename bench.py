@@ -476,10 +476,10 @@ def calibrate_batch(torch, bt, srcs, refs, flags, grid):
 
 # row a10: per site of ovl_dw_grad, algorithmic bytes (x 192 + g 192 read, the link force
 # 36 complex = 576 written, the temporal link 144 read for d/dmu) and FP64 operations counted
-# from the kernel (per direction two projections and 72 complex multiply-adds of the
-# spin-traced colour outer products, about 780; the d/dmu term about 460)
+# from the kernel (per link two hops of two half-spinor projections, 24, and 18 complex
+# multiply-adds of the colour outer products, 144, and their scaled sum, 36; the d/dmu term 72)
 DWGRAD_BYTES_SITE = 192 + 192 + 576 + 144
-DWGRAD_FLOP_SITE = 4 * 780 + 460
+DWGRAD_FLOP_SITE = 4 * (2 * (24 + 144) + 36) + 72
 
 
 def autograd_timing(torch, ovl, U_np, b, flush, k=800, gdims=(24, 24, 24, 24)):
