@@ -375,8 +375,9 @@ int ovl_overlap_eigs(ovl_ctx* ctx, int method, int k, double mu, double kappa, i
 int ovl_sign_arnoldi_restarted(ovl_ctx* ctx, int m, int cycles, double mu, double kappa,
                                const void* b, void* out, int flags, ovl_info* info);
 
-/* Limits of the bounded device waits of the persistent FP32 pass 1 (the grid barriers of
- * OVL_MIXED two-sided Lanczos solves on lattices that fit the GPU): a wait gives up after
+/* Limits of the bounded device waits of the context's persistent kernels (the grid barriers of
+ * two-sided Lanczos on lattices that fit the GPU: both passes of OVL_MIXED solves, the FP64 process of
+ * ovl_sign_krylov and of ovl_sign_grad): a wait gives up after
  * `polls` polls (0 restores the default, 2e7), sets the solve's timeout flag and every block
  * leaves, so the call returns OVL_ETIMEOUT and the context stays usable.  unreachable != 0 adds
  * one arrival to every barrier's target, so every wait runs out: a test of the timeout path

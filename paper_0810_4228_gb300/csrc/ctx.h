@@ -88,7 +88,7 @@ struct ovl_ctx {
 
     ovl_priv::GraphEntry graph;
 
-    // bounded device waits of the persistent pass 1 (ovl_set_wait_limit; 0 = the default limit)
+    // bounded device waits of the persistent kernels of a solve (ovl_set_wait_limit; 0 = the default limit)
     long long wait_polls = 0;
     int wait_unreachable = 0;
 

@@ -758,7 +758,7 @@ extern "C" int ovl_sign_grad(ovl_ctx* c, int k, double mu, double kappa, const v
         OVL_CUDA_TRY(c, cudaMemsetAsync(c->bar, 0, 64, st));
         double2 *vv[3] = {V, nullptr, nullptr}, *ww[3] = {W, nullptr, nullptr};
         if (ovl::launch_l2_f64(c->U64, c->nbr, vv, n, ww, n, ks, c->alpha, c->beta, c->gamma, c->vscale, mu, kappa, k,
-                               part, c->bar, g, c->num_sms, st))
+                               part, c->bar, g, c->num_sms, st, c->wait_polls, c->wait_unreachable))
             return fail(c, OVL_ECUDA, "persistent FP64 process launch");
     } else {
         for (int i = 0; i < k; ++i) {

@@ -34,7 +34,7 @@ namespace {
 
 constexpr int LW = 16;             // warps per block
 constexpr int LT = 32 * LW;
-constexpr long long LSPIN = 20000000;  // polls before a barrier wait gives up (sets ks->timeout)
+constexpr long long LSPIN = 20000000;  // default limit of a barrier wait's polls (a wait that gives up sets ks->timeout)
 
 // Sums over the lanes of one input (lane bit NB = 8 RS): v0 and v1 each, valid in the lane of that input
 // whose lower bits are 0 (v0) or 4 (v1).  First step: the lane bit above or below NB.
@@ -107,6 +107,8 @@ struct L2Args {
     unsigned int* bar;
     double kappa, emu, emum;
     int V, k, npass;
+    long long spin;       // polls before a barrier wait gives up (ovl_set_wait_limit)
+    unsigned int unreach; // added to every barrier's target
 };
 
 // shared memory: half spinors of a warp's units, then own-site state [pass][cur, prev, t][value][thread]
@@ -217,7 +219,7 @@ __global__ void __launch_bounds__(LT) k_l2_f64(L2Args a) {
         }
         __syncthreads();
         if (wid == 0) block_partials(red, nw, a.partA);
-        grid_barrier_mono(a.bar, (unsigned)G * (++nbar), err, 1, LSPIN);
+        grid_barrier_mono(a.bar, (unsigned)G * (++nbar) + a.unreach, err, 1, a.spin);
         if (*(volatile int*)err) return;
         if (wid < 4) grid_partials(a.partA, G, wid, gs);
         __syncthreads();
@@ -276,7 +278,7 @@ __global__ void __launch_bounds__(LT) k_l2_f64(L2Args a) {
         }
         __syncthreads();
         if (wid == 0) block_partials(red, nw, a.partC);
-        grid_barrier_mono(a.bar, (unsigned)G * (++nbar), err, 1, LSPIN);
+        grid_barrier_mono(a.bar, (unsigned)G * (++nbar) + a.unreach, err, 1, a.spin);
         if (*(volatile int*)err) return;
         if (wid < 4) grid_partials(a.partC, G, wid, gs);
         __syncthreads();
@@ -359,6 +361,8 @@ struct R64Args {
     int* err;
     double kappa, emu, emum;
     int V, npass;
+    long long spin;
+    unsigned int unreach;
 };
 
 template <int RS>
@@ -439,7 +443,7 @@ __global__ void __launch_bounds__(LT) k_regen_f64(R64Args a) {
             __syncwarp();
         }
         if (i + 2 < kused) {
-            grid_barrier_mono(a.bar, (unsigned)G * (++nbar), a.err, 1, LSPIN);
+            grid_barrier_mono(a.bar, (unsigned)G * (++nbar) + a.unreach, a.err, 1, a.spin);
             if (*(volatile int*)a.err) return;
         }
     }
@@ -503,7 +507,7 @@ bool l2_f64_ok(const Geom& g, int num_sms) { return split_units(g.V, 2, num_sms)
 int launch_l2_f64(const double2* U64, const int* nbr, double2* const v[3], size_t vstep, double2* const w[3],
                   size_t wstep, KState* ks, double2* alpha, double2* beta, double2* gamma, double2* vscale, double mu,
                   double kappa, int k, double* partials, unsigned int* bar, const Geom& g, int num_sms,
-                  cudaStream_t st) {
+                  cudaStream_t st, long long spin, int unreachable) {
     const Split sp = split_units(g.V, 2, num_sms);
     if (sp.npass > L_MAXPASS) return (int)cudaErrorInvalidValue;
     L2Args a;
@@ -518,13 +522,14 @@ int launch_l2_f64(const double2* U64, const int* nbr, double2* const v[3], size_
     a.bar = bar;
     a.kappa = kappa, a.emu = exp(mu), a.emum = exp(-mu);
     a.V = g.V, a.k = k, a.npass = sp.npass;
+    a.spin = spin > 0 ? spin : LSPIN, a.unreach = unreachable ? 1u : 0u;
     static unsigned long long dev1 = 0, dev2 = 0;
     return sp.rs == 1 ? launch_coop(k_l2_f64<1>, a, sp, dev1, st) : launch_coop(k_l2_f64<2>, a, sp, dev2, st);
 }
 
 int launch_regen_f64(const double2* U64, const int* nbr, double2* const v[3], double2* y, const KState* ks,
                      const double2* coef, double mu, double kappa, unsigned int* bar, int* err, const Geom& g,
-                     int num_sms, cudaStream_t st) {
+                     int num_sms, cudaStream_t st, long long spin, int unreachable) {
     const Split sp = split_units(g.V, 4, num_sms);
     if (sp.npass > L_MAXPASS) return (int)cudaErrorInvalidValue;
     R64Args a;
@@ -538,6 +543,7 @@ int launch_regen_f64(const double2* U64, const int* nbr, double2* const v[3], do
     a.err = err;
     a.kappa = kappa, a.emu = exp(mu), a.emum = exp(-mu);
     a.V = g.V, a.npass = sp.npass;
+    a.spin = spin > 0 ? spin : LSPIN, a.unreach = unreachable ? 1u : 0u;
     static unsigned long long dev1 = 0, dev2 = 0;
     return sp.rs == 1 ? launch_coop(k_regen_f64<1>, a, sp, dev1, st) : launch_coop(k_regen_f64<2>, a, sp, dev2, st);
 }

@@ -329,7 +329,7 @@ class Context:
         return lam[0:2 * m:2] + 1j * lam[1:2 * m:2], R, L
 
     def set_wait_limit(self, polls: int = 0, unreachable: bool = False):
-        """Bounded device waits of the persistent pass 1 give up after `polls` polls (0: default);
+        """Bounded device waits of the persistent kernels give up after `polls` polls (0: default);
         unreachable=True makes every such wait run out (tests of the OVL_ETIMEOUT path)."""
         self._check(self._lib.ovl_set_wait_limit(self._h, int(polls), 1 if unreachable else 0))
 

@@ -83,3 +83,24 @@ def test_gradient_breakdown_orthogonal_upstream(ovl):
     with pytest.raises(ovl.OvlError) as e:
         ctx.sign_grad(100, c4["mu"], KAPPA, torch_c128(b), torch_c128(g))
     assert e.value.code == ovl.EBREAKDOWN
+
+
+@pytest.mark.parametrize("two_pass", [False, True])
+def test_timeout_fp64_then_usable(ovl, two_pass):
+    """The FP64 process (one cooperative launch) gives up in the same way, in a solve and in the gradient."""
+    c4 = config4()
+    ctx = _ctx(ovl, c4)
+    b, g = torch_c128(c4["b"]), torch_c128(synth.gaussian_source(c4["dims"], 78))
+    fl = ovl.TWO_PASS if two_pass else 0
+    ctx.set_wait_limit(1000, unreachable=True)
+    for call in (lambda: ctx.sign_krylov(ovl.LANCZOS2, 200, c4["mu"], KAPPA, b, flags=fl),
+                 lambda: ctx.sign_krylov(ovl.LANCZOS2, 200, c4["mu"], KAPPA, b, flags=fl | ovl.NO_GRAPH),
+                 lambda: ctx.sign_grad(200, c4["mu"], KAPPA, b, g)):
+        with pytest.raises(ovl.OvlError) as e:
+            call()
+        assert e.value.code == ovl.ETIMEOUT
+    ctx.set_wait_limit(0)
+    y, info = ctx.sign_krylov(ovl.LANCZOS2, 400, c4["mu"], KAPPA, b, flags=fl)
+    assert info["status"] == 0 and rel(y.cpu().numpy(), c4["ref"]) < 1e-10
+    _, info = ctx.sign_grad(400, c4["mu"], KAPPA, b, g)
+    assert info["status"] == 0
