@@ -102,5 +102,5 @@ def test_timeout_fp64_then_usable(ovl, two_pass):
     ctx.set_wait_limit(0)
     y, info = ctx.sign_krylov(ovl.LANCZOS2, 400, c4["mu"], KAPPA, b, flags=fl)
     assert info["status"] == 0 and rel(y.cpu().numpy(), c4["ref"]) < 1e-10
-    _, info = ctx.sign_grad(400, c4["mu"], KAPPA, b, g)
-    assert info["status"] == 0
+    gm, info = ctx.sign_grad(400, c4["mu"], KAPPA, b, g)  # (raises on any status but 0)
+    assert info["k_used"] > 300 and np.isfinite(gm)
