@@ -356,8 +356,9 @@ int enqueue_solve(ovl_ctx* c, int method, int k, double mu, double kappa, int fl
             if (lr) return fail(c, OVL_ECUDA, std::string("persistent pass 1 launch: ") +
                                                    cudaGetErrorString((cudaError_t)lr));
         }
-        // FP64 on lattices that fit the SMs' shared memory: the whole process in one launch as well
-        const bool persist64 = !mixed && !(flags & OVL_STEPWISE) && ovl::l2_f64_ok(g, c->num_sms);
+        // FP64 on lattices that fit the SMs' shared memory: the whole process in one launch as well; per-step
+        // kernels where the device does not take the launch
+        bool persist64 = !mixed && !(flags & OVL_STEPWISE) && ovl::l2_f64_ok(g, c->num_sms);
         if (persist64) {
             cudaMemsetAsync(c->bar, 0, 64, st);
             int lr = 0;
@@ -367,8 +368,13 @@ int enqueue_solve(ovl_ctx* c, int method, int k, double mu, double kappa, int fl
                                         c->gamma, c->vscale, mu, kappa, k, part, c->bar, g, c->num_sms, st,
                                         c->wait_polls, c->wait_unreachable);
             });
-            if (lr) return fail(c, OVL_ECUDA, std::string("persistent FP64 process launch: ") +
-                                                   cudaGetErrorString((cudaError_t)lr));
+            if (lr == (int)cudaErrorCooperativeLaunchTooLarge) {
+                cudaGetLastError();
+                persist64 = false;
+            } else if (lr) {
+                return fail(c, OVL_ECUDA, std::string("persistent FP64 process launch: ") +
+                                              cudaGetErrorString((cudaError_t)lr));
+            }
         }
         for (int i = 0; i < (persist || persist64 ? 0 : k); ++i) {
             if (mixed) {

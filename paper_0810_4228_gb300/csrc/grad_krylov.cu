@@ -754,14 +754,22 @@ extern "C" int ovl_sign_grad(ovl_ctx* c, int k, double mu, double kappa, const v
         }
         ovl::launch_native_f32_to_f64(V32, V, g, k, st);
         ovl::launch_native_f32_to_f64(W32, W, g, k, st);
-    } else if (ovl::l2_f64_ok(g, c->num_sms)) {
-        OVL_CUDA_TRY(c, cudaMemsetAsync(c->bar, 0, 64, st));
-        double2 *vv[3] = {V, nullptr, nullptr}, *ww[3] = {W, nullptr, nullptr};
-        if (ovl::launch_l2_f64(c->U64, c->nbr, vv, n, ww, n, ks, c->alpha, c->beta, c->gamma, c->vscale, mu, kappa, k,
-                               part, c->bar, g, c->num_sms, st, c->wait_polls, c->wait_unreachable))
-            return fail(c, OVL_ECUDA, "persistent FP64 process launch");
     } else {
-        for (int i = 0; i < k; ++i) {
+        bool persist = ovl::l2_f64_ok(g, c->num_sms);
+        if (persist) {
+            OVL_CUDA_TRY(c, cudaMemsetAsync(c->bar, 0, 64, st));
+            double2 *vv[3] = {V, nullptr, nullptr}, *ww[3] = {W, nullptr, nullptr};
+            const int lr = ovl::launch_l2_f64(c->U64, c->nbr, vv, n, ww, n, ks, c->alpha, c->beta, c->gamma, c->vscale,
+                                              mu, kappa, k, part, c->bar, g, c->num_sms, st, c->wait_polls,
+                                              c->wait_unreachable);
+            if (lr == (int)cudaErrorCooperativeLaunchTooLarge) {  // per-step kernels, as in the solve
+                cudaGetLastError();
+                persist = false;
+            } else if (lr) {
+                return fail(c, OVL_ECUDA, "persistent FP64 process launch");
+            }
+        }
+        for (int i = 0; i < (persist ? 0 : k); ++i) {
             const double2* vi = V + (size_t)i * n;
             const double2* wi = W + (size_t)i * n;
             ovl::launch_dslash_pair(c->U64, 0, vi, wi, c->t64, c->s64, mu, kappa, ks, c->alpha, i, k - 1, part, cnt, g,

@@ -28,11 +28,11 @@
 #include <algorithm>
 
 #include "hop64.cuh"
+#include "split64.h"
 
 namespace ovl {
 namespace {
 
-constexpr int LW = 16;             // warps per block
 constexpr int LT = 32 * LW;
 constexpr long long LSPIN = 20000000;  // default limit of a barrier wait's polls (a wait that gives up sets ks->timeout)
 
@@ -457,36 +457,20 @@ __global__ void __launch_bounds__(LT) k_regen_f64(R64Args a) {
     }
 }
 
-constexpr int L_MAXPASS = 4;  // passes whose state fits shared memory (57 KB of half spinors + 37 KB each)
+template <class A>
+using CoopKernel = void (*)(A);
 
-// Blocks (one per SM at most), passes over a block's warps, and the row split of a launch over V sites at
-// `spw` sites per warp unsplit.  RS = 2 halves the units' FP64 instructions (74 against 129 of the Lanczos
-// process's first phase) and doubles their number: better while it lowers the count of the busiest SM
-// quarter by more than it adds in all.
-struct Split {
-    int rs, G, npass;
-};
-Split split_units(int V, int spw, int num_sms) {
-    auto make = [&](int rs) {
-        const int units = (V + spw / rs - 1) / (spw / rs);
-        Split s;
-        s.rs = rs;
-        s.G = std::max(1, std::min(units, num_sms));
-        s.npass = ((units + s.G - 1) / s.G + LW - 1) / LW;
-        return s;
-    };
-    auto quarter = [&](const Split& s) {  // units of the busiest SM quarter
-        const int units = (V + spw / s.rs - 1) / (spw / s.rs);
-        return ((units + s.G - 1) / s.G + 3) / 4;
-    };
-    const Split one = make(1), two = make(2);
-    return two.npass == 1 && 74 * quarter(two) < 129 * quarter(one) ? two : one;
+// the shared-memory opt-in of a kernel, once per device (attr_dev: the kernel's own record of devices)
+template <class A>
+void allow_smem(CoopKernel<A> kern, int rs, unsigned long long& attr_dev) {
+    if (first_use_on_device(attr_dev))
+        cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)l2_smem(rs, L_MAXPASS));
 }
+unsigned long long l2_dev[2], regen_dev[2];  // k_l2_f64, k_regen_f64: RS = 1, 2
 
 template <class A>
-int launch_coop(void (*kern)(A), A args, const Split& sp, unsigned long long& attr_dev, cudaStream_t st) {
-    if (first_use_on_device(attr_dev))
-        cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)l2_smem(sp.rs, L_MAXPASS));
+int launch_coop(CoopKernel<A> kern, A args, const Split& sp, unsigned long long& attr_dev, cudaStream_t st) {
+    allow_smem(kern, sp.rs, attr_dev);
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(sp.G);
     cfg.blockDim = dim3(LT);
@@ -502,7 +486,20 @@ int launch_coop(void (*kern)(A), A args, const Split& sp, unsigned long long& at
 
 }  // namespace
 
-bool l2_f64_ok(const Geom& g, int num_sms) { return split_units(g.V, 2, num_sms).npass <= L_MAXPASS; }
+bool l2_f64_ok(const Geom& g, int num_sms) {
+    const Split sp = split_units(g.V, 2, num_sms);
+    if (sp.npass > L_MAXPASS) return false;
+    const CoopKernel<L2Args> kern = sp.rs == 1 ? k_l2_f64<1> : k_l2_f64<2>;
+    allow_smem(kern, sp.rs, l2_dev[sp.rs - 1]);
+    int dev = 0, coop = 0, per_sm = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess ||
+        cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev) != cudaSuccess ||
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, LT, l2_smem(sp.rs, sp.npass)) != cudaSuccess) {
+        cudaGetLastError();  // (the per-step kernels report what is wrong, if anything)
+        return false;
+    }
+    return split_fits(sp, num_sms, per_sm, coop != 0);
+}
 
 int launch_l2_f64(const double2* U64, const int* nbr, double2* const v[3], size_t vstep, double2* const w[3],
                   size_t wstep, KState* ks, double2* alpha, double2* beta, double2* gamma, double2* vscale, double mu,
@@ -523,8 +520,7 @@ int launch_l2_f64(const double2* U64, const int* nbr, double2* const v[3], size_
     a.kappa = kappa, a.emu = exp(mu), a.emum = exp(-mu);
     a.V = g.V, a.k = k, a.npass = sp.npass;
     a.spin = spin > 0 ? spin : LSPIN, a.unreach = unreachable ? 1u : 0u;
-    static unsigned long long dev1 = 0, dev2 = 0;
-    return sp.rs == 1 ? launch_coop(k_l2_f64<1>, a, sp, dev1, st) : launch_coop(k_l2_f64<2>, a, sp, dev2, st);
+    return sp.rs == 1 ? launch_coop(k_l2_f64<1>, a, sp, l2_dev[0], st) : launch_coop(k_l2_f64<2>, a, sp, l2_dev[1], st);
 }
 
 int launch_regen_f64(const double2* U64, const int* nbr, double2* const v[3], double2* y, const KState* ks,
@@ -544,8 +540,8 @@ int launch_regen_f64(const double2* U64, const int* nbr, double2* const v[3], do
     a.kappa = kappa, a.emu = exp(mu), a.emum = exp(-mu);
     a.V = g.V, a.npass = sp.npass;
     a.spin = spin > 0 ? spin : LSPIN, a.unreach = unreachable ? 1u : 0u;
-    static unsigned long long dev1 = 0, dev2 = 0;
-    return sp.rs == 1 ? launch_coop(k_regen_f64<1>, a, sp, dev1, st) : launch_coop(k_regen_f64<2>, a, sp, dev2, st);
+    return sp.rs == 1 ? launch_coop(k_regen_f64<1>, a, sp, regen_dev[0], st)
+                      : launch_coop(k_regen_f64<2>, a, sp, regen_dev[1], st);
 }
 
 }  // namespace ovl

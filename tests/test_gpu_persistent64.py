@@ -61,3 +61,15 @@ def test_fp64_zero_source(ovl):
     z = b * 0
     y, info = ctx.sign_krylov(ovl.LANCZOS2, 20, 0.3, KAPPA, z)
     assert info["k_used"] == 0 and not y.abs().max().item()
+
+
+@pytest.mark.parametrize("dims", [(13, 13, 8, 14), (16, 19, 8, 8), (13, 12, 10, 14)])
+def test_fp64_process_at_the_size_limit(ovl, dims):
+    """Four passes over a block's warps, the last of them partly empty; exactly the 19456 sites that the shared
+    memory of 152 SMs holds; and a lattice above, where both calls run the per-step kernels."""
+    ctx, b = _problem(ovl, dims)
+    for fl in (0, ovl.TWO_PASS):
+        y, i1 = ctx.sign_krylov(ovl.LANCZOS2, 12, 0.3, KAPPA, b, flags=fl)
+        s, i2 = ctx.sign_krylov(ovl.LANCZOS2, 12, 0.3, KAPPA, b, flags=fl | ovl.STEPWISE)
+        assert i1["k_used"] == i2["k_used"] == 12
+        assert rel(y.cpu().numpy(), s.cpu().numpy()) < 1e-10
