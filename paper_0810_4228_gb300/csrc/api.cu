@@ -744,7 +744,10 @@ int ovl_apply_Dw(ovl_ctx* c, double mu, double kappa, const void* x, void* y, in
     }
     const int vprec = prec == 0 ? 0 : 1;
     double2* yout = (flags & OVL_HOST) ? c->stage_out : (double2*)y;
-    if (prec == 0 && !(flags & (OVL_STENCIL_SITE | OVL_STENCIL_SPLIT))) {  // straight on canonical vectors
+    // FP64: straight on canonical vectors, unless x and y share memory (the kernel reads neighbours of x while it
+    // writes y; the way through the device layout has read all of x before it writes)
+    const bool apart = (uintptr_t)yout >= (uintptr_t)xin + cb || (uintptr_t)xin >= (uintptr_t)yout + cb;
+    if (prec == 0 && apart && !(flags & (OVL_STENCIL_SITE | OVL_STENCIL_SPLIT))) {
         ovl::launch_dslash_canon(c->U64, xin, yout, m, kappa, g5, c->g, c->st);
     } else {
         ovl::launch_pack_spinor(xin, c->nat_a, vprec, c->g, c->st);

@@ -32,3 +32,22 @@ def test_lanes_equal_sites(dims, bc_t):
         ctx.apply_Dw(0.3, KAPPA, xn, zn, flags=fl | ovl.NATIVE | ovl.STENCIL_SITE)
         assert float((yn - zn).abs().max()) < 1e-13 * top
     torch.cuda.synchronize()
+
+
+@pytest.mark.parametrize("shift", [12, -12, 1, 600])
+def test_canonical_vectors_that_share_memory(shift):
+    """x and y at different places of one buffer: the result is that of separate vectors.  Only the order of the
+    sums may differ (through the device layout or not): the bound of the forms above."""
+    import torch
+    from paper_0810_4228_gb300 import ovl
+    dims = (3, 5, 3, 4)
+    n = 12 * 3 * 5 * 3 * 4
+    ctx = ovl.Context(dims)
+    ctx.set_gauge(torch_c128(synth.gauge_field(dims, 1.0, 93)))
+    b = torch_c128(synth.gaussian_source(dims, 94))
+    ref = ctx.apply_Dw(0.3, KAPPA, b)
+    buf = torch.zeros(n + abs(shift), dtype=torch.complex128, device="cuda")
+    x, y = (buf[:n], buf[shift:]) if shift > 0 else (buf[-shift:], buf[:n])
+    x.copy_(b)
+    ctx.apply_Dw(0.3, KAPPA, x, y)
+    assert float((y - ref).abs().max()) < 1e-13 * float(ref.abs().max())
