@@ -229,11 +229,12 @@ int ovl_batch_solve(ovl_batch* batch, int k, double mu, double kappa, const void
  * ms3[0] pass 1 (the Krylov recurrence), ms3[1] the inner sign, ms3[2] the regeneration pass or the
  * combination; *nsolves the number of such solves.  reset != 0 clears the totals. */
 int ovl_batch_profile(ovl_batch* batch, double* ms3, int* nsolves, int reset);
-/* Launch shapes of the batched kernels.  The first solve in each precision times the candidates
+/* Launch shapes of the batched kernels.  The first solve in each precision (mixed: with each of the two
+ * regenerations, which share the pass-1 shape of the one that came first) times the candidates
  * (pass-1 site blocks of 64, 128 or 256 sites; the double-float regeneration kernel at 3 or 4 times
  * 128 threads per SM; the FP64 one at 3 to 6 blocks per SM with one sequence per block, or at 2 to 4
  * blocks per SM with two sequences of one lattice per block) with short eager solves of the batch itself and keeps the fastest (OVL_NO_TUNE skips
- * this).  The choice is cached per (GPU model, SM count, precision, lattice extents and
+ * this).  The choice is cached per (GPU model, SM count, precision and regeneration, lattice extents and
  * right-hand sides of every context): later batches of the same shape in the process take it
  * without timing, and when the environment variable OVL_TUNE_CACHE names a file the choices are
  * appended there ("key shape blocks_per_sm pair" lines) and read by later processes.  Writes the

@@ -1162,7 +1162,7 @@ struct ovl_batch {
     bool tuned = false;
     bool pinned = false;        // shapes set by ovl_batch_set_tuning: never retuned
     bool tune_cached = false;   // the shapes came from the tuning cache (no timing)
-    int tuned_mode = -1;
+    int tuned_kind = -1;        // tune_kind of the shapes
     std::vector<ovl::BSeq> hseq;
     std::vector<double2*> b64, bR, bL, pq;
     ovl::KState* ks = nullptr;
@@ -1610,14 +1610,18 @@ int enqueue_batch(ovl_batch* b, int k, double mu, double kappa, int flags, cudaS
 std::mutex g_tune_mu;
 std::map<std::string, std::array<int, 3>> g_tune;
 
-std::string tune_key(const ovl_batch* b) {
+// What the tuned shapes were timed with: the workspace mode, and in the mixed one which regeneration runs
+// (mode 3: the FP64 kernels of OVL_PASS2_F64, whose candidates and best shapes are others).
+int tune_kind(const ovl_batch* b, int flags) { return b->mode == 1 && (flags & OVL_PASS2_F64) ? 3 : b->mode; }
+
+std::string tune_key(const ovl_batch* b, int kind) {
     int dev = 0;
     cudaGetDevice(&dev);
     cudaDeviceProp pr{};
     cudaGetDeviceProperties(&pr, dev);
-    // ("/r2": the double-float regeneration of one thread per site; choices timed for the tile form that
-    // preceded it do not apply)
-    std::string k = std::string(pr.name) + "/" + std::to_string(pr.multiProcessorCount) + "/r2/m" + std::to_string(b->mode);
+    // ("/r3": the double-float regeneration of one thread per site, and the FP64 one under a key of its own;
+    // lines of other forms do not apply)
+    std::string k = std::string(pr.name) + "/" + std::to_string(pr.multiProcessorCount) + "/r3/m" + std::to_string(kind);
     for (size_t j = 0; j < b->ctx.size(); ++j) {
         const ovl::Geom& g = b->ctx[j]->g;
         k += "/" + std::to_string(g.L[0]) + "x" + std::to_string(g.L[1]) + "x" + std::to_string(g.L[2]) + "x" +
@@ -1659,8 +1663,8 @@ void tune_store(const std::string& key, const std::array<int, 3>& v) {
 // Autotuner of the batched kernels' launch shapes (site-block size of the pass-1 kernels, blocks
 // per SM of the regeneration kernel): each candidate runs a short eager solve (TUNE_K steps) of the
 // whole batch with events around its phases; the fastest pass-1 and regeneration candidates are
-// kept for the batch.  The sources must already be packed.
-int autotune(ovl_batch* b, double mu, double kappa, int flags, cudaStream_t st) {
+// kept for the batch.  The sources must already be packed.  fixed_shape >= 0: pass 1 keeps that shape.
+int autotune(ovl_batch* b, double mu, double kappa, int flags, int fixed_shape, cudaStream_t st) {
     if (b->kcap < 8) return OVL_OK;  // too short to time; the defaults stay until a longer solve
     const int TUNE_K = std::min(24, b->kcap);  // the workspace holds kcap steps
     const int saved_shape = b->shape, saved_minb = b->regen_minb;
@@ -1694,11 +1698,11 @@ int autotune(ovl_batch* b, double mu, double kappa, int flags, cudaStream_t st) 
                 if (t2 < best2) best2 = t2, bm = cand[c].minb, bp = cand[c].pair;
             }
         }
-    b->shape = bs;
+    b->shape = fixed_shape >= 0 ? fixed_shape : bs;
     b->regen_minb = bm;
     b->regen_pair = bp;
     b->tuned = true;
-    b->tuned_mode = b->mode;
+    b->tuned_kind = tune_kind(b, flags);
     if (b->exec) cudaGraphExecDestroy(b->exec);  // a captured graph holds the old shapes
     b->exec = nullptr;
     return OVL_OK;
@@ -1820,18 +1824,22 @@ int ovl_batch_solve(ovl_batch* b, int k, double mu, double kappa, const void* co
         }
     }
     // launch shapes: timed once per batch on its own data (short eager solves), unless OVL_NO_TUNE
-    if (!b->pinned && b->tuned_mode != mode && !(flags & OVL_NO_TUNE)) {
-        const std::string key = tune_key(b);
+    const int kind = tune_kind(b, flags);
+    if (!b->pinned && b->tuned_kind != kind && !(flags & OVL_NO_TUNE)) {
+        const std::string key = tune_key(b, kind);
         std::array<int, 3> v;
         if (tune_lookup(key, v)) {  // tuned before for this GPU, batch shape and precision
             b->shape = v[0], b->regen_minb = v[1], b->regen_pair = v[2];
             b->tuned = true;
-            b->tuned_mode = b->mode;
+            b->tuned_kind = kind;
             b->tune_cached = true;
             if (b->exec) cudaGraphExecDestroy(b->exec);
             b->exec = nullptr;
         } else {
-            r = autotune(b, mu, kappa, flags, st);
+            // both regenerations follow the same FP32 pass 1: its shape, and so its order of sums, is one choice
+            std::array<int, 3> other;
+            const bool shared = b->mode == 1 && tune_lookup(tune_key(b, kind == 1 ? 3 : 1), other);
+            r = autotune(b, mu, kappa, flags, shared ? other[0] : -1, st);
             if (r) return r;
             b->tune_cached = false;
             tune_store(key, {b->shape, b->regen_minb, b->regen_pair});

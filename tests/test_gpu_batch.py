@@ -406,3 +406,31 @@ def test_user_batch_recaptures_on_deflation_change(ovl):
     assert rel(y4, y8) > 1e-6  # the deflation size changes the k = 30 result
     bt.close()
     bt2.close()
+
+
+@pytest.mark.parametrize("order", [(0, 1), (1, 0)])
+def test_batch_tuning_per_regeneration(ovl, small, tmp_path, monkeypatch, order):
+    """The FP64 regeneration of a mixed batch (PASS2_F64) is tuned for itself, not with a shape timed for the
+    double-float one nor the other way round; both keep one pass-1 shape, and a later batch finds both."""
+    path = tmp_path / "tune.txt"
+    monkeypatch.setenv("OVL_TUNE_CACHE", str(path))
+    c = _ctx(ovl, small["dims"], small["U"])
+    nrhs = 6 + order[0]  # batch shapes no other test tunes
+    b = torch_c128(_sources(small["dims"], 4500, nrhs))
+    flags = [(ovl.MIXED, ovl.MIXED | ovl.PASS2_F64)[o] for o in order]
+    bt = ovl.Batch([c], [nrhs])
+    shapes, outs = [], []
+    for n, fl in enumerate(flags):
+        outs.append(bt.solve(40, small["mu"], KAPPA, [b], flags=fl)[0][0].cpu().numpy())
+        shapes.append(bt.tuning())
+        lines = path.read_text().splitlines()
+        assert len(lines) == n + 1 and len({ln.split()[0] for ln in lines}) == n + 1
+    assert shapes[0][0] == shapes[1][0]
+    bt2 = ovl.Batch([c], [nrhs])
+    for _ in range(2):  # back and forth on one batch: no new timing
+        for fl, sh, y in zip(flags, shapes, outs):
+            y2 = bt2.solve(40, small["mu"], KAPPA, [b], flags=fl)[0][0].cpu().numpy()
+            assert bt2.tuning() == sh and np.array_equal(y, y2)
+    assert len(path.read_text().splitlines()) == 2
+    bt.close()
+    bt2.close()
