@@ -1052,7 +1052,7 @@ __global__ void __launch_bounds__(8 * TT, MINB) k_b_regen(const BSeq* __restrict
 
 // The regeneration step for two sequences of the same lattice per block (work entry: the two
 // sequences, the tile, whether the second one exists): each hop warp loads the link and computes
-// the neighbour index once and runs the two sequences' double-float products as independent chains
+// the neighbour index once and runs the two sequences' FP64 products as independent chains
 // (twice the work in flight per warp); the epilogue spreads the 2 x 32 sites x 12 components over
 // the 256 threads, three each.  Same arithmetic per sequence as k_b_regen.
 template <int MINB>

@@ -434,3 +434,21 @@ def test_batch_tuning_per_regeneration(ovl, small, tmp_path, monkeypatch, order)
     assert len(path.read_text().splitlines()) == 2
     bt.close()
     bt2.close()
+
+
+def test_batch_fp64_two_sequence_regeneration_equals_one(ovl, mid):
+    """The FP64 regeneration with two sequences per block (the mixed default regenerates in double-float, one
+    kernel for both pins): equal to one per block, on several tiles, two lattices and an odd count."""
+    c4 = config4()
+    ca, cb = _ctx(ovl, c4["dims"], c4["U"]), _ctx(ovl, mid["dims"], mid["U"])
+    srcs = [torch_c128(_sources(c4["dims"], 4301, 2)), torch_c128(_sources(mid["dims"], 4302, 5))]
+    bt = ovl.Batch([ca, cb], [2, 5])
+    for fl in (ovl.MIXED | ovl.PASS2_F64, ovl.TWO_PASS):
+        for minb in (2, 3, 4):
+            ys = []
+            for seqs in (1, 2):
+                bt.set_tuning(128, minb, seqs)
+                ys.append([o.cpu().numpy() for o in bt.solve(300, c4["mu"], KAPPA, srcs, flags=fl)[0]])
+            for u, v in zip(*ys):
+                assert np.array_equal(u, v), (fl, minb)
+    bt.close()
