@@ -29,15 +29,16 @@
 #include <string>
 #include <vector>
 
-// Two-sided Lanczos passes near a breakdown for about one source in a hundred, and the result at a given k
-// then hangs on pass 1's roundings: between two orders of the FP32 products such a source's results differ by
-// 1e-9 to 1e-4 where all others agree to 1e-13.  A batch holds many sources, so its FP32 pass keeps the rounding
-// that it always had (chained multiply-adds would take 2 % off a batch of 48).
-#define OVL_F32_PRODUCTS_FIRST 1
 #include "ctx.h"
 #include "stencil_impl.cuh"
 
 namespace ovl {
+
+// Two-sided Lanczos passes near a breakdown for about one source in a hundred, and the result at a given k
+// then hangs on pass 1's roundings: between two orders of the FP32 products such a source's results differ by
+// 1e-9 to 1e-4 where all others agree to 1e-13.  A batch holds many sources, so its FP32 pass keeps the rounding
+// that it always had (chained multiply-adds would take 2 % off a batch of 48).
+template <class R> constexpr bool B_PF = sizeof(R) == 4;  // mul_link_pf
 
 // per-step coefficients of the double-float regeneration (see k_b_regen_coef)
 struct RegenCoefDf {
@@ -262,7 +263,7 @@ __global__ void __launch_bounds__(SHAPE_SITES[SH], LF == LINK_F64 ? 1 : 768 / SH
         const double2 scale = second ? ks->sw : ks->sv;
         const cx<R> cs = mk((R)scale.x, (R)scale.y);
         Spinor<R> acc[1], self;
-        apply_site<LF, R, 1>(q.g, site, q.U, xs, acc, hcs);
+        apply_site<LF, R, 1, false, B_PF<R>>(q.g, site, q.U, xs, acc, hcs);
         load_spinor(xs[0], q.g.V, site, self);
         finish_site(acc[0], self, true);
 #pragma unroll
@@ -514,7 +515,7 @@ __global__ void __launch_bounds__(BP1_T, 3) k_bp1(BP1Args a) {
             const float4* const xs[2] = {vi, wi};
             const HopCoef<float> hcs[2] = {a.hv, a.hw};
             Spinor<float> acc[2], self[2];
-            apply_site<LF, float, 2, true>(q.g, site, q.U, xs, acc, hcs);
+            apply_site<LF, float, 2, true, B_PF<float>>(q.g, site, q.U, xs, acc, hcs);
             load_spinor_cg(vi, V, site, self[0]);
             load_spinor_cg(wi, V, site, self[1]);
             finish_site(acc[0], self[0], true);

@@ -59,17 +59,6 @@ template <class R> OVL_HD void cfmac(cx<R>& a, cx<R> b, cx<R> c) {
     a.r = mad(b.i, c.i, mad(b.r, c.r, a.r));
     a.i = mad(-b.i, c.r, mad(b.r, c.i, a.i));
 }
-#ifdef OVL_F32_PRODUCTS_FIRST
-// The same with b c (or conj(b) c) formed first and added then, as batch.cu wants its FP32 products rounded.
-OVL_HD void cfma(cx<float>& a, cx<float> b, cx<float> c) {
-    a.r += b.r * c.r - b.i * c.i;
-    a.i += b.r * c.i + b.i * c.r;
-}
-OVL_HD void cfmac(cx<float>& a, cx<float> b, cx<float> c) {
-    a.r += b.r * c.r + b.i * c.i;
-    a.i += b.r * c.i - b.i * c.r;
-}
-#endif
 OVL_HD cx<double> up(cx<float> a) { return mk<double>(a.r, a.i); }
 OVL_HD cx<double> up(cx<double> a) { return a; }
 OVL_HD cx<double> d2c(double2 a) { return mk(a.x, a.y); }
@@ -220,6 +209,41 @@ OVL_HD void mul_link_dag(const Link<R>& U, const Half<R>& h, Half<R>& o) {
             cx<R> z = cdot(U.u[0][a], h.h[s][0]);
             cfmac(z, U.u[1][a], h.h[s][1]);
             cfmac(z, U.u[2][a], h.h[s][2]);
+            o.h[s][a] = z;
+        }
+}
+
+// The same with every product formed first and added then, as the batch wants its FP32 products rounded (the
+// forms above chain two fused multiply-adds per part).
+template <class R>
+OVL_HD void mul_link_pf(const Link<R>& U, const Half<R>& h, Half<R>& o) {
+#pragma unroll
+    for (int s = 0; s < 2; ++s)
+#pragma unroll
+        for (int a = 0; a < 3; ++a) {
+            cx<R> z = U.u[a][0] * h.h[s][0];
+#pragma unroll
+            for (int k = 1; k < 3; ++k) {
+                const cx<R> b = U.u[a][k], c = h.h[s][k];
+                z.r += b.r * c.r - b.i * c.i;
+                z.i += b.r * c.i + b.i * c.r;
+            }
+            o.h[s][a] = z;
+        }
+}
+template <class R>
+OVL_HD void mul_link_dag_pf(const Link<R>& U, const Half<R>& h, Half<R>& o) {
+#pragma unroll
+    for (int s = 0; s < 2; ++s)
+#pragma unroll
+        for (int a = 0; a < 3; ++a) {
+            cx<R> z = cdot(U.u[0][a], h.h[s][0]);
+#pragma unroll
+            for (int k = 1; k < 3; ++k) {
+                const cx<R> b = U.u[k][a], c = h.h[s][k];
+                z.r += b.r * c.r + b.i * c.i;
+                z.i += b.r * c.i - b.i * c.r;
+            }
             o.h[s][a] = z;
         }
 }

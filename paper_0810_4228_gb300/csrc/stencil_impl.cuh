@@ -46,8 +46,8 @@ __device__ __forceinline__ void load_spinor_any(const P* x, int V, int i, Spinor
 
 // The forward hop (1 + gamma_nu) U_{x,nu} psi(x + nu) of direction NU for NIN inputs
 // sharing the link (CG: L2-coherent vector loads, for vectors written by other
-// blocks of the same kernel).
-template <int NU, int LF, class R, int NIN, bool CG = false>
+// blocks of the same kernel; PF: see mul_link_pf).
+template <int NU, int LF, class R, int NIN, bool CG = false, bool PF = false>
 __device__ __forceinline__ void hop_fwd(const Geom& g, const Coord& c, int i, const void* U,
                                         const typename VecT<R>::T* const (&x)[NIN], Spinor<R> (&acc)[NIN],
                                         const HopCoef<R> (&hc)[NIN]) {
@@ -61,13 +61,14 @@ __device__ __forceinline__ void hop_fwd(const Geom& g, const Coord& c, int i, co
     for (int n = 0; n < NIN; ++n) {
         load_spinor_any<CG>(x[n], g.V, f, p);
         project<NU, +1>(p, h);
-        mul_link(L, h, uh);
+        if constexpr (PF) mul_link_pf(L, h, uh);
+        else mul_link(L, h, uh);
         recon_acc<NU, +1>(acc[n], uh, hc[n].f[NU] * ph);
     }
 }
 
 // The backward hop (1 - gamma_nu) U_{x-nu,nu}^dag psi(x - nu).
-template <int NU, int LF, class R, int NIN, bool CG = false>
+template <int NU, int LF, class R, int NIN, bool CG = false, bool PF = false>
 __device__ __forceinline__ void hop_bwd(const Geom& g, const Coord& c, int i, const void* U,
                                         const typename VecT<R>::T* const (&x)[NIN], Spinor<R> (&acc)[NIN],
                                         const HopCoef<R> (&hc)[NIN]) {
@@ -81,18 +82,19 @@ __device__ __forceinline__ void hop_bwd(const Geom& g, const Coord& c, int i, co
     for (int n = 0; n < NIN; ++n) {
         load_spinor_any<CG>(x[n], g.V, b, p);
         project<NU, -1>(p, h);
-        mul_link_dag(L, h, uh);
+        if constexpr (PF) mul_link_dag_pf(L, h, uh);
+        else mul_link_dag(L, h, uh);
         recon_acc<NU, -1>(acc[n], uh, hc[n].b[NU] * ph);
     }
 }
 
 // Both hops of direction NU.
-template <int NU, int LF, class R, int NIN, bool CG = false>
+template <int NU, int LF, class R, int NIN, bool CG = false, bool PF = false>
 __device__ __forceinline__ void hops_dir(const Geom& g, const Coord& c, int i, const void* U,
                                          const typename VecT<R>::T* const (&x)[NIN], Spinor<R> (&acc)[NIN],
                                          const HopCoef<R> (&hc)[NIN]) {
-    hop_fwd<NU, LF, R, NIN, CG>(g, c, i, U, x, acc, hc);
-    hop_bwd<NU, LF, R, NIN, CG>(g, c, i, U, x, acc, hc);
+    hop_fwd<NU, LF, R, NIN, CG, PF>(g, c, i, U, x, acc, hc);
+    hop_bwd<NU, LF, R, NIN, CG, PF>(g, c, i, U, x, acc, hc);
 }
 
 // One of the eight hops, h = 0..7: direction h & 3, forward for h < 4 (uniform per warp).
@@ -196,8 +198,8 @@ __device__ __forceinline__ cx<R> hop_spin(int h, int sp, const cx<R>& h0, const 
 }
 
 // The hopping term of site i for NIN inputs (CG: L2-coherent vector loads, for vectors written by
-// other blocks of the same kernel).
-template <int LF, class R, int NIN, bool CG = false>
+// other blocks of the same kernel; PF: how the link's products are rounded, see mul_link_pf).
+template <int LF, class R, int NIN, bool CG = false, bool PF = false>
 __device__ __forceinline__ void apply_site(const Geom& g, int i, const void* U,
                                            const typename VecT<R>::T* const (&x)[NIN], Spinor<R> (&acc)[NIN],
                                            const HopCoef<R> (&hc)[NIN]) {
@@ -208,10 +210,10 @@ __device__ __forceinline__ void apply_site(const Geom& g, int i, const void* U,
         for (int s = 0; s < 4; ++s)
 #pragma unroll
             for (int a = 0; a < 3; ++a) acc[n].s[s][a] = mk(R(0), R(0));
-    hops_dir<0, LF, R, NIN, CG>(g, c, i, U, x, acc, hc);
-    hops_dir<1, LF, R, NIN, CG>(g, c, i, U, x, acc, hc);
-    hops_dir<2, LF, R, NIN, CG>(g, c, i, U, x, acc, hc);
-    hops_dir<3, LF, R, NIN, CG>(g, c, i, U, x, acc, hc);
+    hops_dir<0, LF, R, NIN, CG, PF>(g, c, i, U, x, acc, hc);
+    hops_dir<1, LF, R, NIN, CG, PF>(g, c, i, U, x, acc, hc);
+    hops_dir<2, LF, R, NIN, CG, PF>(g, c, i, U, x, acc, hc);
+    hops_dir<3, LF, R, NIN, CG, PF>(g, c, i, U, x, acc, hc);
 }
 
 // add the diagonal term and apply gamma5 = diag(1, 1, -1, -1)
