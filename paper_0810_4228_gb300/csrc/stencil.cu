@@ -435,7 +435,8 @@ void launch_dslash(const void* U, int prec, const void* x, void* y, double mu, d
 // Both kinds of block run the same copy of the stencil (34 KB of instructions): with a copy each, warps of
 // the two kinds on one SM waited for instructions a quarter of the time (32^4, FP32: 296 -> 230 us; 48^3 x 64:
 // 1843 -> 1387 us).  Bound by issue slots and load latency, at 2.8 TB/s of its own operands.
-template <int LF, bool ROWS>
+// WIDE: FP32 data summed in FP64 (its exact products too), as the direction split does.
+template <int LF, bool ROWS, bool WIDE = false>
 __global__ void __launch_bounds__(128, LF == LINK_F64 ? 2 : OVL_DSLASH_F32_MINB) k_dslash_pair(const void* __restrict__ U,
                                                      const typename VecT<typename LinkReal<LF>::R>::T* __restrict__ v,
                                                      const typename VecT<typename LinkReal<LF>::R>::T* __restrict__ w,
@@ -451,9 +452,9 @@ __global__ void __launch_bounds__(128, LF == LINK_F64 ? 2 : OVL_DSLASH_F32_MINB)
     const double2 sv = ks->sv, sw = ks->sw;
     const int which = (int)(blockIdx.x & 1u);
     const int i = ROWS ? site_of_rows(g, blockIdx.x >> 1, gridDim.x >> 1) : site_of_block(g, blockIdx.x >> 1);
-    // per-thread sums: FP64 for FP64 data; for FP32 data exact FP32 products summed as compensated
+    // per-thread sums: FP64 for FP64 data and with WIDE; otherwise exact FP32 products summed as compensated
     // FP32 pairs (TwoSum) on the FP32 pipe, widened to FP64 for the block and grid sums
-    using A = typename std::conditional<sizeof(R) == 4, AccF, AccD>::type;
+    using A = typename std::conditional<sizeof(R) == 4 && !WIDE, AccF, AccD>::type;
     A pa[3];
     if (i >= 0) {  // t = sv A v~, partials of w~^dag t and |t|^2; or s = sw A^dag w~
         const typename VecT<R>::T* const xs[1] = {which ? w : v};
@@ -476,8 +477,13 @@ __global__ void __launch_bounds__(128, LF == LINK_F64 ? 2 : OVL_DSLASH_F32_MINB)
             for (int sp = 0; sp < 4; ++sp)
 #pragma unroll
                 for (int a = 0; a < 3; ++a) {
-                    acc_cdot(pa, self.s[sp][a], acc[0].s[sp][a]);  // w~^dag t
-                    acc_norm2(pa[2], acc[0].s[sp][a]);
+                    if constexpr (WIDE) {
+                        acc_cdot(pa, up(self.s[sp][a]), up(acc[0].s[sp][a]));
+                        acc_norm2(pa[2], up(acc[0].s[sp][a]));
+                    } else {
+                        acc_cdot(pa, self.s[sp][a], acc[0].s[sp][a]);  // w~^dag t
+                        acc_norm2(pa[2], acc[0].s[sp][a]);
+                    }
                 }
         }
     }
@@ -485,7 +491,7 @@ __global__ void __launch_bounds__(128, LF == LINK_F64 ? 2 : OVL_DSLASH_F32_MINB)
     double part[3];
 #pragma unroll
     for (int j = 0; j < 3; ++j) {
-        if constexpr (sizeof(R) == 4) part[j] = (double)pa[j].hi + (double)pa[j].lo;
+        if constexpr (sizeof(R) == 4 && !WIDE) part[j] = (double)pa[j].hi + (double)pa[j].lo;
         else part[j] = pa[j].v;
     }
     double out[3];
@@ -507,9 +513,10 @@ __global__ void __launch_bounds__(128, LF == LINK_F64 ? 2 : OVL_DSLASH_F32_MINB)
 
 // The pair's two stencils run in one launch, so one thread per site and stencil is the faster form from few
 // sites on (us of the call, FP32 / FP64, against the direction split: 4096 sites 30.6 / 66.7 against 31.0 / 48.2,
-// 8748 31.1 / 67.7 against 34.7 / 67.7, 20736 34.8 / 130 against 52.9 / 131, 65536 43.8 / 270 against 80.3 / 308).
-// The FP32 form sums alpha in compensated pairs (48 bits; the FP32 rounding of t itself, which both forms share,
-// is what alpha's error is made of).
+// 8748 40.3 / 67.7 against 42.2 / 67.7, 20736 50.2 / 130 against 57.6 / 131, 65536 68.2 / 270 against 88.7 / 308, 118800 82.7
+// against 129.5 in FP32).  Both forms sum alpha and |t|^2 in FP64 there (WIDE): in compensated FP32 pairs the call took
+// 38.1, 38.8, 49.4 and 63.0 us, but alpha's error rose from 1e-18 to 1e-17 of the terms' magnitudes, and products of
+// small or large vectors left the FP32 range.
 static bool pair_ds(const Geom& g) { return g_ds_mode < 0 ? g.V < (1 << 13) : g_ds_mode == 1; }
 // The allocation-free call answers for its grid (ovl_apply_pair_noalloc_blocks) and keeps the one it had.
 int dslash_pair_blocks(const Geom& g) { return pick_ds(g) ? ds_grid(g) : dslash_grid(g, 128); }
@@ -550,14 +557,16 @@ void launch_dslash_pair(const void* U, int prec, const void* v, const void* w, v
                 U, (const double2*)v, (const double2*)w, (double2*)t, (double2*)s, make_coef<double>(mu, kappa),
                 make_coef<double>(-mu, kappa), ks, alpha, step, klast, partials, counter, g);
     } else {
+        const bool wide = use_ds(g);  // up to the volume where the other forms of the call sum in FP64 (pair_ds)
+        auto go = [&](auto kern, dim3 grid) {
+            kern<<<grid, T, 0, st>>>(U, (const float4*)v, (const float4*)w, (float4*)t, (float4*)s,
+                                     make_coef<float>(mu, kappa), make_coef<float>(-mu, kappa), ks, alpha, step, klast,
+                                     partials, counter, g);
+        };
         if (rg.ok)
-            k_dslash_pair<LINK_F32_12, true><<<rg.grid, T, 0, st>>>(
-                U, (const float4*)v, (const float4*)w, (float4*)t, (float4*)s, make_coef<float>(mu, kappa),
-                make_coef<float>(-mu, kappa), ks, alpha, step, klast, partials, counter, g);
+            go(wide ? k_dslash_pair<LINK_F32_12, true, true> : k_dslash_pair<LINK_F32_12, true>, rg.grid);
         else
-            k_dslash_pair<LINK_F32_12, false><<<g1, T, 0, st>>>(
-                U, (const float4*)v, (const float4*)w, (float4*)t, (float4*)s, make_coef<float>(mu, kappa),
-                make_coef<float>(-mu, kappa), ks, alpha, step, klast, partials, counter, g);
+            go(wide ? k_dslash_pair<LINK_F32_12, false, true> : k_dslash_pair<LINK_F32_12, false>, g1);
     }
 }
 

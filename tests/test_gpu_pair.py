@@ -36,3 +36,24 @@ def test_pair_equals_single_applications(dims, prec):
     a, b = w.cpu().numpy().astype(np.complex128), t.cpu().numpy().astype(np.complex128)
     ref = np.vdot(a, b)
     assert abs(alpha - ref) <= 12 * math.prod(dims) * 2.0 ** -48 * np.linalg.norm(a) * np.linalg.norm(b)
+
+
+@pytest.mark.parametrize("scale", [1.0, 1e-21, 1e21])
+@pytest.mark.parametrize("dims", [(8, 8, 8, 8), (9, 9, 9, 12), (16, 12, 16, 16)])
+def test_fp32_pair_sums_alpha_in_fp64(dims, scale):
+    """Below 155648 sites alpha is an FP64 sum of the FP32 vectors' products in both forms of the kernel: vectors
+    whose products leave the FP32 range, and 100 roundings of 2^-53 of the sum of the terms' magnitudes (48 per
+    thread, the block's and the grid's trees), which is at most 2 |w| |t|."""
+    import torch
+    from paper_0810_4228_gb300 import ovl
+    ctx = ovl.Context(dims)
+    ctx.set_gauge(torch_c128(synth.gauge_field(dims, 1.0, 95)))
+    v, w = (ctx.empty_native(1) for _ in range(2))
+    ctx.pack(torch_c128(scale * synth.gaussian_source(dims, 98)), v, 1)
+    ctx.pack(torch_c128(scale * synth.gaussian_source(dims, 99)), w, 1)
+    t, s = (torch.full_like(v, float("nan")) for _ in range(2))
+    alpha = ctx.apply_pair(0.25, KAPPA, v, w, t, s, 1)
+    a, b = (x.cpu().numpy().astype(np.clongdouble) for x in (w, t))
+    ref = (a.conj() * b).sum()
+    size = float(np.sqrt((np.abs(a) ** 2).sum()) * np.sqrt((np.abs(b) ** 2).sum()))
+    assert abs(complex(alpha - complex(ref))) <= 100 * 2.0 ** -53 * 2 * size
