@@ -703,10 +703,12 @@ extern "C" int ovl_sign_grad(ovl_ctx* c, int k, double mu, double kappa, const v
     // ---- workspace: W (k + 1 vectors), Z (k vectors), g_y packed, link gradient, scalars
     const size_t kk1 = (size_t)k + 1;
     // (mixed: the FP32 bases, (k + 1) vectors of n complex64 each, after the FP64 ones)
-    // (FP64: the shares of the link force after everything else)
+    // (FP64: the shares of the link force after everything else; one share, the form of the large lattices, goes
+    // where the mixed form keeps its device-layout links and the scratch vector of grad_b, 36 V + 12 V of its 45 V)
     const int nsplit = mixed ? 0 : ovl::force_splits(g, k, c->num_sms);
+    const size_t shares_extra = nsplit > 1 ? (size_t)nsplit * 45 * g.V : 0;
     const size_t need = ((2 * kk1 + 1 + 3 + 1) * n + 4 * kk1 + (size_t)k * k + 64) * sizeof(double2) +
-                        (mixed ? 2 * kk1 * n * sizeof(float2) : (size_t)nsplit * 45 * g.V * sizeof(double2));
+                        (mixed ? 2 * kk1 * n * sizeof(float2) : shares_extra * sizeof(double2));
     if (c->gwork_bytes < need) {
         if (c->gwork) cudaFree(c->gwork);
         c->gwork = nullptr;
@@ -866,7 +868,7 @@ extern "C" int ovl_sign_grad(ovl_ctx* c, int k, double mu, double kappa, const v
         } else {
             ovl::k_gq_combine_df<<<gz, 256, 0, st>>>(W, M, Z, kk, n);
             const int B32 = (g.V + 31) / 32, nsp = std::min(nsplit, kk);
-            double2* shares = misc + 32;
+            double2* shares = nsplit > 1 ? misc + 32 : gUd;
             ovl::k_force_part<<<dim3(B32, nsp), 128, 0, st>>>(V, Z, kk, shares, g);
             ovl::k_force_reduce<<<B32, 128, 0, st>>>(c->U64, shares, nsp, (double2*)grad_U, kappa, std::exp(mu),
                                                      std::exp(-mu), g, part, cnt, gmu_acc);

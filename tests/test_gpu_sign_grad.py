@@ -204,3 +204,30 @@ def test_sign_grad_8x4_vs_central_differences(mods):
     assert abs(gmu - fd_mu) <= 1e-5 * abs(fd_mu), (gmu, fd_mu)
     assert abs(got_U - fd_U) <= 1e-5 * abs(fd_U), (got_U, fd_U)
     lat.close()
+
+
+def test_gradient_workspace_of_a_large_lattice():
+    """On lattices that fill the SMs the pairs' force has one share, which needs no memory beyond the workspace of
+    (2 k + 7) vectors: k = 4 on 16^3 x 8, where a share of its own would take 24 MB more."""
+    import torch
+    from paper_0810_4228_gb300 import ovl
+    mu, k = 0.2, 4
+
+    def inputs(dims):
+        ctx = ovl.Context(dims)
+        ctx.set_gauge(torch_c128(synth.gauge_field(dims, 0.5, 71)))
+        b, g = torch_c128(synth.gaussian_source(dims, 72)), torch_c128(synth.gaussian_source(dims, 73))
+        return ctx, b, g, torch.empty((int(np.prod(dims)), 4, 3, 3), dtype=torch.complex128, device="cuda")
+
+    ctx, b, g, gU = inputs((4, 4, 4, 4))  # loads the kernels
+    ctx.sign_krylov(ovl.LANCZOS2, 40, mu, KAPPA, b)
+    ctx.sign_grad(40, mu, KAPPA, b, g, grad_U=gU)
+    ctx, b, g, gU = inputs((16, 16, 16, 8))
+    ctx.sign_krylov(ovl.LANCZOS2, k, mu, KAPPA, b)
+    torch.cuda.synchronize()
+    free = torch.cuda.mem_get_info()[0]
+    ctx.sign_grad(k, mu, KAPPA, b, g, grad_U=gU)
+    used = free - torch.cuda.mem_get_info()[0]
+    n = 12 * 16 ** 3 * 8
+    quad = 6 * k * 10240 * 16  # the quadrature's scratch at its finest level
+    assert used <= (2 * (k + 1) + 5) * n * 16 + quad + (8 << 20)  # and 8 MB of allocation granularity
