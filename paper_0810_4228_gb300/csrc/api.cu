@@ -420,7 +420,7 @@ int enqueue_solve(ovl_ctx* c, int method, int k, double mu, double kappa, int fl
             prof(c, KC_INNER, [&] {
                 r = ovl::launch_inner_newton(c->alpha, c->beta, c->gamma, nullptr, 0, 1, ks, c->cvec, c->inner,
                                              c->inner_elems, c->kcap, c->num_sms, st);
-            }, 2);
+            }, ovl::inner_sign_kernels(false));
         else
             prof(c, KC_INNER, [&] {
                 r = ovl::launch_inner_quadrature(c->alpha, c->beta, c->gamma, ks, c->cvec, c->inner,
@@ -429,7 +429,7 @@ int enqueue_solve(ovl_ctx* c, int method, int k, double mu, double kappa, int fl
                 if (!r)
                     r = ovl::launch_inner_newton(c->alpha, c->beta, c->gamma, nullptr, 0, 1, ks, c->cvec, c->inner,
                                                  c->inner_elems, c->kcap, c->num_sms, st, 1);
-            }, 15);
+            }, ovl::inner_sign_kernels(true));
         if (r) return fail(c, OVL_ECUDA, "inner sign launch failed");
         // combination y += |b_perp^R| V_k sgn(G_k) e_1
         if (twopass && persist) {
@@ -506,7 +506,7 @@ int enqueue_solve(ovl_ctx* c, int method, int k, double mu, double kappa, int fl
             prof(c, KC_ANORM, [&] { ovl::launch_adf_normalize(t, x64, ks, n, st); });
         }
         int r = 0;
-        prof(c, KC_INNER, [&] { r = arnoldi_inner_sign(c, ldH, flags); }, (flags & OVL_INNER_NEWTON) ? 2 : 15);
+        prof(c, KC_INNER, [&] { r = arnoldi_inner_sign(c, ldH, flags); }, ovl::inner_sign_kernels(!(flags & OVL_INNER_NEWTON)));
         if (r) return fail(c, OVL_ECUDA, "inner sign launch failed");
         prof(c, KC_COMBINE, [&] { ovl::launch_adf_combine(Vd, n, c->cvec, cdf, ks, c->kcap, c->y64, n, st); }, 2);
     } else {  // Arnoldi
@@ -530,7 +530,7 @@ int enqueue_solve(ovl_ctx* c, int method, int k, double mu, double kappa, int fl
             prof(c, KC_ANORM, [&] { ovl::launch_arnoldi_normalize(t, ks, n, st); });
         }
         int r = 0;
-        prof(c, KC_INNER, [&] { r = arnoldi_inner_sign(c, ldH, flags); }, (flags & OVL_INNER_NEWTON) ? 2 : 15);
+        prof(c, KC_INNER, [&] { r = arnoldi_inner_sign(c, ldH, flags); }, ovl::inner_sign_kernels(!(flags & OVL_INNER_NEWTON)));
         if (r) return fail(c, OVL_ECUDA, "inner sign launch failed");
         prof(c, KC_COMBINE, [&] { ovl::launch_combine(c->V64, n, nullptr, c->cvec, ks, c->kcap, c->y64, n, st); });
     }
@@ -602,7 +602,7 @@ int enqueue_restarted(ovl_ctx* c, int rs, int cycles, double mu, double kappa, i
                 r = ovl::launch_inner_newton(nullptr, nullptr, nullptr, c->Hrs, ldH, 0, ks, c->cvrs, c->innrs,
                                              c->innrs_elems, c->krs_cap, c->num_sms, st);
             }
-        }, (flags & OVL_INNER_NEWTON) ? 2 : 15);
+        }, ovl::inner_sign_kernels(!(flags & OVL_INNER_NEWTON)));
         if (r) return fail(c, OVL_ECUDA, "inner sign launch failed");
         prof(c, KC_COMBINE, [&] { ovl::launch_rs_combine(Vd, n, c->cvrs, cyc * rs, cdf, ks, rs, c->y64, n, st); }, 2);
         prof(c, KC_ANORM, [&] { ovl::launch_rs_restart(Vd, n, rs, h1d, x64, ks, n, cyc + 1 == cycles, st); });

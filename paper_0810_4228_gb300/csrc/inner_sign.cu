@@ -324,6 +324,10 @@ __global__ void k_quad_sum(const double2* __restrict__ work, double2* __restrict
     }
 }
 
+// kernels of an inner sign: the quadrature's preparation, a solve and a sum per level (the first two levels'
+// solves in one launch), and Newton's two behind it
+int inner_sign_kernels(bool quadrature) { return quadrature ? 1 + 2 * QUAD_LEVELS - 1 + 2 : 2; }
+
 static void quad_launch(const double2* alpha, const double2* beta, const double2* gamma, KState* ks, double2* c,
                         double2* work, int kmax, double* partials, unsigned int* counter, int nseq, QStride qs,
                         cudaStream_t st) {

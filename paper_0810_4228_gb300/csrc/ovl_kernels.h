@@ -187,6 +187,8 @@ int launch_regen_f64(const double2* U64, const int* nbr, double2* const v[3], do
                      int num_sms, cudaStream_t st, long long spin = 0, int unreachable = 0);
 
 // ---- inner_sign.cu
+// kernels one inner sign queues (the profile's counts), with the quadrature or by Newton alone
+int inner_sign_kernels(bool quadrature);
 // c[0..n) = nR * sgn(H) e_1 for the upper Hessenberg H (column-major, leading dimension ldH) of
 // size ks->kused, by the same quadrature with Givens-rotation solves of the shifted Hessenberg
 // systems; needs inner_work_elems(kmax, 2) elements of work and kmax * 16 bytes of shared memory

@@ -400,3 +400,20 @@ def test_double_float_pass2_matches_fp64_pass2(ovl, c4, k):
     y_df, _ = _solve(ovl, ctx, ovl.LANCZOS2, k, c4["mu"], c4["b"], flags=ovl.MIXED | ovl.PASS2_DF)
     y_64, _ = _solve(ovl, ctx, ovl.LANCZOS2, k, c4["mu"], c4["b"], flags=ovl.MIXED)
     assert rel(y_df, y_64) < 1e-11
+
+
+def test_profile_counts_inner_sign_kernels():
+    """The profile's kernel count of the inner sign: preparation, five solves (levels 0 and 1 together) and six sums,
+    Newton's two kernels behind them; Newton alone two."""
+    from paper_0810_4228_gb300 import ovl
+    c4 = config4()
+    ctx = ovl.Context(c4["dims"])
+    ctx.set_gauge(torch_c128(c4["U"]))
+    b = torch_c128(c4["b"])
+    for method, fl in ((ovl.LANCZOS2, 0), (ovl.LANCZOS2, ovl.MIXED), (ovl.ARNOLDI, 0), (ovl.ARNOLDI, ovl.MIXED)):
+        for nf, count in ((0, 14), (ovl.INNER_NEWTON, 2)):
+            ctx.profile()
+            ctx.sign_krylov(method, 60, c4["mu"], KAPPA, b, flags=fl | nf | ovl.PROFILE)
+            assert ctx.profile()["inner_sign"]["kernels"] == count, (method, fl, nf)
+    ctx.sign_arnoldi_restarted(20, 3, c4["mu"], KAPPA, b, flags=ovl.PROFILE)
+    assert ctx.profile()["inner_sign"]["kernels"] == 3 * 14
