@@ -452,7 +452,7 @@ __global__ void __launch_bounds__(AD_T, 4) k_adf_dot2(const float4* __restrict__
 
 // (2), one block of 256 threads.  h1 = (c, rho^2) and h2 = (d, e) of step j (h2 unused when fin).  Finishes
 // column j-1 of H (j >= 1), decides a lucky breakdown (nu <= bdtol |H|) and for the update writes
-// ks->red[1] = (1 / nu, nu), ks->red[2] = r, ks->red[3].x != 0 where |c| <= 2^-30 rho.  fin = 1 after the
+// ks->red[1] = (1 / nu, nu), ks->red[2] = r.  fin = 1 after the
 // last step (j = k): only column k-1 is finished and the solve is marked done.  fin = 2 at the end of a
 // restart cycle: column k-1 is finished and ks->red[1] written for the next cycle's start vector
 // (u_k - V c) / nu, and the solve goes on unless the Krylov space is invariant.
@@ -529,7 +529,6 @@ __device__ __forceinline__ void dcgs_block(double2* __restrict__ H, int ldH, con
         const double2 e = __ldcg(h2 + j);
         const double i2 = inu * inu;
         ks->red[2] = make_double2((e.x - er) * i2, (e.y - ei) * i2);
-        ks->red[3] = make_double2(c2 <= 0x1p-60 * rho2 ? 1.0 : 0.0, 0.0);
     }
 }
 
@@ -587,14 +586,13 @@ __global__ void __launch_bounds__(DC_T) k_adf_dot2_reduce(const double2* __restr
 // j + 1 and, as FP64, into x64 (the next stencil's input).  The first hb blocks write the tentative column j
 // of H, a warp per row: H[i, j] = d_i / nu - g_i (i < j), r - c_{j-1} (i = j), g_i = sum_{l >= i-1} H[i, l] c_l / nu (upper
 // Hessenberg rows of the final columns).
-// Bound by loads in flight (3.8 TB/s of basis).  All sweeps of k = 450 on 8^4: 30.1 ms with both sums scalar,
-// 21.4 ms so.
-// c is what the first projection left behind, 2^-40 of u_j or less while Gram-Schmidt works: with
-// |c| <= 2^-30 rho (ks->red[3], the same in every block) s1 is formed in FP32 from the leading parts, which
-// leaves an error below 2^-50 of u_j, under the double-float rounding of u_j itself; otherwise in
-// double-float like s2.
-static constexpr int UP_CH = 512;  // coefficients staged in shared memory at a time
-__global__ void __launch_bounds__(AD_T, 3) k_adf_update2(const float4* __restrict__ V, size_t ld, int j, int cold, int hb,
+// Bound by the FP32 pipe (48 packed operations per term, both sums double-float) beside 16 bytes of basis per term.
+// Solve of k = 450 on 8^4: 56.5 ms (71.2 with scalar sums); two vectors per round at 32 warps per SM, against 56.6 with
+// four at 24 warps, 57.5 with two at 24, 58.7 and 59.2 with four and eight at 16.  (The c sum in FP32 from the
+// leading parts, where |c| is small, takes 51.8: not kept, it is less than the basis's precision.)
+static constexpr int UP_CH = 512;  // coefficients staged in shared memory at a time (a multiple of UP_NV x AD_W)
+static constexpr int UP_NV = 2;   // vectors per warp and round
+__global__ void __launch_bounds__(AD_T, 4) k_adf_update2(const float4* __restrict__ V, size_t ld, int j, int cold, int hb,
                                                          const float4* __restrict__ cdf, const float4* __restrict__ ddf,
                                                          float4* __restrict__ uj, float4* __restrict__ unext,
                                                          const double2* __restrict__ w, double2* __restrict__ x64,
@@ -603,13 +601,11 @@ __global__ void __launch_bounds__(AD_T, 3) k_adf_update2(const float4* __restric
                                                          size_t n, KState* ks) {
     __shared__ float4 red1[AD_W][32];
     __shared__ float4 red2[AD_W][32];
-    __shared__ float4 dsm[UP_CH];
-    __shared__ float2 csm[UP_CH];
+    __shared__ float4 csm[UP_CH], dsm[UP_CH];
     if (ks->done || ks->status) return;
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     const double inu = ks->red[1].x;
     const double2 r = ks->red[2];
-    const bool small = ks->red[3].x != 0.0;
     if ((int)blockIdx.x < hb) {  // a warp per row of H
         const int i = blockIdx.x * AD_W + wid;
         if (i > j) return;
@@ -641,64 +637,46 @@ __global__ void __launch_bounds__(AD_T, 3) k_adf_update2(const float4* __restric
     for (size_t tile = blockIdx.x - hb; tile < ntile; tile += gridDim.x - hb) {
         const size_t e = tile * 32 + lane;
         const bool in = e < n;
-        PAcc a2;
+        PAcc a1, a2;
+        pacc_zero(a1);
         pacc_zero(a2);
-        cx<df> s1 = mk(df(0), df(0));
-        if (small) {
-            float2 fa = make_float2(0.f, 0.f), fb = fa;
-            // four vectors of this warp per round, the next round's loads in flight meanwhile
-            const float4 zero = make_float4(0.f, 0.f, 0.f, 0.f);
-            const float4* Ve = V + e;
-            auto load4 = [&](int l, float4 (&v)[4]) {
+        // UP_NV vectors of this warp per round, the next round's loads in flight meanwhile
+        const float4 zero = make_float4(0.f, 0.f, 0.f, 0.f);
+        const float4* Ve = V + e;
+        auto load = [&](int l, float4 (&v)[UP_NV]) {
 #pragma unroll
-                for (int q = 0; q < 4; ++q) {
-                    const float4* p = Ve + (size_t)(l + q * AD_W) * ld;
-                    v[q] = !in || l + q * AD_W >= j ? zero : l < cold ? ldg_hint(p, pol) : __ldg(p);
-                }
-            };
-            float4 v[4];
-            load4(wid, v);
-            for (int l0 = 0; l0 < j; l0 += UP_CH) {
-                if (l0 > 0 || tile + hb != blockIdx.x) __syncthreads();  // the last chunk has been read
-                for (int l = threadIdx.x; l < UP_CH; l += AD_T) {
-                    const bool ok = l0 + l < j;
-                    dsm[l] = ok ? __ldg(ddf + l0 + l) : zero;
-                    csm[l] = ok ? __ldg(reinterpret_cast<const float2*>(cdf + l0 + l)) : make_float2(0.f, 0.f);
-                }
-                __syncthreads();
-                const int lim = min(UP_CH, j - l0);
-                for (int l = wid; l < lim; l += 4 * AD_W) {
-                    float4 nx[4];
-                    load4(l0 + l + 4 * AD_W, nx);
+            for (int q = 0; q < UP_NV; ++q) {
+                const float4* p = Ve + (size_t)(l + q * AD_W) * ld;
+                v[q] = !in || l + q * AD_W >= j ? zero : l < cold ? ldg_hint(p, pol) : __ldg(p);
+            }
+        };
+        float4 v[UP_NV];
+        load(wid, v);
+        for (int l0 = 0; l0 < j; l0 += UP_CH) {
+            if (l0 > 0 || tile + hb != blockIdx.x) __syncthreads();  // the last chunk has been read
+            for (int l = threadIdx.x; l < UP_CH; l += AD_T) {
+                const bool ok = l0 + l < j;
+                csm[l] = ok ? __ldg(cdf + l0 + l) : zero;
+                dsm[l] = ok ? __ldg(ddf + l0 + l) : zero;
+            }
+            __syncthreads();
+            const int lim = min(UP_CH, j - l0);
+            for (int l = wid; l < lim; l += UP_NV * AD_W) {
+                float4 nx[UP_NV];
+                load(l0 + l + UP_NV * AD_W, nx);
 #pragma unroll
-                    for (int q = 0; q < 4; ++q) {
-                        const float2 c = csm[l + q * AD_W];
-                        fa = f2_fma(c, make_float2(v[q].x, v[q].y), fa);
-                        fb = f2_fma(c, make_float2(v[q].y, v[q].x), fb);
-                        pacc_add(a2, dsm[l + q * AD_W], v[q]);
-                        v[q] = nx[q];
-                    }
+                for (int q = 0; q < UP_NV; ++q) {
+                    pacc_add(a1, csm[l + q * AD_W], v[q]);
+                    pacc_add(a2, dsm[l + q * AD_W], v[q]);
+                    v[q] = nx[q];
                 }
             }
-            s1 = mk(df(fa.x, 0.f) - df(fa.y, 0.f), df(fb.x, 0.f) + df(fb.y, 0.f));
-        } else {
-            PAcc a1;
-            pacc_zero(a1);
-            if (in) {
-#pragma unroll 2
-                for (int l = wid; l < j; l += AD_W) {
-                    const float4 v = __ldg(V + (size_t)l * ld + e);
-                    pacc_add(a1, __ldg(cdf + l), v);
-                    pacc_add(a2, __ldg(ddf + l), v);
-                }
-            }
-            s1 = pacc_product(a1);
         }
-        red1[wid][lane] = to_f4(s1);
+        red1[wid][lane] = to_f4(pacc_product(a1));
         red2[wid][lane] = to_f4(pacc_product(a2));
         __syncthreads();
         if (wid == 0 && in) {
-            s1 = from_f4(red1[0][lane]);
+            cx<df> s1 = from_f4(red1[0][lane]);
             cx<df> s2 = from_f4(red2[0][lane]);
 #pragma unroll
             for (int q = 1; q < AD_W; ++q) {
