@@ -1,5 +1,5 @@
-// The link force of y = A x in half spinors, shared by the derivative of A (grad.cu) and of the sign
-// function (grad_krylov.cu).  With P = 1 + S gamma_nu (P^2 = 2 P, P^dag = P) and the reconstruction of P a
+// The link force of y = A x in half spinors, shared by the derivative of A (grad.cu) and the FP64 derivative of
+// the sign function (grad_krylov.cu; its mixed form has its own FP32 sum in full spinors).  With P = 1 + S gamma_nu (P^2 = 2 P, P^dag = P) and the reconstruction of P a
 // from its upper two spins h_a,
 //   sum_spins (P a)_i conj(b_j) = 1/2 sum_spins (P a)_i conj((P b)_j) = sum_{s = 0, 1} h_a,s,i conj(h_b,s,j),
 // so the colour outer product of four spins takes two, 192 FP64 operations per link (48 projection sums, 144

@@ -311,44 +311,8 @@ __global__ void k_gq_finish(double2* M, double2* sd, int n, const KState* ks, co
 // Z_q = sum_p conj(M~_pq) w~_p for q < k (vectors of n complex, ld n): tiles of 64 elements x 16
 // columns, the p sum in chunks of 16 through shared memory
 constexpr int ZT_E = 64, ZT_Q = 16, ZT_P = 16;
-__global__ void __launch_bounds__(256) k_gq_combine(const double2* __restrict__ W, const double2* __restrict__ M,
-                                                    double2* __restrict__ Z, int k, size_t n) {
-    __shared__ double2 ws[ZT_P][ZT_E];
-    __shared__ double2 ms[ZT_P][ZT_Q];
-    const size_t e0 = (size_t)blockIdx.x * ZT_E;
-    const int q0 = blockIdx.y * ZT_Q;
-    const int te = threadIdx.x & 63, tq = threadIdx.x >> 6;  // 4 groups of 4 columns
-    cx<double> acc[4] = {mk(0.0, 0.0), mk(0.0, 0.0), mk(0.0, 0.0), mk(0.0, 0.0)};
-    for (int p0 = 0; p0 < k; p0 += ZT_P) {
-        for (int x = threadIdx.x; x < ZT_P * ZT_E; x += blockDim.x) {
-            const int pp = x / ZT_E, ee = x % ZT_E;
-            const size_t e = e0 + ee;
-            ws[pp][ee] = (p0 + pp < k && e < n) ? W[(size_t)(p0 + pp) * n + e] : make_double2(0.0, 0.0);
-        }
-        for (int x = threadIdx.x; x < ZT_P * ZT_Q; x += blockDim.x) {
-            const int pp = x / ZT_Q, qq = x % ZT_Q;
-            const double2 m = (p0 + pp < k && q0 + qq < k) ? M[(size_t)(p0 + pp) * k + q0 + qq] : make_double2(0.0, 0.0);
-            ms[pp][qq] = make_double2(m.x, -m.y);
-        }
-        __syncthreads();
-#pragma unroll 4
-        for (int pp = 0; pp < ZT_P; ++pp) {
-            const cx<double> w = d2c(ws[pp][te]);
-#pragma unroll
-            for (int j = 0; j < 4; ++j) cfma(acc[j], d2c(ms[pp][tq * 4 + j]), w);
-        }
-        __syncthreads();
-    }
-    const size_t e = e0 + te;
-    if (e < n)
-#pragma unroll
-        for (int j = 0; j < 4; ++j) {
-            const int q = q0 + tq * 4 + j;
-            if (q < k) Z[(size_t)q * n + e] = c2d(acc[j]);
-        }
-}
 
-// (1 + S gamma_nu) gamma5 x as a full spinor
+// (1 + S gamma_nu) gamma5 x as a full spinor (mixed gradient, with its mu derivative below)
 template <int NU, int S, class R>
 __device__ __forceinline__ void proj_g5_full_r(const Spinor<R>& x, Spinor<R>& o) {
     Spinor<R> g5 = x;
@@ -401,9 +365,7 @@ __device__ __forceinline__ double dmu_site(const Geom& g, const Coord& c, int s,
     return r;
 }
 
-// gU = sum_q force(v~_q, Z_q) (the link adjoint of Re <Z_q, A v~_q>), gmu = sum_q Re <Z_q, dA/dmu v~_q>;
-// one thread per site and direction block, the q sum inside (fixed order)
-// The same product in double-float arithmetic (products exact through the FMA split, sums
+// Z in double-float arithmetic (products exact through the FMA split, sums
 // compensated; about 48 significant bits, on the FP32 pipe), FP64 in and out.
 __global__ void __launch_bounds__(256) k_gq_combine_df(const double2* __restrict__ W, const double2* __restrict__ M,
                                                        double2* __restrict__ Z, int k, size_t n) {

@@ -14,8 +14,8 @@
 // the per-block partial sums of alpha = w^dag t and |t|^2 (and of the
 // re-projection coefficients L^dag t, R^dag s), and after those of
 // w^^dag v^, |v^|^2, |w^|^2.  In-block sums use exact FP32 products with
-// compensated (pair) accumulation; the cross-block sums and all recurrence
-// scalars are FP64 and formed by a single warp -- GB300's FP64 pipe is narrow,
+// compensated (pair) accumulation, and so do the cross-block sums; the recurrence
+// scalars are FP64 and formed by the lanes of two warps -- GB300's FP64 pipe is narrow,
 // so scalar algebra repeated by every warp would cost more than the stencil.  Every block adds the per-block partials
 // in the same fixed order, so all blocks hold bit-identical coefficients.
 // Pass 2 regenerates the basis with one barrier per step: in double-float here, in FP64 (the default) in
@@ -533,12 +533,6 @@ template <class R> struct P2Args {
 // slot 2 accumulates y
 __device__ __forceinline__ int st2_idx(int jt, int slot, int site, int q) { return ((jt * 3 + slot) * PT + site) * 12 + q; }
 
-template <class R> __device__ __forceinline__ cx<R> from_f64(double2 v);
-template <> __device__ __forceinline__ cx<double> from_f64<double>(double2 v) { return d2c(v); }
-template <> __device__ __forceinline__ cx<df> from_f64<df>(double2 v) { return d2df(v); }
-__device__ __forceinline__ double2 to_f64(cx<double> z) { return c2d(z); }
-__device__ __forceinline__ double2 to_f64(cx<df> z) { return df2d(z); }
-
 // regeneration v_{i+1} = ((A - alpha_i) v_i - gamma_{i-1} v_{i-1}) / beta_i, y += c_{i+1} v_{i+1} (Sec. 5)
 template <class R, int LF>
 __global__ void __launch_bounds__(32 * PW2) k_pass2_persistent(P2Args<R> a) {
@@ -563,7 +557,7 @@ __global__ void __launch_bounds__(32 * PW2) k_pass2_persistent(P2Args<R> a) {
                 const int q = 3 * sp + c3;
                 st[st2_idx(jt, 0, site, q)] = ok ? ld_comp_cg<R>((const VT*)a.v[0], g.V, ii, q) : mk(R(0), R(0));
                 st[st2_idx(jt, 1, site, q)] = mk(R(0), R(0));
-                st[st2_idx(jt, 2, site, q)] = ok ? from_f64<R>(__ldcg(a.y + (size_t)q * g.V + ii)) : mk(R(0), R(0));
+                st[st2_idx(jt, 2, site, q)] = ok ? d2df(__ldcg(a.y + (size_t)q * g.V + ii)) : mk(R(0), R(0));
             }
         }
     }
@@ -631,7 +625,7 @@ __global__ void __launch_bounds__(32 * PW2) k_pass2_persistent(P2Args<R> a) {
 #pragma unroll
         for (int c3 = 0; c3 < 3; ++c3) {
             const int q = 3 * sp + c3;
-            a.y[(size_t)q * g.V + ii] = to_f64(st[st2_idx(jt, 2, site, q)]);
+            a.y[(size_t)q * g.V + ii] = df2d(st[st2_idx(jt, 2, site, q)]);
         }
     }
 }
