@@ -23,8 +23,8 @@
 // imaginary parts, both reciprocal square roots in one instruction stream), the breakdown checks by
 // another warp.
 //
-// Measured (GB300): FP64 solve on 6^4, k = 480, 23.0 -> 8.4 ms (48 -> 16 us per step, of which the FP64 pipe
-// of the busiest SM quarter is busy 11); regeneration on 8^4 15.5 -> 12.0 us per step (FP64 pipe 8.5).
+// Measured (GB300): FP64 solve on 6^4, k = 480, 23.0 -> 7.7 ms (48 -> 14.4 us per step, of which the FP64 pipe
+// of the busiest SM quarter is busy 11); regeneration on 8^4 15.5 -> 10.5 us per step (FP64 pipe 8.5).
 #include <algorithm>
 
 #include "hop64.cuh"
@@ -163,7 +163,7 @@ __global__ void __launch_bounds__(LT) k_l2_f64(L2Args a) {
     double svr = ks->sv.x, svpr = ks->svp.x, swr = ks->sw.x, swi = ks->sw.y, swpr = ks->swp.x, swpi = ks->swp.y;
     double anorm2 = ks->anorm * ks->anorm;
     int kused = 0, bd = -1;
-    unsigned int nbar = 0;
+    unsigned int target = a.unreach;  // arrivals of the last barrier
     if (tid == 0) {
         cs[0] = make_double2(svr, 0.0);
         cs[1] = make_double2(swr, swi);
@@ -219,7 +219,7 @@ __global__ void __launch_bounds__(LT) k_l2_f64(L2Args a) {
         }
         __syncthreads();
         if (wid == 0) block_partials(red, nw, a.partA);
-        grid_barrier_mono(a.bar, (unsigned)G * (++nbar) + a.unreach, err, 1, a.spin);
+        grid_barrier_mono(a.bar, target += G, err, 1, a.spin);
         if (*(volatile int*)err) return;
         if (wid < 4) grid_partials(a.partA, G, wid, gs);
         __syncthreads();
@@ -278,7 +278,7 @@ __global__ void __launch_bounds__(LT) k_l2_f64(L2Args a) {
         }
         __syncthreads();
         if (wid == 0) block_partials(red, nw, a.partC);
-        grid_barrier_mono(a.bar, (unsigned)G * (++nbar) + a.unreach, err, 1, a.spin);
+        grid_barrier_mono(a.bar, target += G, err, 1, a.spin);
         if (*(volatile int*)err) return;
         if (wid < 4) grid_partials(a.partC, G, wid, gs);
         __syncthreads();
@@ -399,7 +399,7 @@ __global__ void __launch_bounds__(LT) k_regen_f64(R64Args a) {
         }
     }
     __syncwarp();
-    unsigned int nbar = 0;
+    unsigned int target = a.unreach;  // arrivals of the last barrier
     for (int i = 0; i + 1 < kused; ++i) {
         const int cur = i & 1, prv = cur ^ 1;
         const double2* x = a.v[i % 3];
@@ -443,7 +443,7 @@ __global__ void __launch_bounds__(LT) k_regen_f64(R64Args a) {
             __syncwarp();
         }
         if (i + 2 < kused) {
-            grid_barrier_mono(a.bar, (unsigned)G * (++nbar) + a.unreach, a.err, 1, a.spin);
+            grid_barrier_mono(a.bar, target += G, a.err, 1, a.spin);
             if (*(volatile int*)a.err) return;
         }
     }
