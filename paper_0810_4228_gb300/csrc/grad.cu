@@ -43,10 +43,11 @@ __global__ void __launch_bounds__(128, 4) k_dw_grad(const double2* __restrict__ 
                                                  double kappa, double emu, double emum, Geom g, double* partials,
                                                  unsigned int* counter, double* gmu) {
     __shared__ double red[32];
-    const int nu = ((threadIdx.x >> 5) + blockIdx.x) & 3;
-    const int s = blockIdx.x * 32 + (threadIdx.x & 31);
+    // (without the links' gradient: the temporal link of 128 sites per block)
+    const int nu = gU ? ((threadIdx.x >> 5) + blockIdx.x) & 3 : 3;
+    const int s = gU ? blockIdx.x * 32 + (threadIdx.x & 31) : blockIdx.x * 128 + threadIdx.x;
     double part[1] = {0.0};
-    if (s < g.V && (gU || nu == 3)) {
+    if (s < g.V) {
         int c[4], r = s;
         c[3] = r % g.L[3];
         r /= g.L[3];
@@ -102,7 +103,7 @@ extern "C" int ovl_dw_grad(ovl_ctx* c, double mu, double kappa, const void* x, c
     int r = ensure_solve(c, std::max(c->kcap, 1));
     if (r) return r;
     double* gmu = reinterpret_cast<double*>(c->h2);
-    const int T = 128, B = (c->g.V + 31) / 32;
+    const int T = 128, per = grad_U ? 32 : T, B = (c->g.V + per - 1) / per;  // sites per block (k_dw_grad)
     if (flags & OVL_F32)
         ovl::k_dw_grad<float><<<B, T, 0, c->st>>>(c->U64, (const double2*)x, (const double2*)g, (double2*)grad_U,
                                                   kappa, exp(mu), exp(-mu), c->g, c->partials, c->counter, gmu);
