@@ -76,7 +76,16 @@ typedef struct ovl_ctx ovl_ctx;
                                     significant bits, 16 bytes per complex element as in FP64) and
                                     both Gram-Schmidt sweeps in double-float arithmetic on the FP32
                                     pipe; FP64 stencil, H and inner sign.  Results agree with the
-                                    FP64 Arnoldi run to about 1e-12                          */
+                                    FP64 Arnoldi run to about 1e-12.
+                                    LANCZOS2 near a breakdown: where |w^^dag v^| gets small against
+                                    |v^||w^| the recurrence amplifies pass 1's FP32 roundings, and the
+                                    result at a given k then hangs on the order of its operations:
+                                    against FP64, and between two forms of the solve (single or batch, persistent
+                                    or stepwise, another release) most sources agree to 1e-13, about
+                                    one in a hundred only to 1e-9 ... 1e-4 (8^4, mu = 0.3, k = 480), and
+                                    at mu = 0.5 with 20 deflated pairs every second one only to 1e-8,
+                                    one in eight to 1e-4, for the better as often as for the worse.
+                                    FP64 solves and Arnoldi do not show this at these k            */
 #define OVL_TWO_PASS     0x0400  /* sign_krylov LANCZOS2: do not store the basis, regenerate it
                                     from alpha, beta, gamma in a second pass (Sec. 5)       */
 #define OVL_INNER_NEWTON 0x1000  /* inner sgn(G_k) / sgn(H_k): Roberts/Newton (Sec. 2) instead of
