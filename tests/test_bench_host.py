@@ -81,3 +81,13 @@ def test_measured_peaks_lookup(tmp_path, monkeypatch):
         assert bench.peaks() == (want, "measured")
     monkeypatch.setattr(bench, "ROOT", str(tmp_path))
     assert bench.peaks() == (6800.0, "fallback")
+
+
+def test_counts_of_the_present_kernels():
+    """k_b_regen_df's FP32 operations per site and step (8 hops of 12 sums of 8, 12 sums of 6 products at 64 and 24 spin
+    sums of 8; 168; 24 parts of 52 + 30 + 9), and the launches of a mixed batch of 12 sources with m = 20, k = 550: 12 per
+    sequence (pack, init, four projections, split, two conversions, Newton's two, unpack), pass 1, the inner sign's 12
+    without Newton, three around the regeneration and its 549 steps."""
+    import bench
+    assert bench.REGEN_DFX_OPS_SITE == 8 * (96 + 768 + 192) + 168 + 24 * 91 == 10800
+    assert bench.batch_launches(12, 550, 20, fused_start=True) == 12 * 12 + 1 + 12 + 3 + 549
