@@ -386,12 +386,12 @@ int ovl_sign_arnoldi_restarted(ovl_ctx* ctx, int m, int cycles, double mu, doubl
                                const void* b, void* out, int flags, ovl_info* info);
 
 /* Limits of the bounded device waits of the context's persistent kernels (the grid barriers of
- * two-sided Lanczos on lattices that fit the GPU: both passes of OVL_MIXED solves, the FP64 process of
- * ovl_sign_krylov and of ovl_sign_grad): a wait gives up after
- * `polls` polls (0 restores the default, 2e7), sets the solve's timeout flag and every block
- * leaves, so the call returns OVL_ETIMEOUT and the context stays usable.  unreachable != 0 adds
- * one arrival to every barrier's target, so every wait runs out: a test of the timeout path
- * without a fault (use a small `polls`).  Drops the captured solve graph.  The paper has no
+ * two-sided Lanczos on lattices that fit the GPU: the FP32 pass 1 and the FP64 pass 2 of OVL_MIXED solves,
+ * the FP64 process of ovl_sign_krylov and of ovl_sign_grad): a wait gives up after `polls` polls (0
+ * restores the default, 2e7), sets the solve's timeout flag and every block leaves, so the call returns
+ * OVL_ETIMEOUT and the context stays usable.  unreachable != 0 puts the targets of the barriers of pass 1
+ * and of the FP64 process one arrival out of reach, so every such wait runs out: a test of the timeout
+ * path without a fault (use a small `polls`).  Drops the captured solve graph.  The paper has no
  * counterpart. */
 int ovl_set_wait_limit(ovl_ctx* ctx, long long polls, int unreachable);
 

@@ -360,13 +360,13 @@ int enqueue_solve(ovl_ctx* c, int method, int k, double mu, double kappa, int fl
         // kernels where the device does not take the launch
         bool persist64 = !mixed && !(flags & OVL_STEPWISE) && ovl::l2_f64_ok(g, c->num_sms);
         if (persist64) {
-            cudaMemsetAsync(c->bar, 0, 64, st);
+            cudaMemsetAsync(c->bar, c->wait_unreachable ? 0xff : 0, 64, st);  // (one arrival short: out of reach)
             int lr = 0;
             prof(c, KC_PASS1, [&] {
                 double2* vv[3] = {twopass ? c->R64[0] : c->V64, c->R64[1], c->R64[2]};
                 lr = ovl::launch_l2_f64(c->U64, c->nbr, vv, twopass ? 0 : n, c->W64, 0, ks, c->alpha, c->beta,
                                         c->gamma, c->vscale, mu, kappa, k, part, c->bar, g, c->num_sms, st,
-                                        c->wait_polls, c->wait_unreachable);
+                                        c->wait_polls);
             });
             if (lr == (int)cudaErrorCooperativeLaunchTooLarge) {
                 cudaGetLastError();
@@ -440,7 +440,7 @@ int enqueue_solve(ovl_ctx* c, int method, int k, double mu, double kappa, int fl
                 const float4* udf = (mixed && (flags & OVL_PASS2_DF)) ? c->Udf : nullptr;
                 lr = ovl::launch_pass2_persistent(c->U64, c->nbr, udf, rr, c->y64, ks, c->alpha, c->beta, c->gamma, c->cvec,
                                                   c->H, c->kcap, mu, kappa, c->bar, &ks->timeout, g, c->num_sms,
-                                                  st, c->wait_polls, c->wait_unreachable);
+                                                  st, c->wait_polls);
             });
             if (lr) return fail(c, OVL_ECUDA, std::string("persistent pass 2 launch: ") +
                                                    cudaGetErrorString((cudaError_t)lr));

@@ -587,9 +587,9 @@ __global__ void __launch_bounds__(DC_T) k_adf_dot2_reduce(const double2* __restr
 // of H, a warp per row: H[i, j] = d_i / nu - g_i (i < j), r - c_{j-1} (i = j), g_i = sum_{l >= i-1} H[i, l] c_l / nu (upper
 // Hessenberg rows of the final columns).
 // Bound by the FP32 pipe (48 packed operations per term, both sums double-float) beside 16 bytes of basis per term.
-// Solve of k = 450 on 8^4: 56.5 ms (71.2 with scalar sums); two vectors per round at 32 warps per SM, against 56.6 with
-// four at 24 warps, 57.5 with two at 24, 58.7 and 59.2 with four and eight at 16.  (The c sum in FP32 from the
-// leading parts, where |c| is small, takes 51.8: not kept, it is less than the basis's precision.)
+// The 450 updates of k = 450 on 8^4: 30.1 ms with scalar sums, 24.0 ms so.  The solve takes 56.5 ms with two vectors per
+// round at 32 warps per SM, 56.6 with four at 24 warps, 57.5 with two at 24, 58.7 and 59.2 with four and eight at 16.  (The
+// c sum in FP32 from the leading parts, where |c| is small, takes 51.8: less than the basis's precision, not kept.)
 static constexpr int UP_CH = 512;  // coefficients staged in shared memory at a time (a multiple of UP_NV x AD_W)
 static constexpr int UP_NV = 2;   // vectors per warp and round
 __global__ void __launch_bounds__(AD_T, 4) k_adf_update2(const float4* __restrict__ V, size_t ld, int j, int cold, int hb,

@@ -721,11 +721,10 @@ extern "C" int ovl_sign_grad(ovl_ctx* c, int k, double mu, double kappa, const v
     } else {
         bool persist = ovl::l2_f64_ok(g, c->num_sms);
         if (persist) {
-            OVL_CUDA_TRY(c, cudaMemsetAsync(c->bar, 0, 64, st));
+            OVL_CUDA_TRY(c, cudaMemsetAsync(c->bar, c->wait_unreachable ? 0xff : 0, 64, st));
             double2 *vv[3] = {V, nullptr, nullptr}, *ww[3] = {W, nullptr, nullptr};
             const int lr = ovl::launch_l2_f64(c->U64, c->nbr, vv, n, ww, n, ks, c->alpha, c->beta, c->gamma, c->vscale,
-                                              mu, kappa, k, part, c->bar, g, c->num_sms, st, c->wait_polls,
-                                              c->wait_unreachable);
+                                              mu, kappa, k, part, c->bar, g, c->num_sms, st, c->wait_polls);
             if (lr == (int)cudaErrorCooperativeLaunchTooLarge) {  // per-step kernels, as in the solve
                 cudaGetLastError();
                 persist = false;

@@ -455,17 +455,12 @@ __device__ __forceinline__ void grid_barrier_mono(unsigned int* ctr, unsigned in
     __syncthreads();
     if (threadIdx.x == 0) {
         asm volatile("red.release.gpu.global.add.u32 [%0], %1;" ::"l"(ctr), "r"(1u) : "memory");
-        // (polls in runs of 64, the limit looked at between them: a 64-bit count in the loop itself cost the FP64
-        // process 0.5 % of a solve's time)
-        bool in = false;
-        for (long long left = max_spins; !in; left -= 64) {
-#pragma unroll 1
-            for (int u = 0; u < 64 && !in; ++u) {
-                unsigned int v;
-                asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(ctr) : "memory");
-                in = (int)(v - target) >= 0;
-            }
-            if (!in && left < 64) {
+        long long spins = 0;
+        while (true) {
+            unsigned int v;
+            asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(ctr) : "memory");
+            if ((int)(v - target) >= 0) break;
+            if (++spins > max_spins) {
                 atomicExch(err, code);
                 break;
             }

@@ -168,23 +168,23 @@ int launch_pass2_persistent(const double2* U64, const int* nbr, const float4* Ud
                             const KState* ks,
                             const double2* alpha, const double2* beta, const double2* gamma, const double2* c,
                             double2* coef_work, int kmax, double mu, double kappa, unsigned int* bar, int* err,
-                            const Geom& g, int num_sms, cudaStream_t st, long long spin = 0, int unreachable = 0);
+                            const Geom& g, int num_sms, cudaStream_t st, long long spin = 0);
 
 // ---- persistent64.cu
 // The FP64 two-sided Lanczos process in one cooperative launch, on lattices whose own-site state fits the
 // SMs' shared memory (l2_f64_ok).  v, w: rings of three vectors, or the first vector of a stored basis
 // (v[0], w[0]) with vstep, wstep complex elements between vectors.  partials: 8 x num_sms doubles; bar:
-// arrival counter, zero at launch.  Scales of the stored vectors to vscale (may be null).
+// arrival counter, zero at launch; spin: limit of a barrier wait's polls (0: the default).  Scales of the stored vectors to vscale (may be null).
 bool l2_f64_ok(const Geom& g, int num_sms);
 int launch_l2_f64(const double2* U64, const int* nbr, double2* const v[3], size_t vstep, double2* const w[3],
                   size_t wstep, KState* ks, double2* alpha, double2* beta, double2* gamma, double2* vscale, double mu,
                   double kappa, int k, double* partials, unsigned int* bar, const Geom& g, int num_sms,
-                  cudaStream_t st, long long spin = 0, int unreachable = 0);
+                  cudaStream_t st, long long spin = 0);
 // The FP64 regeneration pass in one cooperative launch (lattices of persistent_ok); coef: per step
 // 1 / beta_i, alpha_i / beta_i, gamma_{i-1} / beta_i, c_{i+1}
 int launch_regen_f64(const double2* U64, const int* nbr, double2* const v[3], double2* y, const KState* ks,
                      const double2* coef, double mu, double kappa, unsigned int* bar, int* err, const Geom& g,
-                     int num_sms, cudaStream_t st, long long spin = 0, int unreachable = 0);
+                     int num_sms, cudaStream_t st, long long spin = 0);
 
 // ---- inner_sign.cu
 // kernels one inner sign queues (the profile's counts), with the quadrature or by Newton alone

@@ -525,8 +525,6 @@ template <class R> struct P2Args {
     HopCoef<R> hc[1];
     Geom g;
     int ntiles;
-    long long spin;
-    unsigned int unreach;
 };
 
 // pass-2 state (R = df): slots 0/1 alternate as v_i and v_{i-1},
@@ -614,7 +612,7 @@ __global__ void __launch_bounds__(32 * PW2) k_pass2_persistent(P2Args<R> a) {
             __syncthreads();
         }
         if (i + 2 < kused) {
-            grid_barrier_mono(a.bar, (unsigned)G * (++nbar) + a.unreach, a.err, 1, a.spin);
+            grid_barrier_mono(a.bar, (unsigned)G * (++nbar), a.err, 1, PSPIN);
             if (*(volatile int*)a.err) return;
         }
     }
@@ -711,7 +709,7 @@ int launch_pass2_persistent(const double2* U64, const int* nbr, const float4* Ud
                             const KState* ks,
                             const double2* alpha, const double2* beta, const double2* gamma, const double2* c,
                             double2* coef_work, int kmax, double mu, double kappa, unsigned int* bar, int* err,
-                            const Geom& g, int num_sms, cudaStream_t st, long long spin, int unreachable) {
+                            const Geom& g, int num_sms, cudaStream_t st, long long spin) {
     const bool dfm = Udf != nullptr;
     const int ntiles = (g.V + PT - 1) / PT;
     const int G = persistent_grid(ntiles, num_sms);
@@ -726,8 +724,6 @@ int launch_pass2_persistent(const double2* U64, const int* nbr, const float4* Ud
         a.err = err;
         a.g = g;
         a.ntiles = ntiles;
-        a.spin = spin > 0 ? spin : PSPIN;
-        a.unreach = unreachable ? 1u : 0u;
     };
     if (tpb > PMAX_TPB) return -1;
     if (dfm) {
@@ -741,8 +737,7 @@ int launch_pass2_persistent(const double2* U64, const int* nbr, const float4* Ud
     k_pass2_coef<double2><<<(kmax + 127) / 128, 128, 0, st>>>(ks, alpha, beta, gamma, c,
                                                                reinterpret_cast<RegenCoef<double2>*>(coef_work), kmax,
                                                                bar);
-    return launch_regen_f64(U64, nbr, v, y, ks, coef_work, mu, kappa, bar, err, g, num_sms, st, spin,
-                            unreachable);
+    return launch_regen_f64(U64, nbr, v, y, ks, coef_work, mu, kappa, bar, err, g, num_sms, st, spin);
 }
 
 }  // namespace ovl

@@ -34,7 +34,7 @@ namespace ovl {
 namespace {
 
 constexpr int LT = 32 * LW;
-constexpr long long LSPIN = 20000000;  // default limit of a barrier wait's polls (a wait that gives up sets ks->timeout)
+constexpr long long LSPIN = 20000000;  // polls before a barrier wait gives up (sets ks->timeout)
 
 // Sums over the lanes of one input (lane bit NB = 8 RS): v0 and v1 each, valid in the lane of that input
 // whose lower bits are 0 (v0) or 4 (v1).  First step: the lane bit above or below NB.
@@ -107,8 +107,7 @@ struct L2Args {
     unsigned int* bar;
     double kappa, emu, emum;
     int V, k, npass;
-    long long spin;       // polls before a barrier wait gives up (ovl_set_wait_limit)
-    unsigned int unreach; // added to every barrier's target
+    long long spin;       // limit of a barrier wait's polls (LIM)
 };
 
 // shared memory: half spinors of a warp's units, then own-site state [pass][cur, prev, t][value][thread]
@@ -119,7 +118,9 @@ size_t l2_smem(int rs, int npass) {
     return (size_t)LW * L2_HP * sizeof(double2) + (size_t)npass * 3 * (rs == 1 ? 3 : 2) * LT * sizeof(double);
 }
 
-template <int RS>
+// LIM: the limit of ovl_set_wait_limit in place of LSPIN.  A form of its own: with the limit an argument of the one
+// form its polls, or what else the compiler then arranges otherwise, cost 0.3 to 1.6 % of a solve.
+template <int RS, bool LIM>
 __global__ void __launch_bounds__(LT) k_l2_f64(L2Args a) {
     extern __shared__ __align__(16) unsigned char smraw[];
     KState* ks = a.ks;
@@ -163,7 +164,7 @@ __global__ void __launch_bounds__(LT) k_l2_f64(L2Args a) {
     double svr = ks->sv.x, svpr = ks->svp.x, swr = ks->sw.x, swi = ks->sw.y, swpr = ks->swp.x, swpi = ks->swp.y;
     double anorm2 = ks->anorm * ks->anorm;
     int kused = 0, bd = -1;
-    unsigned int target = a.unreach;  // arrivals of the last barrier
+    unsigned int nbar = 0;
     if (tid == 0) {
         cs[0] = make_double2(svr, 0.0);
         cs[1] = make_double2(swr, swi);
@@ -219,7 +220,7 @@ __global__ void __launch_bounds__(LT) k_l2_f64(L2Args a) {
         }
         __syncthreads();
         if (wid == 0) block_partials(red, nw, a.partA);
-        grid_barrier_mono(a.bar, target += G, err, 1, a.spin);
+        grid_barrier_mono(a.bar, (unsigned)G * (++nbar), err, 1, LIM ? a.spin : LSPIN);
         if (*(volatile int*)err) return;
         if (wid < 4) grid_partials(a.partA, G, wid, gs);
         __syncthreads();
@@ -278,7 +279,7 @@ __global__ void __launch_bounds__(LT) k_l2_f64(L2Args a) {
         }
         __syncthreads();
         if (wid == 0) block_partials(red, nw, a.partC);
-        grid_barrier_mono(a.bar, target += G, err, 1, a.spin);
+        grid_barrier_mono(a.bar, (unsigned)G * (++nbar), err, 1, LIM ? a.spin : LSPIN);
         if (*(volatile int*)err) return;
         if (wid < 4) grid_partials(a.partC, G, wid, gs);
         __syncthreads();
@@ -361,11 +362,10 @@ struct R64Args {
     int* err;
     double kappa, emu, emum;
     int V, npass;
-    long long spin;
-    unsigned int unreach;
+    long long spin;       // (LIM)
 };
 
-template <int RS>
+template <int RS, bool LIM>
 __global__ void __launch_bounds__(LT) k_regen_f64(R64Args a) {
     extern __shared__ __align__(16) unsigned char smraw[];
     if (a.ks->status || a.ks->timeout) return;  // (pass 1 gave up: the same decision in every block)
@@ -399,7 +399,7 @@ __global__ void __launch_bounds__(LT) k_regen_f64(R64Args a) {
         }
     }
     __syncwarp();
-    unsigned int target = a.unreach;  // arrivals of the last barrier
+    unsigned int nbar = 0;
     for (int i = 0; i + 1 < kused; ++i) {
         const int cur = i & 1, prv = cur ^ 1;
         const double2* x = a.v[i % 3];
@@ -443,7 +443,7 @@ __global__ void __launch_bounds__(LT) k_regen_f64(R64Args a) {
             __syncwarp();
         }
         if (i + 2 < kused) {
-            grid_barrier_mono(a.bar, target += G, a.err, 1, a.spin);
+            grid_barrier_mono(a.bar, (unsigned)G * (++nbar), a.err, 1, LIM ? a.spin : LSPIN);
             if (*(volatile int*)a.err) return;
         }
     }
@@ -466,7 +466,7 @@ void allow_smem(CoopKernel<A> kern, int rs, unsigned long long& attr_dev) {
     if (first_use_on_device(attr_dev))
         cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)l2_smem(rs, L_MAXPASS));
 }
-unsigned long long l2_dev[2], regen_dev[2];  // k_l2_f64, k_regen_f64: RS = 1, 2
+unsigned long long l2_dev[2][2], regen_dev[2][2];  // k_l2_f64, k_regen_f64: RS = 1, 2; LIM
 
 template <class A>
 int launch_coop(CoopKernel<A> kern, A args, const Split& sp, unsigned long long& attr_dev, cudaStream_t st) {
@@ -489,8 +489,8 @@ int launch_coop(CoopKernel<A> kern, A args, const Split& sp, unsigned long long&
 bool l2_f64_ok(const Geom& g, int num_sms) {
     const Split sp = split_units(g.V, 2, num_sms);
     if (sp.npass > L_MAXPASS) return false;
-    const CoopKernel<L2Args> kern = sp.rs == 1 ? k_l2_f64<1> : k_l2_f64<2>;
-    allow_smem(kern, sp.rs, l2_dev[sp.rs - 1]);
+    const CoopKernel<L2Args> kern = sp.rs == 1 ? k_l2_f64<1, false> : k_l2_f64<2, false>;
+    allow_smem(kern, sp.rs, l2_dev[sp.rs - 1][0]);
     int dev = 0, coop = 0, per_sm = 0;
     if (cudaGetDevice(&dev) != cudaSuccess ||
         cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev) != cudaSuccess ||
@@ -504,7 +504,7 @@ bool l2_f64_ok(const Geom& g, int num_sms) {
 int launch_l2_f64(const double2* U64, const int* nbr, double2* const v[3], size_t vstep, double2* const w[3],
                   size_t wstep, KState* ks, double2* alpha, double2* beta, double2* gamma, double2* vscale, double mu,
                   double kappa, int k, double* partials, unsigned int* bar, const Geom& g, int num_sms,
-                  cudaStream_t st, long long spin, int unreachable) {
+                  cudaStream_t st, long long spin) {
     const Split sp = split_units(g.V, 2, num_sms);
     if (sp.npass > L_MAXPASS) return (int)cudaErrorInvalidValue;
     L2Args a;
@@ -519,13 +519,16 @@ int launch_l2_f64(const double2* U64, const int* nbr, double2* const v[3], size_
     a.bar = bar;
     a.kappa = kappa, a.emu = exp(mu), a.emum = exp(-mu);
     a.V = g.V, a.k = k, a.npass = sp.npass;
-    a.spin = spin > 0 ? spin : LSPIN, a.unreach = unreachable ? 1u : 0u;
-    return sp.rs == 1 ? launch_coop(k_l2_f64<1>, a, sp, l2_dev[0], st) : launch_coop(k_l2_f64<2>, a, sp, l2_dev[1], st);
+    a.spin = spin;
+    const bool lim = spin > 0;
+    const CoopKernel<L2Args> kern = sp.rs == 1 ? (lim ? k_l2_f64<1, true> : k_l2_f64<1, false>)
+                                               : (lim ? k_l2_f64<2, true> : k_l2_f64<2, false>);
+    return launch_coop(kern, a, sp, l2_dev[sp.rs - 1][lim], st);
 }
 
 int launch_regen_f64(const double2* U64, const int* nbr, double2* const v[3], double2* y, const KState* ks,
                      const double2* coef, double mu, double kappa, unsigned int* bar, int* err, const Geom& g,
-                     int num_sms, cudaStream_t st, long long spin, int unreachable) {
+                     int num_sms, cudaStream_t st, long long spin) {
     const Split sp = split_units(g.V, 4, num_sms);
     if (sp.npass > L_MAXPASS) return (int)cudaErrorInvalidValue;
     R64Args a;
@@ -539,9 +542,11 @@ int launch_regen_f64(const double2* U64, const int* nbr, double2* const v[3], do
     a.err = err;
     a.kappa = kappa, a.emu = exp(mu), a.emum = exp(-mu);
     a.V = g.V, a.npass = sp.npass;
-    a.spin = spin > 0 ? spin : LSPIN, a.unreach = unreachable ? 1u : 0u;
-    return sp.rs == 1 ? launch_coop(k_regen_f64<1>, a, sp, regen_dev[0], st)
-                      : launch_coop(k_regen_f64<2>, a, sp, regen_dev[1], st);
+    a.spin = spin;
+    const bool lim = spin > 0;
+    const CoopKernel<R64Args> kern = sp.rs == 1 ? (lim ? k_regen_f64<1, true> : k_regen_f64<1, false>)
+                                                : (lim ? k_regen_f64<2, true> : k_regen_f64<2, false>);
+    return launch_coop(kern, a, sp, regen_dev[sp.rs - 1][lim], st);
 }
 
 }  // namespace ovl
