@@ -430,8 +430,10 @@ void launch_dslash(const void* U, int prec, const void* x, void* y, double mu, d
 // t = sv * gamma5 D_w(mu) v~,  s = sw * gamma5 D_w(-mu) w~,  alpha[step] = w^dag t
 // with w = sw w~.  Skipped (uniformly) once the solve is done or failed.
 // The two stencils go to two sets of blocks (which = 0: t and the alpha partials; 1: s), so a thread
-// carries one accumulator spinor (half the registers: more warps per SM); which is the low bit of
-// blockIdx.x, so that both find the links in L2.  Only the t blocks take part in the reduction.
+// carries one accumulator spinor (half the registers: more warps per SM).  which is the low bit of
+// blockIdx.x, so that both find the links in L2, or with t_first (one-dimensional grids only) its upper half:
+// the dearer t blocks then run first and the last wave is made of s blocks (see launch_dslash_pair).  Only the t
+// blocks take part in the reduction.
 // Both kinds of block run the same copy of the stencil (34 KB of instructions): with a copy each, warps of
 // the two kinds on one SM waited for instructions a quarter of the time (32^4, FP32: 296 -> 230 us; 48^3 x 64:
 // 1843 -> 1387 us).  Bound by issue slots and load latency, at 2.8 TB/s of its own operands.
@@ -445,13 +447,16 @@ __global__ void __launch_bounds__(128, LF == LINK_F64 ? 2 : OVL_DSLASH_F32_MINB)
                                                      HopCoef<typename LinkReal<LF>::R> hv,
                                                      HopCoef<typename LinkReal<LF>::R> hw, KState* ks,
                                                      double2* alpha, int step, int klast, double* partials,
-                                                     unsigned int* counter, Geom g) {
+                                                     unsigned int* counter, Geom g, bool t_first) {
     using R = typename LinkReal<LF>::R;
     __shared__ double red[3 * 32];  // grid_sum_last<3>: 32 doubles per value
     if (ks->done || ks->status) return;
     const double2 sv = ks->sv, sw = ks->sw;
-    const int which = (int)(blockIdx.x & 1u);
-    const int i = ROWS ? site_of_rows(g, blockIdx.x >> 1, gridDim.x >> 1) : site_of_block(g, blockIdx.x >> 1);
+    const unsigned nx = gridDim.x >> 1;  // blocks of each kind
+    const bool halves = !ROWS && t_first;
+    const int which = halves ? (int)(blockIdx.x >= nx) : (int)(blockIdx.x & 1u);
+    const unsigned bx = halves ? blockIdx.x - (which ? nx : 0u) : blockIdx.x >> 1;
+    const int i = ROWS ? site_of_rows(g, bx, nx) : site_of_block(g, bx);
     // per-thread sums: FP64 for FP64 data and with WIDE; otherwise exact FP32 products summed as compensated
     // FP32 pairs (TwoSum) on the FP32 pipe, widened to FP64 for the block and grid sums
     using A = typename std::conditional<sizeof(R) == 4 && !WIDE, AccF, AccD>::type;
@@ -495,7 +500,6 @@ __global__ void __launch_bounds__(128, LF == LINK_F64 ? 2 : OVL_DSLASH_F32_MINB)
         else part[j] = pa[j].v;
     }
     double out[3];
-    const unsigned nx = gridDim.x >> 1, bx = blockIdx.x >> 1;
     const unsigned blk = ROWS ? bx + nx * (blockIdx.y + gridDim.y * blockIdx.z) : bx;
     const unsigned nblk = ROWS ? nx * gridDim.y * gridDim.z : nx;
     if (grid_sum_last<3>(part, partials, counter, out, red, blk, nblk)) {
@@ -513,8 +517,8 @@ __global__ void __launch_bounds__(128, LF == LINK_F64 ? 2 : OVL_DSLASH_F32_MINB)
 
 // The pair's two stencils run in one launch, so one thread per site and stencil is the faster form from few
 // sites on (us of the call, FP32 / FP64, against the direction split: 4096 sites 30.6 / 66.7 against 31.0 / 48.2,
-// 8748 40.3 / 67.7 against 42.2 / 67.7, 20736 50.2 / 130 against 57.6 / 131, 65536 68.2 / 270 against 88.7 / 308, 118800 82.7
-// against 129.5 in FP32).  Both forms sum alpha and |t|^2 in FP64 there (WIDE): in compensated FP32 pairs the call took
+// 8748 40.3 / 67.7 against 42.2 / 67.7, 20736 50.2 / 130 against 57.6 / 131, 65536 68.2 / 270 against 88.7 / 308, 116280 76.4
+// against 125.0 in FP32).  Both forms sum alpha and |t|^2 in FP64 there (WIDE): in compensated FP32 pairs the call took
 // 38.1, 38.8, 49.4 and 63.0 us, but alpha's error rose from 1e-18 to 1e-17 of the terms' magnitudes, and products of
 // small or large vectors left the FP32 range.
 static bool pair_ds(const Geom& g) { return g_ds_mode < 0 ? g.V < (1 << 13) : g_ds_mode == 1; }
@@ -547,21 +551,27 @@ void launch_dslash_pair(const void* U, int prec, const void* v, const void* w, v
     RowGrid rg = row_grid(g, T);
     rg.grid.x *= 2;  // the two stencils
     const dim3 g1(2 * B);
+    // t blocks first while the links stay in L2 (129 MB) until the s blocks come, and in FP64, which waits for its pipe
+    // instead (us, interleaved / t first: FP32 20736 sites 52.3 / 52.1, 43680 64.8 / 54.1, 116280 89.0 / 76.4, 166320 78.2 / 66.0,
+    // 317952 104.4 / 102.2, 706440 178.4 / 176.9, 1079296 243.8 / 250.6; FP64 43680 207 / 199, 1079296 3720 / 3700)
+    const bool t_first = prec == 0 || (size_t)g.V * 192 <= (size_t)129 << 20;
     if (prec == 0) {
         if (rg.ok)
             k_dslash_pair<LINK_F64, true><<<rg.grid, T, 0, st>>>(
                 U, (const double2*)v, (const double2*)w, (double2*)t, (double2*)s, make_coef<double>(mu, kappa),
-                make_coef<double>(-mu, kappa), ks, alpha, step, klast, partials, counter, g);
+                make_coef<double>(-mu, kappa), ks, alpha, step, klast, partials, counter, g,
+                t_first);
         else
             k_dslash_pair<LINK_F64, false><<<g1, T, 0, st>>>(
                 U, (const double2*)v, (const double2*)w, (double2*)t, (double2*)s, make_coef<double>(mu, kappa),
-                make_coef<double>(-mu, kappa), ks, alpha, step, klast, partials, counter, g);
+                make_coef<double>(-mu, kappa), ks, alpha, step, klast, partials, counter, g,
+                t_first);
     } else {
         const bool wide = use_ds(g);  // up to the volume where the other forms of the call sum in FP64 (pair_ds)
         auto go = [&](auto kern, dim3 grid) {
             kern<<<grid, T, 0, st>>>(U, (const float4*)v, (const float4*)w, (float4*)t, (float4*)s,
                                      make_coef<float>(mu, kappa), make_coef<float>(-mu, kappa), ks, alpha, step, klast,
-                                     partials, counter, g);
+                                     partials, counter, g, t_first);
         };
         if (rg.ok)
             go(wide ? k_dslash_pair<LINK_F32_12, true, true> : k_dslash_pair<LINK_F32_12, true>, rg.grid);

@@ -57,3 +57,29 @@ def test_fp32_pair_sums_alpha_in_fp64(dims, scale):
     ref = (a.conj() * b).sum()
     size = float(np.sqrt((np.abs(a) ** 2).sum()) * np.sqrt((np.abs(b) ** 2).sum()))
     assert abs(complex(alpha - complex(ref))) <= 100 * 2.0 ** -53 * 2 * size
+
+
+@pytest.mark.parametrize("prec", [0, 1])
+@pytest.mark.parametrize("dims", [(18, 21, 20, 22), (32, 31, 32, 34)])
+def test_pair_block_orders(dims, prec):
+    """Lattices without whole rows per block on both sides of the volume (704512 sites in FP32) where the two kinds of
+    block go from one behind the other to alternating: the bounds of the single applications above, and alpha
+    against the FP64 sum over the t that is returned."""
+    import torch
+    from paper_0810_4228_gb300 import ovl
+    V, f, eps = math.prod(dims), (0, ovl.F32)[prec], (2.0 ** -53, 2.0 ** -24)[prec]
+    ctx = ovl.Context(dims)
+    ctx.set_gauge(synth.gauge_field_torch(dims, 1.0, 95))
+    gen = torch.Generator("cuda").manual_seed(96)
+    v, w = (ctx.empty_native(prec) for _ in range(2))
+    for x in (v, w):
+        ctx.pack(torch.randn(12 * V, dtype=torch.complex128, device="cuda", generator=gen), x, prec)
+    t, s, t1, s1 = (torch.full_like(v, float("nan")) for _ in range(4))
+    alpha = ctx.apply_pair(0.25, KAPPA, v, w, t, s, prec)
+    ctx.apply_Dw(0.25, KAPPA, v, t1, flags=ovl.GAMMA5 | ovl.NATIVE | f)
+    ctx.apply_Dw(0.25, KAPPA, w, s1, flags=ovl.DAGGER | ovl.NATIVE | f)
+    for x, y in ((t, t1), (s, s1)):
+        assert float((x - y).abs().max()) <= 1000 * eps * float(y.abs().max())
+    a, b = (x.to(torch.complex128).flatten() for x in (w, t))
+    size = float(torch.linalg.vector_norm(a) * torch.linalg.vector_norm(b))
+    assert abs(alpha - complex(torch.vdot(a, b))) <= 12 * V * 2.0 ** -48 * size
